@@ -49,7 +49,7 @@ def parse_args():
     ap.add_argument("--workload", default=DEFAULT_WORKLOAD, choices=sorted(inputs.WORKLOADS) + ["batched"])
     ap.add_argument("--count", type=int, default=512, help="batched workload: number of matrices")
     ap.add_argument("--fp64-mode", type=int, default=2, choices=[0, 1, 2],
-                    help="FP64 updates: 0 DFMA pipe, 1 emulated on FP8 tensor cores (exact digit planes), "
+                    help="FP64 updates: 0 DFMA pipe, 1 emulated on the tensor cores (exact digit planes), "
                          "2 as 1 plus inverse-based TRSM in mixed precision")
     ap.add_argument("--fp32-updates", type=int, default=0, choices=[0, 1],
                     help="FP32 output tiles with emulated FP64: 0 on 10 digit planes, 1 as TF32 x 3")
@@ -208,9 +208,9 @@ def factor_probe_berr(A, L, n, b, dev, nprobe=3, seed=5):
 
 
 # Output precision -> (kernel, dtype its tensor work runs in, nominal ratio of that dtype's
-# dense peak to BF16's).  FP64 and FP32 output tiles are updated on E4M3 digit planes.
-KERNELS = {0: ("k_zgemm<14> (FP64 outputs, E4M3 digit planes)", "e4m3", 2.0),
-           1: ("k_zgemm<10> (FP32 outputs, E4M3 digit planes)", "e4m3", 2.0),
+# dense peak to BF16's).  FP64 output tiles of an all-FP64 map are updated on FP16 digit planes.
+KERNELS = {0: ("k_zgemm<7> (FP64 outputs, FP16 digit planes)", "fp16", 1.0),
+           1: ("k_zgemm<5> (FP32 outputs, FP16 digit planes)", "fp16", 1.0),
            2: ("k_qgemm<2> (FP16 outputs)", "fp16", 1.0),
            3: ("k_qgemm<3> (FP8 E4M3 outputs)", "e4m3", 2.0)}
 
@@ -245,8 +245,8 @@ def probed_peaks() -> dict:
         return {}
 
 
-MIXED_KERNELS = {0: "k_zgemm64 (FP64 outputs of a mixed map, 128 x 64 items, E4M3 digit planes)",
-                 1: "k_zgemm64 (FP32 outputs of a mixed map, 128 x 64 items, E4M3 digit planes)"}
+MIXED_KERNELS = {0: ("k_zgemm64 (FP64 outputs of a mixed map, 128 x 64 items, E4M3 digit planes)", "e4m3", 2.0),
+                 1: ("k_zgemm64 (FP32 outputs of a mixed map, 128 x 64 items, E4M3 digit planes)", "e4m3", 2.0)}
 
 
 def tensor_rooflines(st, t_step, fp32_updates, mixed=False):
@@ -263,7 +263,7 @@ def tensor_rooflines(st, t_step, fp32_updates, mixed=False):
             continue
         name, dt, ratio = KERNELS[p]
         if mixed and p in MIXED_KERNELS:
-            name = MIXED_KERNELS[p]
+            name, dt, ratio = MIXED_KERNELS[p]
         if p == 1 and fp32_updates:
             name, dt, ratio = "k_qgemm<1> (FP32 outputs, TF32 x 3)", "tf32", 0.5
         executed = st.tensor_flops[p] / (ms / 1e3) / 1e12
@@ -505,7 +505,7 @@ def run_ours(args, ws, rank, local):
             "metric": METRIC, "value": value, "unit": "TFLOP/s", "n_gpus": ws, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": t / args.steps * 1e3, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None,
-            "dtype": ("f64" if args.fp64_mode == 0 else "f64 (updates emulated on e4m3 tensor cores)")
+            "dtype": ("f64" if args.fp64_mode == 0 else "f64 (updates emulated on f16 tensor cores)")
             if not w.mixed else "f64+f32+f16+e4m3 (f64/f32 updates on e4m3 digit planes)",
             "data": "synthetic", "impl": "ours",
             "config": workload_config(w, n, b, ws),
@@ -548,7 +548,7 @@ def fp64_workload_comparisons(tc, local, stream):
         if tc.tile_chol_factor(H.h, n, b, A, None, st) == 0:
             out["fp64_path"] = {"value": n ** 3 / 3.0 / (st.t_ms / 1e3) / 1e12, "unit": "TFLOP/s",
                                 "t_factor_ms": st.t_ms,
-                                "what": "this library, fp64_mode 2 (updates and TRSM on E4M3 digit planes)"}
+                                "what": "this library, fp64_mode 2 (updates and TRSM on FP16 digit planes)"}
     torch.cuda.empty_cache()
     out.update(fp64_baselines(tc, n, b, A, local, stream))
     del A
@@ -668,18 +668,19 @@ def fp64_roofline(upd_flops, upd_ms, t):
             "update_share_of_step": (upd_ms / 1e3) / t if t > 0 else None}
 
 
-def zgemm_roofline(upd_flops, upd_ms, t):
-    """Emulated FP64 update: 105 E4M3 plane-pair products per FP64 product, so the tensor work
-    is 105 x the algorithmic flops; the roofline is the FP8 dense peak (measured BF16 x the
-    nominal FP8/BF16 ratio 2), reported both as executed and as algorithmic FP64 flops."""
+def zgemm_roofline(upd_flops, upd_ms, t, pairs=105, ratio=2.0):
+    """Emulated FP64 update: `pairs` plane-pair products per FP64 product, so the tensor work is
+    that many times the algorithmic flops; the roofline is the planes' dense peak (measured BF16 x
+    the nominal ratio: base 16 in E4M3 105 pairs at 2, base 256 in FP16 28 pairs at 1), reported
+    both as executed and as algorithmic FP64 flops."""
     pk, pk_kind = peaks()
-    fp8_peak = (pk.get("bf16_tflops_sustained") or pk["bf16_tflops"]) * 2.0
+    peak = (pk.get("bf16_tflops_sustained") or pk["bf16_tflops"]) * ratio
     alg = (upd_flops / (upd_ms / 1e3) / 1e12) if upd_ms > 0 else None
-    executed = alg * 105 if alg else None
-    return {"kernel": "k_zgemm", "bound": "tensor", "achieved": executed, "peak": fp8_peak, "unit": "TFLOP/s",
-            "frac": (executed / fp8_peak) if executed else None, "traffic": None,
-            "peak_source": f"{pk_kind} bf16 sustained x nominal fp8/bf16 ratio 2",
-            "algorithmic_fp64_tflops": alg, "pairs_per_fp64_product": 105,
+    executed = alg * pairs if alg else None
+    return {"kernel": "k_zgemm", "bound": "tensor", "achieved": executed, "peak": peak, "unit": "TFLOP/s",
+            "frac": (executed / peak) if executed else None, "traffic": None,
+            "peak_source": f"{pk_kind} bf16 sustained x nominal ratio {ratio:g}",
+            "algorithmic_fp64_tflops": alg, "pairs_per_fp64_product": pairs,
             "update_share_of_step": (upd_ms / 1e3) / t if t > 0 else None}
 
 
@@ -1026,12 +1027,13 @@ def run_ooc(args, ws, rank, local):
             "precision": (f"per-tile map, eps_high {OOC_MXP_EPS}, FP64 band {OOC_MXP_BAND}" if args.ooc_mxp
                           else "FP64")},
             ("f64+f32+f16+e4m3" if args.ooc_mxp else
-             "f64" if args.fp64_mode == 0 else "f64 (updates emulated on e4m3 tensor cores)"))
-        rf = zgemm_roofline if args.fp64_mode >= 1 else fp64_roofline
-        line["roofline"] = rf(st.update_flops[0], st.t_update_ms[0], tf)
+             "f64" if args.fp64_mode == 0 else "f64 (updates emulated on f16 tensor cores)"))
         if args.fp64_mode >= 1:
+            line["roofline"] = zgemm_roofline(st.update_flops[0], st.t_update_ms[0], tf, pairs=28, ratio=1.0)
             line["roofline"]["kernel"] = "k_zgemm (grouped out-of-core form)"
-        line["config"]["fp64_updates"] = "emulated (E4M3 digit planes)" if args.fp64_mode >= 1 else "DFMA"
+        else:
+            line["roofline"] = fp64_roofline(st.update_flops[0], st.t_update_ms[0], tf)
+        line["config"]["fp64_updates"] = "emulated (FP16 digit planes)" if args.fp64_mode >= 1 else "DFMA"
         # host-link volume of every scheduling policy at this size and cache, from the schedule
         # simulator (which the tests hold equal to the library's counters)
         emu = args.fp64_mode >= 1

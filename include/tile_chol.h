@@ -84,10 +84,11 @@ typedef struct {
     int fp64_mode;              /* how SYRK/GEMM updates of FP64 (and FP32) output tiles run:
                                    0: FP64 tiles on the FP64 pipe (DFMA), FP32 tiles as
                                       3 x TF32 tensor-core products;
-                                   1: both on the FP8 tensor cores through exact base-16
-                                      digit planes of every final tile (14 planes for FP64
-                                      outputs: normwise FP64 accuracy; 10 for FP32 outputs:
-                                      below 2^-40 of the tile scale); needs 14 b^2 extra
+                                   1: both on the tensor cores through exact digit planes
+                                      of every final tile (56 bits for FP64 outputs:
+                                      normwise FP64 accuracy; 40 for FP32 outputs: below
+                                      2^-40 of the tile scale; base 256 in FP16, with a
+                                      mixed map base 16 in E4M3); needs 14 b^2 extra
                                       bytes per lower tile and a tile size multiple of 128;
                                    2: as 1, and the TRSMs of a one-matrix factorization
                                       (in core or out of core) run on the emulated engine as
@@ -218,8 +219,8 @@ int tile_chol_precision_map(tc_handle h, int64_t n, int b, const double *A_tiles
  *   updates run on the tensor cores with FP32 accumulation.  FP64 and FP32 updates
  *   follow cfg.fp64_mode: with 0, FP64 on the DFMA pipe and FP32 as three TF32
  *   tensor-core products (hi*hi + hi*lo + lo*hi); with 1 or 2, both as exact products of
- *   base-16 digit planes on the E4M3 tensor cores (14 planes for FP64 outputs, 10 for
- *   FP32, or TF32 x 3 with cfg.fp32_updates = 1) with FP64 sums.  POTRF is FP64; the
+ *   digit planes on the tensor cores (56 bits for FP64 outputs, 40 for FP32, or TF32 x 3
+ *   with cfg.fp32_updates = 1) with sums of at least FP64 precision.  POTRF is FP64; the
  *   TRSM is FP64 substitution (modes 0, 1) or, in mode 2, products with L_kk^{-1} on the
  *   emulated engine (see fp64_mode).  Each final L_mk is then stored in p(m, k).
  * Runs in device memory: the handle holds a working copy of the factor (and, when

@@ -191,7 +191,7 @@ Plan build_plan(tc_handle h, double *W, int *status) {
                     }
                     if (!fp64) continue;
                     if (zmode) {
-                        // emulated FP64: 128 x 16 blocks (the diagonal SYRK keeps blocks reaching the lower part)
+                        // emulated FP64: 128 x zw blocks (the diagonal SYRK keeps blocks reaching the lower part)
                         double *Cp = T(M, m, k);
                         const int xo = (int)(M.tile0 + tidx(m, 0)), yo = (int)(M.tile0 + tidx(k, 0));
                         int items = 0;
@@ -201,9 +201,11 @@ Plan build_plan(tc_handle h, double *W, int *status) {
                             ++items;
                         }, zw);
                         P.update_flops[TC_FP64] += (m == k ? 1.0 : 2.0) * (double)b * b * K;
+                        // all-FP64 plans: 28 base-256 plane pairs per product; mixed ones: base 16
                         for (int nn = 0; nn < k; ++nn)
                             P.tensor_flops[TC_FP64] += 2.0 * 128.0 * zw * b * items *
-                                                       plane_pairs(stored_planes(M, m, nn), stored_planes(M, k, nn), 14);
+                                (zw == Z_BN ? plane_pairs(ZF_PLANES, ZF_PLANES, ZF_PLANES)
+                                            : plane_pairs(stored_planes(M, m, nn), stored_planes(M, k, nn), 14));
                         continue;
                     }
                     jobs_here.push_back((int)P.jobs.size());
@@ -559,7 +561,7 @@ int prepare_factor(tc_handle h, const Plan &P, const MxpPlan *M, PlanDev &D) {
         // digit planes (14 per tile), exponents, amax, the Z items and the digit tile lists
         const int64_t Tt = P.Ttot;
         const size_t bb = (size_t)h->b * h->b;
-        if ((rc = ensure(h, h->dpool, (size_t)Tt * 14 * bb))) return rc;
+        if ((rc = ensure(h, h->dpool, (size_t)Tt * Z_SLOT * bb))) return rc;
         const size_t oz = 0, oy = align_up(P.zitems.size() * sizeof(ZItem));
         const size_t ov = align_up(oy + P.zitems32.size() * sizeof(ZItem));
         const size_t ovc = align_up(ov + P.zinv.size() * sizeof(ZItem));
@@ -615,10 +617,10 @@ int prepare_factor(tc_handle h, const Plan &P, const MxpPlan *M, PlanDev &D) {
             D.pairs = reinterpret_cast<unsigned long long *>(zb + opc);
         }
         h->pairs_dev = D.pairs;
-        if (make_digit_map(&h->map_zx, h->dpool.p, Tt * 14 * h->b, h->b, 128) ||
-            make_digit_map(&h->map_zy, h->dpool.p, Tt * 14 * h->b, h->b, Z_BN))
+        if (P.zwidth == Z_BN && (make_digit_map(&h->map_zx, h->dpool.p, Tt, h->b, 128) ||
+                                 make_digit_map(&h->map_zy, h->dpool.p, Tt, h->b, Z_BN)))
             return set_err(h, TC_ERR_CUDA, "cuTensorMapEncodeTiled failed for the digit planes");
-        if (P.zwidth == Z64_BN && make_zgemm64_maps(&h->maps64, h->dpool.p, Tt * 14, h->b))
+        if (P.zwidth == Z64_BN && make_zgemm64_maps(&h->maps64, h->dpool.p, Tt * Z16_PLANES, h->b))
             return set_err(h, TC_ERR_CUDA, "cuTensorMapEncodeTiled failed for the digit planes (3D maps)");
     }
     D.mixed = M != nullptr;
@@ -667,6 +669,7 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
         CK(cudaMemsetAsync(D.mx.exps16, 0, M->T * sizeof(int), h->s));
         CK(cudaMemsetAsync(D.mx.exps8, 0, M->T * sizeof(int), h->s));
     }
+    const bool e4m3 = P.zwidth == Z64_BN;     // digit planes of k_zgemm64 (mixed precision), else of k_zgemm
     for (int k = 0; k < P.ntmax; ++k) {
         const ColPlan &C = P.cols[k];
         if (C.nit) {
@@ -686,20 +689,16 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
                 launch_zgemm64(h->maps64, D.zitems + C.z0, C.nz, D.zexps, k, b, status + 1, h->s, zp64, 0,
                                wait_limit_ns(h), wait_test(h));
             else
-                launch_zgemm(h->map_zx, h->map_zy, D.zitems + C.z0, C.nz, D.zexps, k, b, status + 1, h->s, 14, 0,
-                             D.zplanes ? &zp64 : nullptr, wait_limit_ns(h), wait_test(h));
+                launch_zgemm(h->map_zx, h->map_zy, D.zitems + C.z0, C.nz, D.zexps, k, b, status + 1, h->s, 14, 0, 0,
+                             wait_limit_ns(h), wait_test(h));
             span_end(h, sp);
             CK_LAUNCH();
             ++h->upd_launches[TC_FP64];
         }
         if (C.ny) {
             const int sp = spans ? span_begin(h, CAT_UPD32) : -1;
-            if (P.zwidth == Z64_BN)
-                launch_zgemm64(h->maps64, D.zitems32 + C.y0, C.ny, D.zexps, k, b, status + 1, h->s, zp32, 0,
-                               wait_limit_ns(h), wait_test(h));
-            else
-                launch_zgemm(h->map_zx, h->map_zy, D.zitems32 + C.y0, C.ny, D.zexps, k, b, status + 1, h->s, 10, 0,
-                             D.zplanes ? &zp32 : nullptr, wait_limit_ns(h), wait_test(h));
+            launch_zgemm64(h->maps64, D.zitems32 + C.y0, C.ny, D.zexps, k, b, status + 1, h->s, zp32, 0,
+                           wait_limit_ns(h), wait_test(h));
             span_end(h, sp);
             CK_LAUNCH();
             ++h->upd_launches[TC_FP32];
@@ -735,7 +734,7 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
                 CK_LAUNCH();
                 launch_tile_amax(W, b, D.dinv + C.ti0, C.nti, D.zamax2, h->s, inv);
                 CK_LAUNCH();
-                launch_digits(W, b, D.dinv + C.ti0, C.nti, D.zamax2, pool, D.zexps, h->s, inv);
+                launch_digits(W, b, D.dinv + C.ti0, C.nti, D.zamax2, pool, D.zexps, h->s, e4m3, inv);
                 CK_LAUNCH();
             } else {                       // one matrix: its shared-memory column panel would not fit
                 const int gkk = (int)(Md.tile0 + tidx(k, k));
@@ -746,30 +745,22 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
                 CK_LAUNCH();
                 launch_amax_ptr(inv, bb, D.zamax2 + gkk, h->s);
                 CK_LAUNCH();
-                launch_digits_src(inv, b, 1, gkk, D.zamax2 + gkk, pool, D.zexps, h->s);
+                launch_digits_src(inv, b, 1, gkk, D.zamax2 + gkk, pool, D.zexps, h->s, e4m3);
                 CK_LAUNCH();
             }
             launch_tile_amax(W, b, D.dtiles + C.dg0, C.ndg, D.zamax2, h->s);
             CK_LAUNCH();
-            launch_digits(W, b, D.dtiles + C.dg0, C.ndg, D.zamax2, pool, D.zexps, h->s);
+            launch_digits(W, b, D.dtiles + C.dg0, C.ndg, D.zamax2, pool, D.zexps, h->s, e4m3);
             CK_LAUNCH();
             if (!P.inv_refine) {
                 // the product's truncation stays below the rounding to each stored precision
                 int off = C.v0;
                 for (int p = 0; p < 4; ++p) {
-                    if (P.zwidth == Z64_BN) {
-                        ZPlanes fixed;                  // every source on the precision's plane count
-                        fixed.src_planes_tab = nullptr;
-                        fixed.out_amax = nullptr;
-                        fixed.rref = ZTRSM_PLANES[p];
-                        fixed.margin = 0;
-                        fixed.pair_count = nullptr;
-                        launch_zgemm64(h->maps64, D.zinv + off, C.nvp[p], D.zexps, 1, b, status + 1, h->s, fixed, 1,
-                                       wait_limit_ns(h), wait_test(h));
-                    } else {
-                        launch_zgemm(h->map_zx, h->map_zy, D.zinv + off, C.nvp[p], D.zexps, 1, b, status + 1, h->s,
-                                     ZTRSM_PLANES[p], 1, nullptr, wait_limit_ns(h), wait_test(h));
-                    }
+                    ZPlanes fixed;                  // every source on the precision's plane count
+                    fixed.rref = ZTRSM_PLANES[p];
+                    fixed.margin = 0;
+                    launch_zgemm64(h->maps64, D.zinv + off, C.nvp[p], D.zexps, 1, b, status + 1, h->s, fixed, 1,
+                                   wait_limit_ns(h), wait_test(h));
                     CK_LAUNCH();
                     off += C.nvp[p];
                 }
@@ -784,22 +775,22 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
                 CK_LAUNCH();
                 launch_digits_src(Lkk, b, 0, gl, am_l + gl, pool, D.zexps, h->s);
                 CK_LAUNCH();
-                launch_zgemm(h->map_zx, h->map_zy, D.zinvc + C.v0, C.nv, D.zexps, 1, b, status + 1, h->s, 14, 1, nullptr,
+                launch_zgemm(h->map_zx, h->map_zy, D.zinvc + C.v0, C.nv, D.zexps, 1, b, status + 1, h->s, 14, 1, 1,
                              wait_limit_ns(h), wait_test(h));
                 CK_LAUNCH();
                 launch_tile_amax(W, b, D.dtiles + C.dg0, C.ndg, am_x, h->s, X0);
                 CK_LAUNCH();
-                launch_digits(W, b, D.dtiles + C.dg0, C.ndg, am_x, pool, D.zexps, h->s, X0);
+                launch_digits(W, b, D.dtiles + C.dg0, C.ndg, am_x, pool, D.zexps, h->s, false, X0);
                 CK_LAUNCH();
-                launch_zgemm(h->map_zx, h->map_zy, D.zref + C.v0, C.nv, D.zexps, 1, b, status + 1, h->s, 14, 0, nullptr,
+                launch_zgemm(h->map_zx, h->map_zy, D.zref + C.v0, C.nv, D.zexps, 1, b, status + 1, h->s, 14, 0, 1,
                              wait_limit_ns(h), wait_test(h));
                 CK_LAUNCH();
                 launch_tile_amax(W, b, D.dtiles + C.dg0, C.ndg, am_r, h->s);
                 CK_LAUNCH();
-                launch_digits(W, b, D.dtiles + C.dg0, C.ndg, am_r, pool, D.zexps, h->s);
+                launch_digits(W, b, D.dtiles + C.dg0, C.ndg, am_r, pool, D.zexps, h->s, false);
                 CK_LAUNCH();
-                launch_zgemm(h->map_zx, h->map_zy, D.zinv + C.v0, C.nv, D.zexps, 1, b, status + 1, h->s, ZREF_PLANES, 1,
-                             nullptr, wait_limit_ns(h), wait_test(h));
+                launch_zgemm(h->map_zx, h->map_zy, D.zinv + C.v0, C.nv, D.zexps, 1, b, status + 1, h->s, ZREF_PLANES, 1, 1,
+                             wait_limit_ns(h), wait_test(h));
                 CK_LAUNCH();
                 launch_add_tiles(W, b, D.dtiles + C.dg0, C.ndg, X0, h->s);
                 CK_LAUNCH();
@@ -820,7 +811,7 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
             const int sp = spans ? span_begin(h, CAT_CONVERT) : -1;
             launch_tile_amax(W, b, D.dtiles + C.dg0, C.ndg, D.zamax, h->s);
             CK_LAUNCH();
-            launch_digits(W, b, D.dtiles + C.dg0, C.ndg, D.zamax, static_cast<uint8_t *>(h->dpool.p), D.zexps, h->s);
+            launch_digits(W, b, D.dtiles + C.dg0, C.ndg, D.zamax, static_cast<uint8_t *>(h->dpool.p), D.zexps, h->s, e4m3);
             span_end(h, sp);
             CK_LAUNCH();
         }

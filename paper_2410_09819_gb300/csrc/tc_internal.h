@@ -204,7 +204,10 @@ inline int tile_ctas(int ntiles) {
     const int c = ntiles > 0 ? 2432 / ntiles : 64;
     return c < 64 ? 64 : (c > 1024 ? 1024 : c);
 }
-constexpr int Z_BN = 16;     // columns of one emulated-update work item (rows: 128)
+constexpr int Z_BN = 32;     // columns of one emulated-update work item (rows: 128)
+// Digit planes of a tile (a slot of 14 b^2 bytes): 7 base-256 planes in FP16 (k_zgemm: all-FP64
+// and out-of-core factorizations) or 14 base-16 planes in E4M3 (k_zgemm64: mixed precision)
+constexpr int ZF_PLANES = 7, Z16_PLANES = 14, Z_SLOT = 14;
 constexpr int Z64_BN = 64;   // columns of a work item of the mixed-precision update kernel (k_ozaki64.cu)
 // 3D maps over the digit-plane pool (K bytes, rows of a plane, plane index) for k_zgemm64:
 // x[d-1] boxes of d X planes (128 rows), y[d-1] boxes of d Y planes (64 rows)
@@ -250,16 +253,22 @@ void launch_qgemm_group(int kind, const CUtensorMap &mx, const CUtensorMap &my, 
 // ------------------------------------------------------------------ launchers (k_ozaki.cu)
 size_t zgemm_smem_bytes();
 void launch_digits(const double *W, int b, const int *tiles, int ntiles, const double *amax, uint8_t *pool, int *exps,
-                   cudaStream_t s, const double *alt = nullptr);
+                   cudaStream_t s, bool e4m3, const double *alt = nullptr);
 void launch_lower_only(double *T, int b, cudaStream_t s);
 void launch_add_tiles(double *W, int b, const int *tiles, int ntiles, const double *src, cudaStream_t s);
 void launch_add_tile(double *dst, const double *src, int b, cudaStream_t s);     // dst += src, one b x b tile
-// planes: digit planes of the output precision (14 FP64, 10 FP32, fewer for TRSM products);
-// src_planes_tab: per digit slot, the leading planes that can be non-zero (nullptr: all);
-// limit_ns: bound of each pipeline wait (0: 4 s), after which *err is set and the call ends;
-// stall != 0: the failure-detection test hook (the MMA issuer waits on a barrier nothing arrives at).
-// Plane counts of a mixed-precision update launch (k_zgemm's SKIP form): per source, the X / Y
-// planes its stored formats can have non-zero (src_planes_tab), and a pair budget relative to
+// Products on base-256 planes.  planes: base-16 digits that the result is to be worth (14 FP64,
+// 10 FP32 outputs, fewer for TRSM products); assign: C = sum X Y^T instead of C -= it; tri: the
+// Y tiles are lower triangular; limit_ns: bound of each pipeline wait (0: 4 s), after which *err
+// is set and the call ends; stall != 0: the failure-detection test hook (the MMA issuer waits on
+// a barrier nothing arrives at).
+void launch_zgemm(const CUtensorMap &mx, const CUtensorMap &my, const ZItem *items, int nitems, const int *exps, int k,
+                  int b, int *err, cudaStream_t s, int planes, int assign, int tri, unsigned long long limit_ns,
+                  int stall);
+void launch_zgemm_group(const CUtensorMap &mx, const CUtensorMap &my, const ZGroup &g, const int *exps, int b,
+                        int *err, cudaStream_t s, int planes, int tri, unsigned long long limit_ns, int stall);
+// Plane counts of a mixed-precision update launch (k_zgemm64): per source, the X / Y planes its
+// stored formats can have non-zero (src_planes_tab; nullptr: all), and a pair budget relative to
 // the output tile's scale: su = rref - floor((e_out - e_x - e_y - 4 margin) / 4), within
 // [1, 14], e_out the digit exponent of the output tile's input amax (out_amax[it.ct]).  The
 // launch adds the plane pairs it multiplies to *pair_count.
@@ -269,16 +278,11 @@ struct ZPlanes {
     int rref = 14, margin = 2;
     unsigned long long *pair_count = nullptr;
 };
-void launch_zgemm(const CUtensorMap &mx, const CUtensorMap &my, const ZItem *items, int nitems, const int *exps, int k,
-                  int b, int *err, cudaStream_t s, int planes = 14, int assign = 0,
-                  const ZPlanes *mixed = nullptr, unsigned long long limit_ns = 0, int stall = 0);
-void launch_zgemm_group(const CUtensorMap &mx, const CUtensorMap &my, const ZGroup &g, const int *exps, int b,
-                        int *err, cudaStream_t s, int planes = 14, unsigned long long limit_ns = 0, int stall = 0);
 void launch_digits_src(const double *src, int b, int transpose, int dst, const double *amax, uint8_t *pool, int *exps,
-                       cudaStream_t s);
+                       cudaStream_t s, bool e4m3 = false);
 void launch_amax_ptr(const double *src, int64_t count, double *out, cudaStream_t s);
 void launch_set_identity(double *T, int b, cudaStream_t s);
-int make_digit_map(CUtensorMap *map, void *pool, int64_t rows, int b, int box_rows);
+int make_digit_map(CUtensorMap *map, void *pool, int64_t nslots, int b, int box_rows);
 
 // ------------------------------------------------------------------ launchers (k_mxp.cu)
 int make_pool_map(CUtensorMap *map, void *pool, int64_t nslots, int b, int esize, int box_rows);

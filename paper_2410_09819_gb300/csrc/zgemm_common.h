@@ -58,6 +58,11 @@ __device__ __forceinline__ uint64_t z_desc(uint32_t saddr) {   // K-major, 128-b
     return (uint64_t)((saddr & 0x3FFFF) >> 4) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) |
            (2ull << 61);
 }
+// the same with rows of 64 bytes and the 64-byte swizzle (8-row groups 512 bytes apart)
+__device__ __forceinline__ uint64_t z_desc64(uint32_t saddr) {
+    return (uint64_t)((saddr & 0x3FFFF) >> 4) | (1ull << 16) | ((uint64_t)(512 >> 4) << 32) | (1ull << 46) |
+           (4ull << 61);
+}
 __device__ __forceinline__ void z_mma(uint32_t d, uint64_t a, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
@@ -83,6 +88,63 @@ __device__ __forceinline__ void z_mma3(uint32_t d, uint64_t a, uint64_t b, uint3
         "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %4, %5, %3, q;\n\t"
         "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %6, %7, %3, q;\n\t}\n" ::"r"(d),
         "l"(a + 2), "l"(b + 2), "r"(idesc), "l"(a + 4), "l"(b + 4), "l"(a + 6), "l"(b + 6));
+}
+// Forms for a whole converged warp: elect.sync picks the issuing lane inside the asm block, so the
+// operands stay warp-uniform registers.  From a one-lane branch (if (lane == 0)) every tcgen05.mma
+// cost the issuing thread 47 cycles, and so became the floor of short MMAs; in this form it costs
+// 9, and an MMA of M = 128 then runs at max(41, N / 2) cycles (measured, K = 32 bytes).
+__device__ __forceinline__ bool z_wait_all(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
+                                           unsigned long long limit_ns) {
+    return __all_sync(0xffffffffu, z_wait(bar, parity, abort_flag, limit_ns));
+}
+__device__ __forceinline__ void z_commit_w(uint64_t *bar) {
+    asm volatile(
+        "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(z_smem(bar))
+        : "memory");
+}
+__device__ __forceinline__ void z_expect_w(uint64_t *bar, uint32_t bytes) {
+    asm volatile(
+        "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+        "@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}\n" ::"r"(z_smem(bar)), "r"(bytes)
+        : "memory");
+}
+__device__ __forceinline__ void z_tma_w(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar) {
+    asm volatile(
+        "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+        "@e cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n\t}\n" ::"r"(
+            z_smem(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z_smem(bar))
+        : "memory");
+}
+// The two MMAs of one 64-byte K block with FP16 operands (kind::f16; 16 elements = 32 bytes of K
+// per MMA): the first takes the accumulate predicate, the second accumulates.
+__device__ __forceinline__ void z_mma2_h(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred e, p, q;\n\telect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 q, %4, %4;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %5, %6, %3, q;\n\t}\n" ::"r"(d),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc), "l"(a + 2), "l"(b + 2));
+}
+// two 16-column TMEM loads in flight before one wait
+__device__ __forceinline__ void z_ld16x2(uint32_t t0, uint32_t t1, float (&u)[16], float (&v)[16]) {
+    uint32_t r[16], q[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(t0));
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(q[0]), "=r"(q[1]), "=r"(q[2]), "=r"(q[3]), "=r"(q[4]), "=r"(q[5]), "=r"(q[6]), "=r"(q[7]),
+          "=r"(q[8]), "=r"(q[9]), "=r"(q[10]), "=r"(q[11]), "=r"(q[12]), "=r"(q[13]), "=r"(q[14]), "=r"(q[15])
+        : "r"(t1));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        u[i] = __uint_as_float(r[i]);
+        v[i] = __uint_as_float(q[i]);
+    }
 }
 __device__ __forceinline__ void z_ld16(uint32_t taddr, float (&v)[16]) {
     uint32_t r[16];
