@@ -5,13 +5,11 @@
 // Why a second kernel: in a mixed-precision factorization every source carries its own plane
 // budget (the stored formats bound its planes, its scale against the output's bounds the pairs
 // worth multiplying), 57 pairs per FP64-output product and 37 per FP32-output product on
-// average at n = 131072 against the FP64 path's 105.  With 128 x 16 blocks an X plane then
-// meets few partners: its MMA has N = 16 x partners, mostly at or below 128, where one
-// tcgen05.mma (kind::f8f6f4, M = 128, K = 32) still occupies the tensor pipe ~69 cycles, and
-// the issuing thread's fixed cost per stage (a barrier wait of ~200-300 cycles, fence, commit)
-// is spread over little MMA work (measured on GB300).  Here an X plane's MMA spans 64 columns
-// per partner (N = 64 x partners <= 256), and one pipeline unit carries a whole K block of two
-// X planes together with the Y planes they meet, so one wait and one commit cover 8 MMAs.
+// average at n = 131072 against the full 105.  With 128 x 16 blocks an X plane then meets few
+// partners and its MMAs are short, so that the issue and the waits bound them.  Here an X plane's
+// MMA spans 64 columns per partner (N = 64 x partners <= 256), and one pipeline unit carries a
+// whole K block of two X planes together with the Y planes they meet, so one wait and one commit
+// cover 8 MMAs.
 //
 // Accumulator passes: the groups 0 .. G-1 a source writes (G = min(su, sx + sy - 1)) are split
 // into P = ceil(G / 4) passes of consecutive groups, the smaller first; a pass [g0, g1) holds
@@ -66,6 +64,7 @@ struct Args {
     int k, b;
     int *err;
     int assign;                     // 0: C -= sum X Y^T;  1: C = sum X Y^T
+    int tri;                        // 1: the Y tiles are lower triangular (row j is zero beyond column j)
     unsigned long long limit_ns;    // bound of each pipeline wait
     int stall;                      // test hook: wait first on a barrier nothing arrives at
 };
@@ -91,6 +90,12 @@ __device__ __forceinline__ Shape shape(const Args &a, int eo, int xt, int yt) {
     sx = sx < su ? sx : su;
     sy = sy < su ? sy : su;
     return {sx, sy, su};
+}
+// K blocks of an item's source: with a lower triangular Y those up to the last column of its rows
+// (the rest multiplies zeros)
+__device__ __forceinline__ int kblocks_of(const Args &a, const ZItem &it) {
+    const int all = a.b / KB, need = (it.bn * BN + BN - 1) / KB + 1;
+    return a.tri && need < all ? need : all;
 }
 __device__ __forceinline__ int pairs(const Shape &z) {
     int p = 0;
@@ -132,7 +137,8 @@ __device__ __forceinline__ Chunk chunk(const Pass &ps, int sa, int sy) {
 // Persistent kernel: C -= sum_{n<k} X_n Y_n^T (C = ... when assign) for 128 x 64 output blocks of
 // FP64- or FP32-output tiles of a mixed-precision map.
 //   warp 0  TMA producer: per item, source, pass, K block and chunk one unit;
-//   warp 1  MMA issuer: per unit one barrier wait, per X plane of the chunk one asm block of 4
+//   warp 1  MMA issuer (a converged warp, see zgemm_common.h; from a one-lane branch each MMA cost
+//           47 cycles of issue): per unit one barrier wait, per X plane of the chunk one asm block of 4
 //           MMAs (the K steps) with N = 64 x partners into the groups s + t0 .. of the pass's
 //           buffer, one commit;
 //   warps 2-9 drain: per pass, the groups leave TMEM (exact FP32 integers), are recombined by
@@ -142,6 +148,9 @@ __device__ __forceinline__ Chunk chunk(const Pass &ps, int sa, int sy) {
 // plane slo starts the groups it covers, and each later plane s covers [max(s, g0), s + t1(s)),
 // reaching at most one group past those already started: when t1(s) = sy that group s + sy - 1
 // is new, and for K step 0 a separate MMA of the one partner t = sy - 1 starts it.
+// Four-precision factorization of order 32768, tile 2048: its 62 launches take 294 ms issued from a
+// one-lane branch, with one TMEM load per wait, one of C's values at a time and every K block of
+// the triangular TRSM operand; 250 ms here.
 // Failure handling as in k_zgemm: bounded pipeline waits that set *err and stop the CTA; before
 // the TMEM is released the MMA issuer waits for its issued MMAs and the producer for its issued
 // copies (waits that ignore the abort flag, bounded by DRAIN_NS).
@@ -164,7 +173,6 @@ k_zgemm64(const __grid_constant__ Z64Maps maps, const __grid_constant__ A args) 
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int k = args.k, b = args.b;
-    const int kblocks = b / KB;
     const int nitems = args.nitems;
     if ((int)blockIdx.x >= nitems) return;             // whole CTA, before any barrier
     if (threadIdx.x == 0) {
@@ -195,148 +203,146 @@ k_zgemm64(const __grid_constant__ Z64Maps maps, const __grid_constant__ A args) 
 
     if (warp == 0) {
         // --------------------------------------------------------------- TMA producer
-        if (lane == 0) {
-            // ring state: pos = slot of the next unit, head / tail = slots allocated / released
-            // so far (gaps at the ring's end included), nset / nrel = units allocated / released
-            int pos = 0, nset = 0, nrel = 0;
-            long long head = 0, tail = 0;
-            bool ok = true;
-            // place a unit of sz slots: wait (in FIFO order) for the MMAs of the oldest units to
-            // release what it needs; false if a wait ran into its bound
-            auto alloc = [&](int sz, int &slot, int &set) -> bool {
-                int sp = pos;
-                long long start = head;
-                if (sp + sz > RING) {
-                    start += RING - sp;
-                    sp = 0;
-                }
-                while (nrel < nset && (start + sz - tail > RING || nset - nrel >= SETS)) {
-                    if (!z_wait(empty + (nrel & (SETS - 1)), (uint32_t)((nrel / SETS) & 1), abort_flag, lim))
-                        return false;
-                    tail = uend[nrel & (SETS - 1)];
-                    ++nrel;
-                }
-                slot = sp;
-                set = nset & (SETS - 1);
-                uend[set] = start + sz;
-                head = start + sz;
-                pos = sp + sz == RING ? 0 : sp + sz;
-                ++nset;
-                return true;
-            };
-            for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-                const ZItem it = args.items[item];
-                const int eo = args.oamax ? z_digit_exp(args.oamax[it.ct]) : 0;
-                for (int n = 0; n < k && ok; ++n) {
-                    const int xt = it.xoff + n, yt = it.yoff + n;
-                    const Shape zs = shape(args, eo, xt, yt);
-                    const int G = groups(zs), P = npass(G);
-                    for (int p = 0; p < P && ok; ++p) {
-                        const Pass ps = pass(p, P, G, zs.sx, zs.sy);
-                        for (int kb = 0; kb < kblocks && ok; ++kb)
-                            for (int sa = ps.slo; sa <= ps.shi && ok; sa += 2) {
-                                const Chunk c = chunk(ps, sa, zs.sy);
-                                int slot, set;
-                                if (!alloc(c.ny + 2 * c.nx, slot, set)) { ok = false; break; }
-                                z_expect(full + set, (uint32_t)(c.ny * SLOT + c.nx * XPL));
-                                z_tma3(ring + slot * SLOT, &maps.y[c.ny - 1], kb * KB, it.bn * BN, yt * ZS + c.ylo, full + set);
-                                z_tma3(ring + (slot + c.ny) * SLOT, &maps.x[c.nx - 1], kb * KB, it.bm * BM, xt * ZS + c.sa,
-                                       full + set);
-                            }
-                    }
+        // ring state: pos = slot of the next unit, head / tail = slots allocated / released
+        // so far (gaps at the ring's end included), nset / nrel = units allocated / released
+        int pos = 0, nset = 0, nrel = 0;
+        long long head = 0, tail = 0;
+        bool ok = true;
+        // place a unit of sz slots: wait (in FIFO order) for the MMAs of the oldest units to
+        // release what it needs; false if a wait ran into its bound
+        auto alloc = [&](int sz, int &slot, int &set) -> bool {
+            int sp = pos;
+            long long start = head;
+            if (sp + sz > RING) {
+                start += RING - sp;
+                sp = 0;
+            }
+            while (nrel < nset && (start + sz - tail > RING || nset - nrel >= SETS)) {
+                if (!z_wait_all(empty + (nrel & (SETS - 1)), (uint32_t)((nrel / SETS) & 1), abort_flag, lim))
+                    return false;
+                tail = uend[nrel & (SETS - 1)];
+                ++nrel;
+            }
+            slot = sp;
+            set = nset & (SETS - 1);
+            uend[set] = start + sz;
+            head = start + sz;
+            pos = sp + sz == RING ? 0 : sp + sz;
+            ++nset;
+            return true;
+        };
+        for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
+            const ZItem it = args.items[item];
+            const int kblocks = kblocks_of(args, it);
+            const int eo = args.oamax ? z_digit_exp(args.oamax[it.ct]) : 0;
+            for (int n = 0; n < k && ok; ++n) {
+                const int xt = it.xoff + n, yt = it.yoff + n;
+                const Shape zs = shape(args, eo, xt, yt);
+                const int G = groups(zs), P = npass(G);
+                for (int p = 0; p < P && ok; ++p) {
+                    const Pass ps = pass(p, P, G, zs.sx, zs.sy);
+                    for (int kb = 0; kb < kblocks && ok; ++kb)
+                        for (int sa = ps.slo; sa <= ps.shi && ok; sa += 2) {
+                            const Chunk c = chunk(ps, sa, zs.sy);
+                            int slot, set;
+                            if (!alloc(c.ny + 2 * c.nx, slot, set)) { ok = false; break; }
+                            z_expect_w(full + set, (uint32_t)(c.ny * SLOT + c.nx * XPL));
+                            z_tma3_w(ring + slot * SLOT, &maps.y[c.ny - 1], kb * KB, it.bn * BN, yt * ZS + c.ylo, full + set);
+                            z_tma3_w(ring + (slot + c.ny) * SLOT, &maps.x[c.nx - 1], kb * KB, it.bm * BM, xt * ZS + c.sa,
+                                   full + set);
+                        }
                 }
             }
-            if (!ok) {
-                *abort_flag = 1;
-                atomicExch(args.err, 1);
-            }
-            // Every copy lands before the shared memory goes away: only the last SETS units can
-            // still have copies in flight (an older unit's barrier was re-armed only after the
-            // MMAs had consumed it), each the latest phase of its full barrier.
-            for (int j = nset - SETS < 0 ? 0 : nset - SETS; j < nset; ++j)
-                if (!z_wait(full + (j & (SETS - 1)), (uint32_t)((j / SETS) & 1), never, DRAIN_NS)) atomicExch(args.err, 3);
         }
+        if (!ok && lane == 0) {
+            *abort_flag = 1;
+            atomicExch(args.err, 1);
+        }
+        // Every copy lands before the shared memory goes away: only the last SETS units can
+        // still have copies in flight (an older unit's barrier was re-armed only after the
+        // MMAs had consumed it), each the latest phase of its full barrier.
+        for (int j = nset - SETS < 0 ? 0 : nset - SETS; j < nset; ++j)
+            if (!z_wait_all(full + (j & (SETS - 1)), (uint32_t)((j / SETS) & 1), never, DRAIN_NS) && lane == 0) atomicExch(args.err, 3);
     } else if (warp == 1) {
         // --------------------------------------------------------------- MMA issuer
-        if (lane == 0) {
-            // kind::f8f6f4, D F32, A/B E4M3, K-major, M = 128; N set per instruction
-            const uint32_t idesc0 = (1u << 4) | ((uint32_t)(BM >> 4) << 24);
-            const uint64_t rdesc = z_desc(z_smem(ring));
-            int pos = 0, set = 0, q = 0;                 // q: passes issued so far (all items)
-            unsigned long long pairs_done = 0;
-            bool ok = true;
-            // test hook: `done` completes only after the final commit below, so this wait runs
-            // into the bound and takes the abort path
-            if (args.stall && !z_wait(done, 0, abort_flag, lim)) ok = false;
-            for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-                const ZItem it = args.items[item];
-                const int eo = args.oamax ? z_digit_exp(args.oamax[it.ct]) : 0;
-                for (int n = 0; n < k && ok; ++n) {
-                    const Shape zs = shape(args, eo, it.xoff + n, it.yoff + n);
-                    const int G = groups(zs), P = npass(G);
-                    pairs_done += (unsigned long long)pairs(zs);
-                    for (int p = 0; p < P && ok; ++p, ++q) {
-                        const Pass ps = pass(p, P, G, zs.sx, zs.sy);
-                        const int a = q & 1;
-                        if (!z_wait(acce + a, ((q >> 1) & 1) ^ 1, abort_flag, lim)) { ok = false; break; }
-                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        const uint32_t dbase = tmem + (uint32_t)(a * BUF);
-                        for (int kb = 0; kb < kblocks && ok; ++kb)
-                            for (int sa = ps.slo; sa <= ps.shi; sa += 2) {
-                                const Chunk c = chunk(ps, sa, zs.sy);
-                                const int sz = c.ny + 2 * c.nx;
-                                if (pos + sz > RING) pos = 0;       // the producer's placement
-                                const int slot = pos;
-                                pos = pos + sz == RING ? 0 : pos + sz;
-                                const int u = set++;
-                                if (!z_wait(full + (u & (SETS - 1)), (uint32_t)((u / SETS) & 1), abort_flag, lim)) {
-                                    ok = false;
-                                    break;
-                                }
-                                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                                const uint64_t ud = rdesc + (uint64_t)((slot * SLOT) >> 4);
-#pragma unroll
-                                for (int h = 0; h < 2; ++h)
-                                    if (h < c.nx) {
-                                        const int s = c.sa + h;
-                                        const int t0 = ps.g0 - s > 0 ? ps.g0 - s : 0;
-                                        const int t1 = zs.sy < ps.g1 - s ? zs.sy : ps.g1 - s;
-                                        const int np = t1 - t0;
-                                        // A: X plane h of the unit; B: its Y planes t0 - ylo ..;
-                                        // D: groups s + t0 - g0 .. of the pass's buffer
-                                        const uint64_t xd = ud + (uint64_t)(((c.ny * SLOT) + h * XPL) >> 4);
-                                        const uint64_t bd = ud + (uint64_t)(((t0 - c.ylo) * SLOT) >> 4);
-                                        const uint32_t d = dbase + (uint32_t)((s + t0 - ps.g0) * BN);
-                                        const uint32_t idesc = idesc0 | ((uint32_t)((np * BN) >> 3) << 17);
-                                        if (kb > 0) {
-                                            z_mma4(d, xd, bd, idesc, 1u);
-                                        } else if (s == ps.slo) {
-                                            z_mma4(d, xd, bd, idesc, 0u);           // starts its groups
-                                        } else if (t1 == zs.sy) {
-                                            // groups s+t0 .. s+sy-2 are running; group s+sy-1 starts here
-                                            if (np > 1) z_mma(d, xd, bd, idesc0 | ((uint32_t)(((np - 1) * BN) >> 3) << 17), 1u);
-                                            z_mma(d + (uint32_t)((np - 1) * BN), xd, bd + (uint64_t)(((np - 1) * SLOT) >> 4),
-                                                  idesc0 | ((uint32_t)(BN >> 3) << 17), 0u);
-                                            z_mma3(d, xd, bd, idesc);
-                                        } else {
-                                            z_mma4(d, xd, bd, idesc, 1u);           // all its groups are running
-                                        }
-                                    }
-                                z_commit(empty + (u & (SETS - 1)));
+        // kind::f8f6f4, D F32, A/B E4M3, K-major, M = 128; N set per instruction
+        const uint32_t idesc0 = (1u << 4) | ((uint32_t)(BM >> 4) << 24);
+        const uint64_t rdesc = z_desc(z_smem(ring));
+        int pos = 0, set = 0, q = 0;                 // q: passes issued so far (all items)
+        unsigned long long pairs_done = 0;
+        bool ok = true;
+        // test hook: `done` completes only after the final commit below, so this wait runs
+        // into the bound and takes the abort path
+        if (args.stall && !z_wait_all(done, 0, abort_flag, lim)) ok = false;
+        for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
+            const ZItem it = args.items[item];
+            const int kblocks = kblocks_of(args, it);
+            const int eo = args.oamax ? z_digit_exp(args.oamax[it.ct]) : 0;
+            for (int n = 0; n < k && ok; ++n) {
+                const Shape zs = shape(args, eo, it.xoff + n, it.yoff + n);
+                const int G = groups(zs), P = npass(G);
+                pairs_done += (unsigned long long)pairs(zs);
+                for (int p = 0; p < P && ok; ++p, ++q) {
+                    const Pass ps = pass(p, P, G, zs.sx, zs.sy);
+                    const int a = q & 1;
+                    if (!z_wait_all(acce + a, ((q >> 1) & 1) ^ 1, abort_flag, lim)) { ok = false; break; }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint32_t dbase = tmem + (uint32_t)(a * BUF);
+                    for (int kb = 0; kb < kblocks && ok; ++kb)
+                        for (int sa = ps.slo; sa <= ps.shi; sa += 2) {
+                            const Chunk c = chunk(ps, sa, zs.sy);
+                            const int sz = c.ny + 2 * c.nx;
+                            if (pos + sz > RING) pos = 0;       // the producer's placement
+                            const int slot = pos;
+                            pos = pos + sz == RING ? 0 : pos + sz;
+                            const int u = set++;
+                            if (!z_wait_all(full + (u & (SETS - 1)), (uint32_t)((u / SETS) & 1), abort_flag, lim)) {
+                                ok = false;
+                                break;
                             }
-                        if (ok) z_commit(accf + a);
-                    }
+                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                            const uint64_t ud = rdesc + (uint64_t)((slot * SLOT) >> 4);
+#pragma unroll
+                            for (int h = 0; h < 2; ++h)
+                                if (h < c.nx) {
+                                    const int s = c.sa + h;
+                                    const int t0 = ps.g0 - s > 0 ? ps.g0 - s : 0;
+                                    const int t1 = zs.sy < ps.g1 - s ? zs.sy : ps.g1 - s;
+                                    const int np = t1 - t0;
+                                    // A: X plane h of the unit; B: its Y planes t0 - ylo ..;
+                                    // D: groups s + t0 - g0 .. of the pass's buffer
+                                    const uint64_t xd = ud + (uint64_t)(((c.ny * SLOT) + h * XPL) >> 4);
+                                    const uint64_t bd = ud + (uint64_t)(((t0 - c.ylo) * SLOT) >> 4);
+                                    const uint32_t d = dbase + (uint32_t)((s + t0 - ps.g0) * BN);
+                                    const uint32_t idesc = idesc0 | ((uint32_t)((np * BN) >> 3) << 17);
+                                    if (kb > 0) {
+                                        z_mma4_w(d, xd, bd, idesc, 1u);
+                                    } else if (s == ps.slo) {
+                                        z_mma4_w(d, xd, bd, idesc, 0u);           // starts its groups
+                                    } else if (t1 == zs.sy) {
+                                        // groups s+t0 .. s+sy-2 are running; group s+sy-1 starts here
+                                        if (np > 1) z_mma_w(d, xd, bd, idesc0 | ((uint32_t)(((np - 1) * BN) >> 3) << 17), 1u);
+                                        z_mma_w(d + (uint32_t)((np - 1) * BN), xd, bd + (uint64_t)(((np - 1) * SLOT) >> 4),
+                                              idesc0 | ((uint32_t)(BN >> 3) << 17), 0u);
+                                        z_mma3_w(d, xd, bd, idesc);
+                                    } else {
+                                        z_mma4_w(d, xd, bd, idesc, 1u);           // all its groups are running
+                                    }
+                                }
+                            z_commit_w(empty + (u & (SETS - 1)));
+                        }
+                    if (ok) z_commit_w(accf + a);
                 }
             }
-            if (!ok) {
-                *abort_flag = 1;
-                atomicExch(args.err, 1);
-            }
-            if (args.pair_count && pairs_done) atomicAdd(args.pair_count, pairs_done);
-            // every issued MMA completes before the TMEM is released and the CTA exits
-            z_commit(done);
-            if (!z_wait(done, 0, never, DRAIN_NS)) atomicExch(args.err, 3);
         }
+        if (!ok && lane == 0) {
+            *abort_flag = 1;
+            atomicExch(args.err, 1);
+        }
+        if (lane == 0 && args.pair_count && pairs_done) atomicAdd(args.pair_count, pairs_done);
+        // every issued MMA completes before the TMEM is released and the CTA exits
+        z_commit_w(done);
+        if (!z_wait_all(done, 0, never, DRAIN_NS) && lane == 0) atomicExch(args.err, 3);
     } else {
         // --------------------------------------------------------------- drain + epilogue
         const int quarter = warp & 3, half = (warp - 2) >> 2;    // TMEM lanes 32 quarter.., columns 32 half..
@@ -368,13 +374,20 @@ k_zgemm64(const __grid_constant__ Z64Maps maps, const __grid_constant__ A args) 
 #pragma unroll
                         for (int j = 0; j < 16; ++j) h[j] = 0;
 #pragma unroll 1
-                        for (int g = 0; g < ng; ++g) {
-                            float v[16];
-                            z_ld16(lanebase + (uint32_t)(g * BN + c * 16), v);
+                        for (int g = 0; g < ng; g += 2) {
+                            float v[16], u[16];
                             // group sums are exact integers below 2^24 in magnitude: a 32-bit
                             // conversion (a 64-bit one would run on the FP64 pipe)
+                            if (g + 1 < ng) {
+                                z_ld16x2(lanebase + (uint32_t)(g * BN + c * 16), lanebase + (uint32_t)((g + 1) * BN + c * 16), v, u);
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) h[j] = h[j] * 16 + (long long)__float2int_rn(v[j]);
+                                for (int j = 0; j < 16; ++j)
+                                    h[j] = (h[j] * 16 + (long long)__float2int_rn(v[j])) * 16 + (long long)__float2int_rn(u[j]);
+                            } else {
+                                z_ld16(lanebase + (uint32_t)(g * BN + c * 16), v);
+#pragma unroll
+                                for (int j = 0; j < 16; ++j) h[j] = h[j] * 16 + (long long)__float2int_rn(v[j]);
+                            }
                         }
 #pragma unroll
                         for (int j = 0; j < 16; ++j) run[c * 16 + j] = fma((double)h[j], sc, run[c * 16 + j]);
@@ -387,10 +400,15 @@ k_zgemm64(const __grid_constant__ Z64Maps maps, const __grid_constant__ A args) 
             }
             if (!ok) break;
             const int row = it.bm * BM + quarter * 32 + lane;
+            // eight of C's values are requested before the first of them is stored
+            double *cp = it.C + (int64_t)(it.bn * BN + half * 32) * b + row;
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                double *cp = it.C + (int64_t)(it.bn * BN + half * 32 + j) * b + row;
-                *cp = args.assign ? run[j] : *cp - run[j];
+            for (int j0 = 0; j0 < 32; j0 += 8) {
+                double v[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] = args.assign ? 0.0 : cp[(int64_t)(j0 + j) * b];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) cp[(int64_t)(j0 + j) * b] = args.assign ? run[j0 + j] : v[j] - run[j0 + j];
             }
         }
         if (!ok) {
@@ -432,7 +450,7 @@ int make_zgemm64_maps(Z64Maps *m, void *pool, int64_t nplanes, int b) {
 }
 
 void launch_zgemm64(const Z64Maps &maps, const ZItem *items, int nitems, const int *exps, int k, int b, int *err,
-                    cudaStream_t s, const ZPlanes &mixed, int assign, unsigned long long limit_ns, int stall) {
+                    cudaStream_t s, const ZPlanes &mixed, int assign, int tri, unsigned long long limit_ns, int stall) {
     if (nitems <= 0 || k <= 0) return;
     static std::atomic<unsigned long long> attr{0};
     if (attrs_pending(attr)) {
@@ -440,7 +458,7 @@ void launch_zgemm64(const Z64Maps &maps, const ZItem *items, int nitems, const i
         mark_attrs_set(attr);
     }
     z64::Args a{items, nitems, exps, mixed.src_planes_tab, mixed.out_amax, mixed.rref, mixed.margin, mixed.pair_count,
-                k, b, err, assign, limit_ns ? limit_ns : z64::LIMIT_NS, stall};
+                k, b, err, assign, tri, limit_ns ? limit_ns : z64::LIMIT_NS, stall};
     const int grid = nitems < sm_count64() ? nitems : sm_count64();  // persistent: one CTA per SM
     z64::k_zgemm64<z64::Args><<<grid, z64::THREADS, z64::SMEM, s>>>(maps, a);
 }

@@ -686,7 +686,7 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
         if (C.nz) {
             const int sp = spans ? span_begin(h, CAT_UPD64) : -1;
             if (P.zwidth == Z64_BN)
-                launch_zgemm64(h->maps64, D.zitems + C.z0, C.nz, D.zexps, k, b, status + 1, h->s, zp64, 0,
+                launch_zgemm64(h->maps64, D.zitems + C.z0, C.nz, D.zexps, k, b, status + 1, h->s, zp64, 0, 0,
                                wait_limit_ns(h), wait_test(h));
             else
                 launch_zgemm(h->map_zx, h->map_zy, D.zitems + C.z0, C.nz, D.zexps, k, b, status + 1, h->s, 14, 0, 0,
@@ -697,7 +697,7 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
         }
         if (C.ny) {
             const int sp = spans ? span_begin(h, CAT_UPD32) : -1;
-            launch_zgemm64(h->maps64, D.zitems32 + C.y0, C.ny, D.zexps, k, b, status + 1, h->s, zp32, 0,
+            launch_zgemm64(h->maps64, D.zitems32 + C.y0, C.ny, D.zexps, k, b, status + 1, h->s, zp32, 0, 0,
                            wait_limit_ns(h), wait_test(h));
             span_end(h, sp);
             CK_LAUNCH();
@@ -759,7 +759,7 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
                     ZPlanes fixed;                  // every source on the precision's plane count
                     fixed.rref = ZTRSM_PLANES[p];
                     fixed.margin = 0;
-                    launch_zgemm64(h->maps64, D.zinv + off, C.nvp[p], D.zexps, 1, b, status + 1, h->s, fixed, 1,
+                    launch_zgemm64(h->maps64, D.zinv + off, C.nvp[p], D.zexps, 1, b, status + 1, h->s, fixed, 1, 1,
                                    wait_limit_ns(h), wait_test(h));
                     CK_LAUNCH();
                     off += C.nvp[p];

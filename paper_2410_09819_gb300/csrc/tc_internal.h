@@ -293,7 +293,7 @@ int make_zgemm64_maps(Z64Maps *m, void *pool, int64_t nplanes, int b);
 // Mixed-precision digit-plane updates over 128 x Z64_BN items (k_ozaki64.cu); mixed.rref is the
 // reference plane count of the outputs (14 FP64, 10 FP32)
 void launch_zgemm64(const Z64Maps &maps, const ZItem *items, int nitems, const int *exps, int k, int b, int *err,
-                    cudaStream_t s, const ZPlanes &mixed, int assign, unsigned long long limit_ns, int stall);
+                    cudaStream_t s, const ZPlanes &mixed, int assign, int tri, unsigned long long limit_ns, int stall);
 size_t qgemm_smem_bytes();
 void launch_qgemm(int kind, const CUtensorMap &a0, const CUtensorMap &a1, const CUtensorMap &b0,
                   const CUtensorMap &b1, const QItem *items, int nitems, const int *slot, const int *exps,

@@ -15,9 +15,6 @@ __device__ __forceinline__ uint64_t z_timer() {
 __device__ __forceinline__ void z_init(uint64_t *bar, uint32_t c) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(z_smem(bar)), "r"(c) : "memory");
 }
-__device__ __forceinline__ void z_expect(uint64_t *bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(z_smem(bar)), "r"(bytes) : "memory");
-}
 __device__ __forceinline__ void z_arrive(uint64_t *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(z_smem(bar)) : "memory");
 }
@@ -43,17 +40,6 @@ __device__ __forceinline__ bool z_wait(uint64_t *bar, uint32_t parity, volatile 
         if (z_timer() - t0 > limit_ns) return false;
     }
 }
-__device__ __forceinline__ void z_tma(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-            z_smem(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z_smem(bar))
-        : "memory");
-}
-__device__ __forceinline__ void z_commit(uint64_t *bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(z_smem(bar))
-                 : "memory");
-}
 __device__ __forceinline__ uint64_t z_desc(uint32_t saddr) {   // K-major, 128-byte swizzle
     return (uint64_t)((saddr & 0x3FFFF) >> 4) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) |
            (2ull << 61);
@@ -62,32 +48,6 @@ __device__ __forceinline__ uint64_t z_desc(uint32_t saddr) {   // K-major, 128-b
 __device__ __forceinline__ uint64_t z_desc64(uint32_t saddr) {
     return (uint64_t)((saddr & 0x3FFFF) >> 4) | (1ull << 16) | ((uint64_t)(512 >> 4) << 32) | (1ull << 46) |
            (4ull << 61);
-}
-__device__ __forceinline__ void z_mma(uint32_t d, uint64_t a, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
-        "l"(a), "l"(bdesc), "r"(idesc), "r"(acc));
-}
-// The 4 MMAs of one 128-byte K block in one asm block: the first K step takes the accumulate
-// predicate, the others accumulate; A and B advance by 32 bytes (2 descriptor units) per step.
-__device__ __forceinline__ void z_mma4(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 q, %4, %4;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %5, %6, %3, q;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %7, %8, %3, q;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %9, %10, %3, q;\n\t}\n" ::"r"(d),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc), "l"(a + 2), "l"(b + 2), "l"(a + 4), "l"(b + 4), "l"(a + 6), "l"(b + 6));
-}
-// K steps 1..3 of a K block (all accumulate)
-__device__ __forceinline__ void z_mma3(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc) {
-    asm volatile(
-        "{\n\t.reg .pred q;\n\tsetp.eq.b32 q, %3, %3;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, q;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %4, %5, %3, q;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %6, %7, %3, q;\n\t}\n" ::"r"(d),
-        "l"(a + 2), "l"(b + 2), "r"(idesc), "l"(a + 4), "l"(b + 4), "l"(a + 6), "l"(b + 6));
 }
 // Forms for a whole converged warp: elect.sync picks the issuing lane inside the asm block, so the
 // operands stay warp-uniform registers.  From a one-lane branch (if (lane == 0)) every tcgen05.mma
@@ -116,6 +76,41 @@ __device__ __forceinline__ void z_tma_w(void *dst, const CUtensorMap *map, int x
             z_smem(dst)),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z_smem(bar))
         : "memory");
+}
+// 3D tile load (K bytes, rows within a digit plane, plane index): consecutive planes in one copy
+__device__ __forceinline__ void z_tma3_w(void *dst, const CUtensorMap *map, int x, int y, int z, uint64_t *bar) {
+    asm volatile(
+        "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+        "@e cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];\n\t}\n" ::"r"(
+            z_smem(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(z_smem(bar))
+        : "memory");
+}
+// E4M3 operands: one MMA (K = 32 bytes), the 4 MMAs of a 128-byte K block (the first K step takes
+// the accumulate predicate, the others accumulate; A and B advance by 32 bytes, 2 descriptor units,
+// per step), and K steps 1..3 alone
+__device__ __forceinline__ void z_mma_w(uint32_t d, uint64_t a, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred e, p;\n\telect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
+        "l"(a), "l"(bdesc), "r"(idesc), "r"(acc));
+}
+__device__ __forceinline__ void z_mma4_w(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred e, p, q;\n\telect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 q, %4, %4;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %5, %6, %3, q;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %7, %8, %3, q;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %9, %10, %3, q;\n\t}\n" ::"r"(d),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc), "l"(a + 2), "l"(b + 2), "l"(a + 4), "l"(b + 4), "l"(a + 6), "l"(b + 6));
+}
+__device__ __forceinline__ void z_mma3_w(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc) {
+    asm volatile(
+        "{\n\t.reg .pred e, q;\n\telect.sync _|e, 0xffffffff;\n\tsetp.eq.b32 q, %3, %3;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, q;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %4, %5, %3, q;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %6, %7, %3, q;\n\t}\n" ::"r"(d),
+        "l"(a + 2), "l"(b + 2), "r"(idesc), "l"(a + 4), "l"(b + 4), "l"(a + 6), "l"(b + 6));
 }
 // The two MMAs of one 64-byte K block with FP16 operands (kind::f16; 16 elements = 32 bytes of K
 // per MMA): the first takes the accumulate predicate, the second accumulates.
@@ -158,14 +153,6 @@ __device__ __forceinline__ void z_ld16(uint32_t taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// 3D tile load (K bytes, rows within a digit plane, plane index): consecutive planes in one copy
-__device__ __forceinline__ void z_tma3(void *dst, const CUtensorMap *map, int x, int y, int z, uint64_t *bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
-            z_smem(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(z_smem(bar))
-        : "memory");
-}
 // Smallest e with amax <= 2^e (0 for amax <= 0): a tile's digit exponent.
 __device__ __forceinline__ int z_digit_exp(double amax) {
     if (!(amax > 0.0)) return 0;
