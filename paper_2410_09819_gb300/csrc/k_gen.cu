@@ -4,6 +4,8 @@
 // element).
 #include "tc_internal.h"
 
+#include <cooperative_groups.h>
+
 // Device-only unless a host test harness asks for both sides.
 #ifndef MATERN_FN
 #define MATERN_FN __device__
@@ -179,36 +181,71 @@ k_matern(double *A, int64_t n, int b, const double *__restrict__ pts, double sig
     }
 }
 
-// Sum of squares of the valid (row, column < n) elements of every tile; one CTA per tile,
-// fixed reduction order.
-// Sum of squares of tile t0 + blockIdx.x (global packed index; the tile itself at
-// A + blockIdx.x b^2), padding excluded.
-__global__ void __launch_bounds__(256) k_tile_sumsq(const double *A, int b, int64_t n, double *out, int t0) {
-    __shared__ double red[256];
-    const int t = t0 + (int)blockIdx.x;
-    int i = (int)((sqrt(8.0 * t + 1.0) - 1.0) * 0.5);
+// Sum of squares of tile t0 + blockIdx.x / 8 (global packed index; the tile itself at
+// A + (blockIdx.x / 8) b^2), padding excluded: a cluster of eight CTAs per tile, each the columns of
+// an eighth of it, whose sums meet in the cluster's first CTA in a fixed order.  Bound by the FP64
+// pipe (one multiply-add an element, 1.0 ms for a matrix of order 32768) and then by the bytes
+// (0.63 ms); one CTA per tile with 8-byte loads and a division for every element's row and column
+// took 8.8 ms (136 tiles of 2048 on 152 SMs).
+constexpr int SUMSQ_CLUSTER = 8;
+__global__ void __cluster_dims__(SUMSQ_CLUSTER, 1, 1) __launch_bounds__(256)
+k_tile_sumsq(const double *A, int b, int64_t n, double *out, int t0) {
+    __shared__ double red[8];
+    __shared__ double part;
+    const int rank = (int)blockIdx.x % SUMSQ_CLUSTER, lt = (int)blockIdx.x / SUMSQ_CLUSTER, t = t0 + lt;
+    int i = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
     while ((int64_t)i * (i + 1) / 2 > t) --i;
     while ((int64_t)(i + 1) * (i + 2) / 2 <= t) ++i;
-    const int j = t - i * (i + 1) / 2;
-    const double *T = A + (int64_t)blockIdx.x * b * b;
-    const int64_t bb = (int64_t)b * b;
-    const int nvr = (int)((n - (int64_t)i * b) < b ? (n - (int64_t)i * b) : b);
-    const int nvc = (int)((n - (int64_t)j * b) < b ? (n - (int64_t)j * b) : b);
-    double s = 0.0;
-    for (int64_t e = threadIdx.x; e < bb; e += 256) {
-        const int r = (int)(e % b), c = (int)(e / b);
-        if (r < nvr && c < nvc) {
-            const double v = T[e];
-            s = fma(v, v, s);
+    const int j = t - (int)((int64_t)i * (i + 1) / 2);
+    const double *T = A + (int64_t)lt * b * b;
+    const int nvr = (int)min((int64_t)b, n - (int64_t)i * b), nvc = (int)min((int64_t)b, n - (int64_t)j * b);
+    const int c0 = rank * (b / SUMSQ_CLUSTER), c1 = min(nvc, c0 + b / SUMSQ_CLUSTER);
+    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+    if (nvr == b && ((uintptr_t)A & 15) == 0) {          // whole columns: one run of 16-byte loads
+        const double2 *p = reinterpret_cast<const double2 *>(T + (int64_t)c0 * b);
+        const int64_t m = c1 > c0 ? (int64_t)(c1 - c0) * b / 2 : 0;
+        int64_t e = threadIdx.x;
+        for (; e + 768 < m; e += 1024) {
+            const double2 u = p[e], v = p[e + 256], w = p[e + 512], x = p[e + 768];
+            s0 = fma(u.x, u.x, s0);
+            s1 = fma(u.y, u.y, s1);
+            s2 = fma(v.x, v.x, s2);
+            s3 = fma(v.y, v.y, s3);
+            s0 = fma(w.x, w.x, s0);
+            s1 = fma(w.y, w.y, s1);
+            s2 = fma(x.x, x.x, s2);
+            s3 = fma(x.y, x.y, s3);
         }
+        for (; e < m; e += 256) {
+            const double2 u = p[e];
+            s0 = fma(u.x, u.x, s0);
+            s1 = fma(u.y, u.y, s1);
+        }
+    } else {
+        for (int c = c0; c < c1; ++c)
+            for (int r = threadIdx.x; r < nvr; r += 256) {
+                const double v = T[(int64_t)c * b + r];
+                s0 = fma(v, v, s0);
+            }
     }
-    red[threadIdx.x] = s;
+    double s = (s0 + s1) + (s2 + s3);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
+    if (threadIdx.x == 0) {
+        double v = 0.0;
+        for (int w = 0; w < 8; ++w) v += red[w];
+        part = v;
     }
-    if (threadIdx.x == 0) out[t] = red[0];
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    cl.sync();
+    if (rank == 0 && threadIdx.x == 0) {
+        double v = 0.0;
+        for (int q = 0; q < SUMSQ_CLUSTER; ++q) v += *cl.map_shared_rank(&part, q);
+        out[t] = v;
+    }
+    cl.sync();                                           // `part` stays until it has been read
 }
 
 void launch_matern(double *A, int64_t n, int b, int nt, const double *pts, double sigma2, double a,
@@ -221,10 +258,10 @@ void launch_matern(double *A, int64_t n, int b, int nt, const double *pts, doubl
 
 void launch_tile_sumsq(const double *A, int nt, int b, int64_t n, double *out, cudaStream_t s) {
     const int T = nt * (nt + 1) / 2;
-    k_tile_sumsq<<<T, 256, 0, s>>>(A, b, n, out, 0);
+    k_tile_sumsq<<<T * SUMSQ_CLUSTER, 256, 0, s>>>(A, b, n, out, 0);
 }
 void launch_tile_sumsq_range(const double *A_first, int t0, int count, int b, int64_t n, double *out, cudaStream_t s) {
-    if (count > 0) k_tile_sumsq<<<count, 256, 0, s>>>(A_first, b, n, out, t0);
+    if (count > 0) k_tile_sumsq<<<count * SUMSQ_CLUSTER, 256, 0, s>>>(A_first, b, n, out, t0);
 }
 
 }  // namespace tc
