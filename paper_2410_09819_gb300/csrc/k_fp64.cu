@@ -5,6 +5,9 @@
 // 64 x 64 register-blocked tile below keeps the pipe saturated from one CTA per SM.
 #include "tc_internal.h"
 
+#define FIXED_FN __device__ __forceinline__
+#include "fixed_exp.h"
+
 #include <cmath>
 
 namespace tc {
@@ -95,52 +98,86 @@ k_dgemm_reduce(const DRed *__restrict__ reds, int ld, const double *__restrict__
 }
 
 // ------------------------------------------------------------------------------- POTRF
-// Factor the 64 x 64 lower block at D in place (right-looking in shared memory).  A
-// non-positive pivot records the 1-based global column in *status and stops.  Each step
-// touches only the trailing triangle (threads: row r = tid % 64, columns c = j+1+tid/64 step 4)
-// and scales the column by the pivot's reciprocal: GB300 retires about 2 FP64 operations per
-// clock per SM, so every skipped multiply-add and division counts.
-__device__ __forceinline__ void potrf64_body(double *D, int ld, int col0, int *status) {
-    __shared__ double S[64][65];
-    __shared__ int fail;
-    __shared__ double rp;
-    const int tid = threadIdx.x, r = tid & 63, cg = tid >> 6;
-    for (int idx = tid; idx < 4096; idx += 256) {
-        const int rr = idx & 63, c = idx >> 6;
-        S[rr][c] = (rr >= c) ? D[(int64_t)c * ld + rr] : 0.0;
+// Factor the 64 x 64 lower block at D in place (right-looking in shared memory).  A non-positive
+// pivot records the 1-based global column in *status and stops.
+//
+// What bounds it: latency, then the FP64 pipe of one SM.  A dependent FP64 operation takes 66
+// cycles, a division 440 and a square root 690, and a warp's FP64 instruction holds its SM quarter
+// for 64 cycles whatever lanes are active.  So 128 threads (one warp a quarter); the pivot's root and
+// its reciprocal come from integer arithmetic (fixed_exp.h: the same correctly rounded values in
+// about 450 cycles together); while warps 0 and 1 form column j, warps 2 and 3 already go through
+// what is left of step j - 1, element lists in column order so that a finished column costs nothing.
+// Every element sees the same operations in the same order as in the plain loop.  A block took 94 us
+// with a square root, a division and three barriers of 256 threads in every step.
+constexpr int POTRF_THREADS = 128;
+__device__ __forceinline__ void pivot_root(double d, double &sd, double &rp) {
+    if (d > 1e-280 && d < 1e280) {
+        const fx::Num h = fx::sqrt_rn(d);
+        sd = fx::value(h);
+        rp = fx::value(fx::recip_rn(h));
+    } else {
+        sd = sqrt(d);
+        rp = 1.0 / sd;
     }
-    if (tid == 0) fail = 0;
+}
+__device__ __forceinline__ void potrf64_body(double *D, int ld, int col0, int *status) {
+    __shared__ double S[64][65];                 // S[c][r], r >= c: L_rc once column c is done
+    __shared__ double zs[2][64], ls[2][64];      // column j before and after its scaling
+    __shared__ uint16_t tab[2080];               // elements (c << 8 | r), columns from the last to the first
+    const int tid = threadIdx.x, warp = tid >> 5;
+    for (int idx = tid; idx < 4096; idx += POTRF_THREADS) {
+        const int r = idx & 63, c = idx >> 6;
+        if (r >= c) {
+            const double v = D[(int64_t)c * ld + r];
+            S[c][r] = v;
+            if (c == 0) zs[0][r] = v;
+            tab[(63 - c) * (64 - c) / 2 + r - c] = (uint16_t)(c << 8 | r);
+        }
+    }
     __syncthreads();
+    int fail = 0;
     for (int j = 0; j < 64; ++j) {
-        if (tid == 0) {
-            const double d = S[j][j];
-            if (!(d > 0.0)) {
-                fail = j + 1;
-            } else {
-                const double sd = sqrt(d);
-                S[j][j] = sd;
-                rp = 1.0 / sd;
+        // zs[j & 1]: column j; ls[j - 1 & 1]: column j - 1 of L, which columns j + 1 .. 63 have not
+        // seen yet
+        const int cur = j & 1, prv = cur ^ 1;
+        const double d = zs[cur][j];
+        if (!(d > 0.0)) {                        // every thread reads the same pivot
+            fail = j + 1;
+            break;
+        }
+        const int n = j > 0 ? (63 - j) * (64 - j) / 2 : 0;   // elements of columns j + 1 ..
+        // the root costs a warp about as much as 320 elements
+        const int h = n + 640 < 2 * n ? (n + 640) / 2 : n;
+        if (warp < 2) {
+            double sd, rp;
+            pivot_root(d, sd, rp);
+            if (tid >= j) {
+                const double l = tid == j ? sd : zs[cur][tid] * rp;
+                ls[cur][tid] = l;
+                S[j][tid] = l;
             }
         }
+        const int e1 = warp < 2 ? n : h;
+#pragma unroll 4
+        for (int e = (warp < 2 ? h : 0) + (tid & 63); e < e1; e += 64) {
+            const int c = tab[e] >> 8, r = tab[e] & 63;
+            S[c][r] = fma(-ls[prv][r], ls[prv][c], S[c][r]);
+        }
         __syncthreads();
-        if (fail) break;
-        if (tid > j && tid < 64) S[tid][j] *= rp;
-        __syncthreads();
-        const double lrj = S[r][j];
-        for (int c = j + 1 + cg; c < 64; c += 4)
-            if (r >= c) S[r][c] = fma(-lrj, S[c][j], S[r][c]);
+        if (j < 63 && tid > j && tid < 64)       // column j + 1 of step j
+            zs[prv][tid] = fma(-ls[cur][tid], ls[cur][j + 1], S[j + 1][tid]);
         __syncthreads();
     }
     if (fail) {
         if (tid == 0) atomicCAS(status, 0, col0 + fail);
         return;
     }
-    for (int idx = tid; idx < 4096; idx += 256) {
-        const int rr = idx & 63, c = idx >> 6;
-        if (rr >= c) D[(int64_t)c * ld + rr] = S[rr][c];
+    for (int idx = tid; idx < 4096; idx += POTRF_THREADS) {
+        const int r = idx & 63, c = idx >> 6;
+        if (r >= c) D[(int64_t)c * ld + r] = S[c][r];
     }
 }
-__global__ void __launch_bounds__(256) k_potrf_block(double *D, int ld, int col0, int *status) {
+__global__ void __launch_bounds__(POTRF_THREADS) k_potrf_block(double *D, int ld, int col0, int *status) {
     if (failed(status)) return;
     potrf64_body(D, ld, col0, status);
 }
@@ -161,32 +198,74 @@ __device__ __forceinline__ void strip_solve(double (*Ss)[65], double (*Ls)[65], 
     }
 }
 
-// POTRF panel: rows below the factored 64-block within the diagonal tile, 16-row strips
-// (the solve is bound by one SM's FP64 rate, so more, smaller strips finish sooner).
-constexpr int PANEL_ROWS = 16;
+// POTRF panel: rows below the factored 64-block within the diagonal tile, X L^T = C for
+// PANEL_ROWS rows a CTA, one warp a row: lane l holds columns l and l + 32, x_j travels by shuffle,
+// and no step needs a barrier.  Bound by the FP64 pipe (160 warp operations of 64 cycles a row): 8
+// rows take 10 us, against 28 us for 16 rows with two block barriers a step.
+constexpr int PANEL_ROWS = 8;
 __device__ __forceinline__ void panel_body(double *Pb, const double *L, int ld) {
-    __shared__ double Ls[64][65], Ss[PANEL_ROWS][65], rinv[64];
-    const int tid = threadIdx.x;
+    __shared__ double Ls[64][65], rinv[64];      // Ls[j][c] = l_cj, c >= j
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     for (int idx = tid; idx < 4096; idx += 256) {
-        const int r = idx & 63, c = idx >> 6;
-        Ls[r][c] = (r >= c) ? L[(int64_t)c * ld + r] : 0.0;
+        const int c = idx & 63, j = idx >> 6;
+        if (c >= j) Ls[j][c] = L[(int64_t)j * ld + c];
     }
-    for (int idx = tid; idx < PANEL_ROWS * 64; idx += 256) {
-        const int r = idx % PANEL_ROWS, c = idx / PANEL_ROWS;
-        Ss[r][c] = Pb[(int64_t)c * ld + r];
-    }
+    double z0 = Pb[(int64_t)lane * ld + warp], z1 = Pb[(int64_t)(lane + 32) * ld + warp];
     __syncthreads();
     if (tid < 64) rinv[tid] = 1.0 / Ls[tid][tid];
     __syncthreads();
-    strip_solve<PANEL_ROWS>(Ss, Ls, rinv);
-    for (int idx = tid; idx < PANEL_ROWS * 64; idx += 256) {
-        const int r = idx % PANEL_ROWS, c = idx / PANEL_ROWS;
-        Pb[(int64_t)c * ld + r] = Ss[r][c];
+#pragma unroll 8
+    for (int j = 0; j < 32; ++j) {
+        const double x = __shfl_sync(0xffffffffu, z0, j) * rinv[j];
+        if (lane > j) z0 = fma(-x, Ls[j][lane], z0);
+        z1 = fma(-x, Ls[j][lane + 32], z1);
     }
+#pragma unroll 8
+    for (int j = 0; j < 32; ++j) {
+        const double x = __shfl_sync(0xffffffffu, z1, j) * rinv[j + 32];
+        if (lane > j) z1 = fma(-x, Ls[j + 32][lane + 32], z1);
+    }
+    Pb[(int64_t)lane * ld + warp] = z0 * rinv[lane];
+    Pb[(int64_t)(lane + 32) * ld + warp] = z1 * rinv[lane + 32];
 }
 __global__ void __launch_bounds__(256) k_trsm_rows(double *P, const double *L, int ld, const int *status) {
     if (failed(status)) return;
     panel_body(P + blockIdx.x * PANEL_ROWS, L, ld);
+}
+
+// One warp solves two rows x L^T = s in place (their chains interleave), Ls[j][c] = l_cj.
+__device__ __forceinline__ void row_solve2(const double (*Ls)[65], double *s, double *t, const double *rinv) {
+    const int lane = threadIdx.x & 31;
+    double z0 = s[lane], z1 = s[lane + 32], y0 = t[lane], y1 = t[lane + 32];
+#pragma unroll 8
+    for (int j = 0; j < 32; ++j) {
+        // the two rows' pivots in one multiplication: lanes 0 .. 15 hold one, 16 .. 31 the other
+        const double zj = __shfl_sync(0xffffffffu, z0, j), yj = __shfl_sync(0xffffffffu, y0, j);
+        const double p = (lane < 16 ? zj : yj) * rinv[j];
+        const double xz = __shfl_sync(0xffffffffu, p, 0), xy = __shfl_sync(0xffffffffu, p, 16);
+        const double l0 = Ls[j][lane], l1 = Ls[j][lane + 32];
+        if (lane > j) {
+            z0 = fma(-xz, l0, z0);
+            y0 = fma(-xy, l0, y0);
+        }
+        z1 = fma(-xz, l1, z1);
+        y1 = fma(-xy, l1, y1);
+    }
+#pragma unroll 8
+    for (int j = 0; j < 32; ++j) {
+        const double zj = __shfl_sync(0xffffffffu, z1, j), yj = __shfl_sync(0xffffffffu, y1, j);
+        const double p = (lane < 16 ? zj : yj) * rinv[j + 32];
+        const double xz = __shfl_sync(0xffffffffu, p, 0), xy = __shfl_sync(0xffffffffu, p, 16);
+        const double l1 = Ls[j + 32][lane + 32];
+        if (lane > j) {
+            z1 = fma(-xz, l1, z1);
+            y1 = fma(-xy, l1, y1);
+        }
+    }
+    s[lane] = z0 * rinv[lane];
+    s[lane + 32] = z1 * rinv[lane + 32];
+    t[lane] = y0 * rinv[lane];
+    t[lane + 32] = y1 * rinv[lane + 32];
 }
 
 // Column TRSM (Algorithm 1: A_mk = A_mk L_kk^{-T}): one CTA per 64-row strip of a tile,
@@ -223,6 +302,58 @@ k_trsm_strips(const TStrip *__restrict__ strips, int ld, int b, const int *statu
             const int r = idx & 63, c = idx >> 6;
             X[(int64_t)(jb * 64 + c) * ld + r] = Ss[r][c];
         }
+        __syncthreads();
+    }
+}
+
+// The same for 16-row strips, four times as many CTAs: for a column with too few 64-row strips to
+// fill the SMs (each strip's b^2 / 2 multiply-adds a row run on one SM).  Products: a thread holds
+// one row and four columns of the 16 x 64 block; triangles as in panel_body, a warp per row.
+constexpr int SMALL_STRIP = 16;
+__global__ void __launch_bounds__(256)
+k_trsm_strips16(const TStrip *__restrict__ strips, int ld, int b, const int *status) {
+    if (failed(status) || failed(strips[blockIdx.x].status)) return;
+    __shared__ double M[64][65], rinv[64], buf[16 * SMALL_STRIP + 16 * 64];
+    double(*Xs)[SMALL_STRIP] = reinterpret_cast<double(*)[SMALL_STRIP]>(buf);          // product operands ...
+    double(*Ys)[64] = reinterpret_cast<double(*)[64]>(buf + 16 * SMALL_STRIP);
+    double(*Ss)[65] = reinterpret_cast<double(*)[65]>(buf);                            // ... then the strip
+    static_assert(SMALL_STRIP * 65 <= 16 * SMALL_STRIP + 16 * 64, "the strip fits the operands' place");
+    const TStrip st = strips[blockIdx.x];
+    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tx = tid & 15, ty = tid >> 4;
+    double *X = st.C + st.r0;
+    for (int jb = 0; jb < b / 64; ++jb) {
+        double acc[4] = {};
+        const double *Lb = st.L + (int64_t)jb * 64;
+        for (int k = 0; k < jb * 64; k += 16) {
+            Xs[ty][tx] = X[(int64_t)(k + ty) * ld + tx];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int idx = tid + 256 * e;
+                Ys[idx >> 6][idx & 63] = Lb[(int64_t)(k + (idx >> 6)) * ld + (idx & 63)];
+            }
+            __syncthreads();
+#pragma unroll
+            for (int l = 0; l < 16; ++l) {
+                const double a = Xs[l][tx];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc[q] = fma(a, Ys[l][ty + 16 * q], acc[q]);
+            }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) Ss[tx][ty + 16 * q] = X[(int64_t)(jb * 64 + ty + 16 * q) * ld + tx] - acc[q];
+        for (int idx = tid; idx < 4096; idx += 256) {
+            const int c = idx & 63, j = idx >> 6;
+            if (c >= j) M[j][c] = Lb[(int64_t)(jb * 64 + j) * ld + c];
+        }
+        __syncthreads();
+        if (tid < 64) rinv[tid] = 1.0 / M[tid][tid];
+        __syncthreads();
+        row_solve2(M, Ss[warp], Ss[warp + 8], rinv);
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) X[(int64_t)(jb * 64 + ty + 16 * q) * ld + tx] = Ss[tx][ty + 16 * q];
         __syncthreads();
     }
 }
@@ -718,7 +849,7 @@ __global__ void __launch_bounds__(1024) k_dot_self(const double *v, int64_t n, d
 
 
 // Batched POTRF step: one CTA per matrix entry (same 64-block position in each).
-__global__ void __launch_bounds__(256) k_potrf_blocks(const PEntry *__restrict__ e, int ld) {
+__global__ void __launch_bounds__(POTRF_THREADS) k_potrf_blocks(const PEntry *__restrict__ e, int ld) {
     const PEntry E = e[blockIdx.x];
     if (failed(E.status)) return;
     potrf64_body(E.D, ld, E.col0, E.status);
@@ -732,12 +863,71 @@ __global__ void __launch_bounds__(256) k_trsm_rows_batched(const PEntry *__restr
 }
 
 void launch_potrf_blocks(const PEntry *e, int n, int ld, cudaStream_t s) {
-    if (n > 0) k_potrf_blocks<<<n, 256, 0, s>>>(e, ld);
+    if (n > 0) k_potrf_blocks<<<n, POTRF_THREADS, 0, s>>>(e, ld);
 }
 void launch_trsm_rows_batched(const PEntry *e, int n, int max_rows, int ld, cudaStream_t s) {
     if (n > 0 && max_rows > 0) k_trsm_rows_batched<<<dim3(max_rows / PANEL_ROWS, n), 256, 0, s>>>(e, ld);
 }
 
+
+// POTRF trailing update: C -= P P^T with the 64 columns P below the factored block at D, on the
+// 64 x 64 blocks of the lower part (diagonal ones whole), four CTAs of 32 x 32 elements each.  The FP64
+// pipe bounds it (1.7 multiply-adds a clock and SM): one CTA a 64 x 64 block keeps its SM busy for 69
+// us, and the 15 x 16 / 2 of them below the first panel of a 1024 tile are fewer than the SMs, so
+// every step took 69 us; with quarter-size blocks the steps of that tile take half of that on average.
+constexpr int SYRK_B = 32;
+__device__ __forceinline__ void syrk_body(double *D, int ld) {
+    __shared__ double X[64][SYRK_B], Y[64][SYRK_B];
+    const int t = blockIdx.x >> 2, tid = threadIdx.x;
+    int bi = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
+    while (bi * (bi + 1) / 2 > t) --bi;
+    while ((bi + 1) * (bi + 2) / 2 <= t) ++bi;
+    const int bj = 2 * (t - bi * (bi + 1) / 2) + ((blockIdx.x >> 1) & 1);
+    bi = 2 * bi + (blockIdx.x & 1);
+    const double *P = D + 64;
+    double *C = D + (int64_t)(64 + bj * SYRK_B) * ld + 64 + bi * SYRK_B;
+    const int r = tid & 31, q = tid >> 5;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        X[q + 4 * k][r] = P[(int64_t)(q + 4 * k) * ld + bi * SYRK_B + r];
+        Y[q + 4 * k][r] = P[(int64_t)(q + 4 * k) * ld + bj * SYRK_B + r];
+    }
+    // 2 rows x 4 columns a thread
+    const int tx = tid & 15, ty = tid >> 4;
+    double acc[2][4] = {};
+    __syncthreads();
+#pragma unroll 16
+    for (int k = 0; k < 64; ++k) {
+        const double a0 = X[k][tx], a1 = X[k][tx + 16];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const double y = Y[k][ty + 8 * c];
+            acc[0][c] = fma(a0, y, acc[0][c]);
+            acc[1][c] = fma(a1, y, acc[1][c]);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        C[(int64_t)(ty + 8 * c) * ld + tx] -= acc[0][c];
+        C[(int64_t)(ty + 8 * c) * ld + tx + 16] -= acc[1][c];
+    }
+}
+__global__ void __launch_bounds__(128) k_syrk_rows_batched(const PEntry *__restrict__ e, int ld) {
+    const PEntry E = e[blockIdx.y];
+    if (!failed(E.status)) syrk_body(E.D, ld);
+}
+__global__ void __launch_bounds__(128) k_syrk_rows(double *D, int ld, const int *status) {
+    if (!failed(status)) syrk_body(D, ld);
+}
+void launch_syrk_rows_batched(const PEntry *e, int n, int rows, int ld, cudaStream_t s) {
+    const int m = rows / 64;
+    for (int i = 0; i < n && m > 0; i += 65535)
+        k_syrk_rows_batched<<<dim3(2 * m * (m + 1), n - i < 65535 ? n - i : 65535), 128, 0, s>>>(e + i, ld);
+}
+void launch_syrk_rows(double *D, int rows, int ld, const int *status, cudaStream_t s) {
+    const int m = rows / 64;
+    if (m > 0) k_syrk_rows<<<2 * m * (m + 1), 128, 0, s>>>(D, ld, status);
+}
 
 // log|A_i| = 2 sum log L_ii for every matrix of a batch (one CTA each, fixed order)
 __global__ void __launch_bounds__(256) k_logdet_batched(const LEntry *__restrict__ e, int b, double *out) {
@@ -1097,19 +1287,24 @@ void launch_dgemm_reduce(const DRed *reds, int nreds, int ld, const double *part
     if (nreds > 0) k_dgemm_reduce<<<nreds, 256, 0, s>>>(reds, ld, partials, status);
 }
 void launch_potrf_block(double *D, int ld, int col0, int *status, cudaStream_t s) {
-    k_potrf_block<<<1, 256, 0, s>>>(D, ld, col0, status);
+    k_potrf_block<<<1, POTRF_THREADS, 0, s>>>(D, ld, col0, status);
 }
 void launch_trsm_rows(double *P, const double *L, int ld, int rows, const int *status, cudaStream_t s) {
     if (rows > 0) k_trsm_rows<<<rows / PANEL_ROWS, 256, 0, s>>>(P, L, ld, status);
 }
-void launch_trsm_strips(const TStrip *strips, int nstrips, int ld, int b, const int *status, cudaStream_t s) {
+void launch_trsm_strips(const TStrip *strips, int nstrips, int rows, int ld, int b, const int *status, cudaStream_t s) {
+    if (nstrips <= 0) return;
+    if (rows == SMALL_STRIP) {
+        k_trsm_strips16<<<nstrips, 256, 0, s>>>(strips, ld, b, status);
+        return;
+    }
     const size_t smem = (32 * 64 + 2 * 64 * 65 + 64) * sizeof(double);
     static std::atomic<unsigned long long> attr{0};
     if (attrs_pending(attr)) {
         cudaFuncSetAttribute(k_trsm_strips, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         mark_attrs_set(attr);
     }
-    if (nstrips > 0) k_trsm_strips<<<nstrips, 256, smem, s>>>(strips, ld, b, status);
+    k_trsm_strips<<<nstrips, 256, smem, s>>>(strips, ld, b, status);
 }
 void launch_logdet(const double *W, int nt, int b, int64_t n, double *out, cudaStream_t s) {
     (void)nt;
@@ -1250,12 +1445,16 @@ k_trsm_tile(const __grid_constant__ TGroup g, const double *L, int ld, int b, co
     }
 }
 
-// Y = L^{-1} for a lower-triangular b x b tile L (column-major, ld = b), by forward
+// Mixed maps: Y = L^{-1} for a lower-triangular b x b tile L (column-major, ld = b), by forward
 // substitution L y_c = e_c column by column.  CTA x owns columns 4x .. 4x+3 and
 // b-4-4x .. b-1-4x: a long and a short group, so every CTA carries about the same work
 // (column c costs (b - c)^2 / 2 multiply-adds).  For each group, and each 64-row block from
 // the group's first nonzero row on, the product with the already solved rows (kept in shared
 // memory) is followed by the 64 x 64 diagonal solve.
+// The products with Y of a mixed factorization keep 10, 6 or 4 of its digit planes, so what they
+// cut off, and with it the last bit of a stored FP32, FP16 or FP8 value here and there, follows the
+// inverse's own rounding: it stays this column-by-column substitution, although the doubling of
+// k_bgemm.cu (all-FP64 maps) is several times as fast.
 constexpr int TRINV_COLS = 4;
 __device__ __forceinline__ void trinv_body(const double *__restrict__ L, int b, double *__restrict__ Y) {
     extern __shared__ double tsm[];
@@ -1297,10 +1496,7 @@ __device__ __forceinline__ void trinv_body(const double *__restrict__ L, int b, 
         }
     }
 }
-__global__ void __launch_bounds__(256) k_trinv(const double *__restrict__ L, int b, double *__restrict__ Y) {
-    trinv_body(L, b, Y);
-}
-// the same for several tiles at once (grid.y = entry): the diagonal tiles of a batch's column
+// several tiles at once (grid.y = entry): the diagonal tiles of a batch's column
 __global__ void __launch_bounds__(256) k_trinv_batched(const TEntry *__restrict__ e, int b) {
     const TEntry E = e[blockIdx.y];
     trinv_body(E.L, b, E.Y);
@@ -1417,17 +1613,7 @@ void launch_trsm_group(double *const *C, int ntiles, const double *L, int ld, in
     for (int t = 0; t < ntiles; ++t) g.C[t] = C[t];
     k_trsm_tile<<<dim3(b / 64, ntiles), 256, smem, s>>>(g, L, ld, b, status);
 }
-void launch_trinv(const double *L, int b, double *Y, cudaStream_t s) {
-    const size_t smem = ((size_t)b * TRINV_COLS + 64 * 65 + 64 * TRINV_COLS) * sizeof(double);
-    static std::atomic<unsigned long long> attr{0};
-    if (attrs_pending(attr)) {     // sized for the largest tile it serves (b <= 2048)
-        cudaFuncSetAttribute(k_trinv, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(((size_t)2048 * TRINV_COLS + 64 * 65 + 64 * TRINV_COLS) * sizeof(double)));
-        mark_attrs_set(attr);
-    }
-    k_trinv<<<b / (2 * TRINV_COLS), 256, smem, s>>>(L, b, Y);
-}
-void launch_trinv_batched(const TEntry *e, int n, int b, cudaStream_t s) {
+void launch_trinv_columns(const TEntry *e, int n, int b, cudaStream_t s) {
     if (n <= 0) return;
     const size_t smem = ((size_t)b * TRINV_COLS + 64 * 65 + 64 * TRINV_COLS) * sizeof(double);
     static std::atomic<unsigned long long> attr{0};

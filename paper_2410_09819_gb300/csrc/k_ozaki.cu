@@ -24,6 +24,7 @@
 // sums outgrow 24 bits after 128 elements of K, not a whole source tile, so TMEM is drained
 // every 128 elements; the drain is integer work (a 32-bit conversion and a 64-bit multiply-add
 // per value) and stays hidden behind the MMAs.
+#include "digits.h"
 #include "tc_internal.h"
 #include "zgemm_common.h"
 
@@ -57,57 +58,12 @@ constexpr unsigned long long ZLIMIT_NS = 4000000000ull;   // default bound of a 
 constexpr unsigned long long ZDRAIN_NS = 2000000000ull;   // bound of the teardown waits
 
 // ------------------------------------------------------------------- digit planes
-// Digits of one element in integer arithmetic (GB300 runs FP64 at 2 operations per clock per
-// SM): q = x 2^(BITS - e) rounded to the nearest integer from the bit pattern (|x| <= 2^e).
-template <int BITS>
-__device__ __forceinline__ long long fixed_point(double x, int e) {
-    const long long bits = __double_as_longlong(x);
-    int ex = (int)((bits >> 52) & 0x7FF);
-    long long m = bits & 0xFFFFFFFFFFFFFLL;
-    if (ex == 0) ex = 1;                       // subnormal (or zero): no hidden bit
-    else m |= 1LL << 52;                       // |x| = m 2^(ex - 1075)
-    const int sh = ex - (1075 - BITS) - e;     // x 2^(BITS - e) = m 2^sh, sh <= BITS - 52
-    long long q;
-    if (sh >= 0) q = m << sh;
-    else if (sh > -63) q = (m + (1LL << (-sh - 1))) >> (-sh);
-    else q = 0;
-    return bits < 0 ? -q : q;
-}
-
-// Base-256 planes in FP16 (k_zgemm) of eight adjacent columns of a row, one 16-byte store per
-// plane.  With q = x 2^(56 - e) and the bias 0x80 in the six low bytes, byte 6 - s of q + bias
-// is digit s plus 128, and what remains above them is the top digit.  A byte u under the
-// exponent byte 0x64 is the FP16 number 1024 + u, and 1024 + u - 1152 the digit, exactly: a
-// byte permute, a logic operation and a half2 subtraction make one digit of two elements.
+// Base-256 planes of eight adjacent columns of a row (k_zgemm), one 16-byte store per plane.
 __device__ __forceinline__ void put_planes8(const long long (&q)[8], __half *P, int64_t o, int64_t bb) {
     uint32_t lo[8], hi[8];
+    biased8(q, lo, hi);
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-        const unsigned long long n = (unsigned long long)q[u] + 0x0000808080808080ull;
-        lo[u] = (uint32_t)n;
-        hi[u] = (uint32_t)(n >> 32);
-    }
-#pragma unroll
-    for (int s = 0; s < ZS; ++s) {
-        // 1024 + 128, and 1024 + 256 for the top digit
-        const __half2 off = __half2half2(__ushort_as_half((unsigned short)(s == 0 ? 0x6500 : 0x6480)));
-        uint32_t w[4];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            uint32_t h;
-            if (s == 0) {                       // top digit in [-256, 256]: 256 + digit in 10 bits
-                h = __byte_perm(hi[2 * v] + 0x01000000u, hi[2 * v + 1] + 0x01000000u, 0x7632u) | 0x64006400u;
-            } else {
-                const int byte = 6 - s;
-                const uint32_t a = byte < 4 ? lo[2 * v] : hi[2 * v], c = byte < 4 ? lo[2 * v + 1] : hi[2 * v + 1];
-                const uint32_t sel = (uint32_t)(byte & 3) | ((uint32_t)(4 + (byte & 3)) << 8);
-                h = (__byte_perm(a, c, sel) & 0x00FF00FFu) | 0x64006400u;
-            }
-            const __half2 d = __hsub2(*reinterpret_cast<const __half2 *>(&h), off);
-            w[v] = *reinterpret_cast<const uint32_t *>(&d);
-        }
-        *reinterpret_cast<uint4 *>(P + (int64_t)s * bb + o) = make_uint4(w[0], w[1], w[2], w[3]);
-    }
+    for (int s = 0; s < ZS; ++s) *reinterpret_cast<uint4 *>(P + (int64_t)s * bb + o) = digit8(lo, hi, s);
 }
 
 // Base-16 planes in E4M3 (k_zgemm64): q = x 2^(56 - e) (|q| <= 2^56), then balanced digits from
@@ -168,7 +124,7 @@ __device__ __forceinline__ void planes_of_tile(const double *T, int b, bool tran
             const int c = ((threadIdx.x >> 2) & 7) * 8, r = (threadIdx.x & 3) + 4 * (threadIdx.x >> 5);
             long long q[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) q[u] = fixed_point<56>(S[c + u][r], e);
+            for (int u = 0; u < 8; ++u) q[u] = fixed56(S[c + u][r], e);
             put_planes8(q, reinterpret_cast<__half *>(P), (int64_t)(r0 + r) * b + c0 + c, bb);
         } else {
 #pragma unroll
@@ -176,7 +132,7 @@ __device__ __forceinline__ void planes_of_tile(const double *T, int b, bool tran
                 const int c = (threadIdx.x & 7) * 4 + 32 * h, r = threadIdx.x >> 3;
                 long long q[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) q[u] = fixed_point<56>(S[c + u][r], e);
+                for (int u = 0; u < 4; ++u) q[u] = fixed56(S[c + u][r], e);
                 put_digits4(q, P, (int64_t)(r0 + r) * b + c0 + c, bb);
             }
         }

@@ -29,7 +29,6 @@ namespace {
 // so each launch below serves the whole batch.
 struct PotrfStep {
     int pe0 = 0, npe = 0;        // PEntry range (one per matrix)
-    int it0 = 0, nit = 0;        // trailing-update items
     int rows = 0;                // panel rows below the 64-block
 };
 
@@ -42,7 +41,7 @@ struct ColPlan {
     int dg0 = 0, ndg = 0;        // tiles whose digit planes are made after the column's TRSMs
     int it0 = 0, nit = 0;        // FP64 update items
     int red0 = 0, nred = 0;      // split-K reductions
-    int st0 = 0, nst = 0;        // TRSM strips
+    int st0 = 0, nst = 0, srows = 64;   // TRSM strips and their rows
     std::vector<PotrfStep> potrf;
 };
 
@@ -285,31 +284,22 @@ Plan build_plan(tc_handle h, double *W, int *status) {
                 P.pentries.push_back({D + (int64_t)jb * 64 * b + jb * 64, status + 2 + mi, k * b + jb * 64, ps.rows});
             }
             ps.npe = (int)P.pentries.size() - ps.pe0;
-            ps.it0 = (int)P.items.size();
-            if (ps.rows > 0)
-                for (int mi = 0; mi < nmat; ++mi) {
-                    const MatDesc &M = h->mats[mi];
-                    if (M.nt <= k) continue;
-                    double *D = T(M, k, k);
-                    const double *Pn = D + (int64_t)jb * 64 * b + (jb + 1) * 64;
-                    const int job = (int)P.jobs.size();
-                    P.jobs.push_back({D + (int64_t)(jb + 1) * 64 * b + (jb + 1) * 64, Pn, Pn, 64, ps.rows, ps.rows, 1,
-                                      status + 2 + mi});
-                    int dummy = 0;
-                    emit_job_items(P, job, b, 1, dummy);
-                }
-            ps.nit = (int)P.items.size() - ps.it0;
             C.potrf.push_back(ps);
         }
         // 3. TRSM strips of the tiles below the diagonal
         C.st0 = (int)P.strips.size();
+        // 64-row strips where they give every SM two, else 16-row ones (a strip runs on one SM: at
+        // n = 2048, tile 256, the first column's 28 strips of 64 rows take 610 us each)
+        int64_t strips64 = 0;
+        for (int mi = 0; mi < nmat; ++mi) strips64 += (int64_t)std::max(0, h->mats[mi].nt - k - 1) * (b / 64);
+        C.srows = strips64 >= 2 * NSM ? 64 : 16;
         for (int mi = 0; mi < nmat; ++mi) {
             const MatDesc &M = h->mats[mi];
             if (M.nt <= k) continue;
             P.potrf_flops += (double)b * b * b / 3.0;
             for (int m = k + 1; m < M.nt; ++m) {
                 if (!P.inv_trsm)
-                    for (int r0 = 0; r0 < b; r0 += 64) P.strips.push_back({T(M, m, k), T(M, k, k), status + 2 + mi, r0});
+                    for (int r0 = 0; r0 < b; r0 += C.srows) P.strips.push_back({T(M, m, k), T(M, k, k), status + 2 + mi, r0});
                 P.trsm_flops += (double)b * b * b;
             }
         }
@@ -714,7 +704,7 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
             if (ps.rows > 0) {
                 launch_trsm_rows_batched(D.pentries + ps.pe0, ps.npe, ps.rows, b, h->s);
                 CK_LAUNCH();
-                launch_dgemm_update(D.jobs, D.items + ps.it0, ps.nit, b, parts, nullptr, h->s);
+                launch_syrk_rows_batched(D.pentries + ps.pe0, ps.npe, ps.rows, b, h->s);
                 CK_LAUNCH();
             }
         }
@@ -727,16 +717,17 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
             const MatDesc &Md = h->mats[0];
             double *inv = static_cast<double *>(h->invbuf.p);
             uint8_t *pool = static_cast<uint8_t *>(h->dpool.p);
-            if (b <= 2048) {
-                // inverse e of the column at inv + e b^2 (one per matrix), then its amax and
-                // digit planes into the diagonal tile's slot
-                launch_trinv_batched(D.tinv + C.ti0, C.nti, b, h->s);
+            // inverse e of the column at inv + e b^2 (one per matrix), then its amax and digit planes
+            // into the diagonal tile's slot
+            if (P.inv_refine || b <= 2048) {
+                if (P.inv_refine) launch_trinv_batched(D.tinv + C.ti0, C.nti, b, h->s);
+                else launch_trinv_columns(D.tinv + C.ti0, C.nti, b, h->s);
                 CK_LAUNCH();
                 launch_tile_amax(W, b, D.dinv + C.ti0, C.nti, D.zamax2, h->s, inv);
                 CK_LAUNCH();
                 launch_digits(W, b, D.dinv + C.ti0, C.nti, D.zamax2, pool, D.zexps, h->s, e4m3, inv);
                 CK_LAUNCH();
-            } else {                       // one matrix: its shared-memory column panel would not fit
+            } else {                       // mixed, one matrix: the columns' shared-memory panel would not fit
                 const int gkk = (int)(Md.tile0 + tidx(k, k));
                 const double *Lkk0 = W + (Md.tile0 + tidx(k, k)) * bb;
                 launch_set_identity(inv, b, h->s);
@@ -799,7 +790,7 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
         }
         if (C.nst) {
             const int sp = spans ? span_begin(h, CAT_TRSM) : -1;
-            launch_trsm_strips(D.strips + C.st0, C.nst, b, b, nullptr, h->s);
+            launch_trsm_strips(D.strips + C.st0, C.nst, C.srows, b, b, nullptr, h->s);
             span_end(h, sp);
             CK_LAUNCH();
         }

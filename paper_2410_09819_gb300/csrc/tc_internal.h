@@ -72,7 +72,6 @@ struct TEntry {         // triangular inverse of one diagonal tile: Y = L^{-1} (
     const double *L;
     double *Y;
 };
-void launch_trinv_batched(const TEntry *e, int n, int b, cudaStream_t s);
 struct SRes {           // residual / |A| x of one 64-row chunk of one matrix
     const double *A;    // the matrix's tiles
     int64_t n;
@@ -115,12 +114,21 @@ void launch_potrf_block(double *D, int ld, int col0, int *status, cudaStream_t s
 void launch_trsm_rows(double *P, const double *L, int ld, int rows, const int *status, cudaStream_t s);
 void launch_potrf_blocks(const PEntry *e, int n, int ld, cudaStream_t s);
 void launch_trsm_rows_batched(const PEntry *e, int n, int max_rows, int ld, cudaStream_t s);
-void launch_trsm_strips(const TStrip *strips, int nstrips, int ld, int b, const int *status, cudaStream_t s);
+// the POTRF step's trailing update: the lower part of the rows below the panel, C -= P P^T
+void launch_syrk_rows_batched(const PEntry *e, int n, int rows, int ld, cudaStream_t s);
+void launch_syrk_rows(double *D, int rows, int ld, const int *status, cudaStream_t s);
+// TRSM strips of `rows` rows each (64 or 16)
+void launch_trsm_strips(const TStrip *strips, int nstrips, int rows, int ld, int b, const int *status, cudaStream_t s);
 void launch_logdet(const double *W, int nt, int b, int64_t n, double *out, cudaStream_t s);
 void launch_fix_padding(double *W, int nt, int b, int64_t n, cudaStream_t s);
 void launch_zero_upper_diag(double *W, int nt, int b, int64_t n, cudaStream_t s);
 void launch_logdet_batched(const LEntry *e, int count, int b, double *out, cudaStream_t s);
 void launch_fix_padding_batched(const LEntry *e, int count, int ntmax, int b, cudaStream_t s);
+
+// ------------------------------------------------------------------ launchers (k_bgemm.cu)
+// Y = L^{-1} of lower-triangular b x b tiles (column-major; Y's upper part zero)
+void launch_trinv_batched(const TEntry *e, int n, int b, cudaStream_t s);
+void launch_trinv(const double *L, int b, double *Y, cudaStream_t s);
 
 // tile-pointer variants (out-of-core executor)
 void launch_dgemm_tile(const DJob &job, int ld, cudaStream_t s);
@@ -142,7 +150,8 @@ inline bool attrs_pending(const std::atomic<unsigned long long> &mask) {
 inline void mark_attrs_set(std::atomic<unsigned long long> &mask) {
     mask.fetch_or(device_bit(), std::memory_order_release);
 }
-void launch_trinv(const double *L, int b, double *Y, cudaStream_t s);   // Y = L^{-1}, b x b
+// the same inverses column by column (mixed maps; b <= 2048)
+void launch_trinv_columns(const TEntry *e, int n, int b, cudaStream_t s);
 void launch_trsm_group(double *const *C, int ntiles, const double *L, int ld, int b, const int *status,
                        cudaStream_t s);
 void launch_logdiag_tile(const double *D, int b, int nv, double *out, cudaStream_t s);

@@ -668,9 +668,7 @@ extern "C" int tile_chol_factor_ooc(tc_handle h, int64_t n, int b, double *A_til
                         launch_trsm_rows(D + (int64_t)jb * 64 * b + (jb + 1) * 64, D + (int64_t)jb * 64 * b + jb * 64,
                                          b, rows, status, h->s);
                         CK_LAUNCH();
-                        const double *Pn = D + (int64_t)jb * 64 * b + (jb + 1) * 64;
-                        launch_dgemm_tile({D + (int64_t)(jb + 1) * 64 * b + (jb + 1) * 64, Pn, Pn, 64, rows, rows, 1, nullptr},
-                                          b, h->s);
+                        launch_syrk_rows(D + (int64_t)jb * 64 * b + jb * 64, rows, b, status, h->s);
                         CK_LAUNCH();
                     }
                 }
@@ -681,14 +679,8 @@ extern "C" int tile_chol_factor_ooc(tc_handle h, int64_t n, int b, double *A_til
                 if (inv_trsm && k + 1 < nt) {
                     const int spi = span_begin(h, CAT_TRSM);
                     launch_lower_only(D, b, h->s);
-                    if (b <= 2048) {
-                        launch_trinv(D, b, inv, h->s);
-                        C.planes_of(inv, vslot, 0);
-                    } else {
-                        launch_set_identity(inv, b, h->s);
-                        launch_trsm_tile(inv, D, b, b, nullptr, h->s);   // L_kk^{-T}
-                        C.planes_of(inv, vslot, 1);
-                    }
+                    launch_trinv(D, b, inv, h->s);
+                    C.planes_of(inv, vslot);
                     C.planes_of(D, diag_slot, 0);    // L_kk (a diagonal tile is never an update operand)
                     C.dig[diag_slot] = 0;
                     C.has_amax[diag_slot] = 0;
