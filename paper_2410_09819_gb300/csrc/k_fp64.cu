@@ -586,73 +586,9 @@ __global__ void __launch_bounds__(256) k_fwd_diag(const double *L, int ld, int b
     fwd_diag_body(L, ld, b, R + blockIdx.x * ldr);
 }
 
-// r_i -= L_ij z_j for every tile row i > j; one CTA per 64-row chunk of a tile row.
-template <int NQ>
-__global__ void __launch_bounds__(256)
-k_fwd_update(const double *W, int b, int j, double *R, int64_t ldr, int nrhs) {
-    __shared__ double zs[128][16];
-    __shared__ double red[64][17];
-    const int chunks = b / 64;
-    const int i = j + 1 + blockIdx.x / chunks, r0 = (blockIdx.x % chunks) * 64;
-    const double *L = W + ((int64_t)i * (i + 1) / 2 + j) * (int64_t)b * b;
-    const int tid = threadIdx.x, rr = tid & 63, part = tid >> 6;
-    double acc[NQ];
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) acc[q] = 0.0;
-    for (int c0 = 0; c0 < b; c0 += 128) {
-        __syncthreads();
-        for (int e = tid; e < 128 * nrhs; e += 256) {
-            const int c = e % 128, q = e / 128;
-            zs[c][q] = R[q * ldr + (int64_t)j * b + c0 + c];
-        }
-        __syncthreads();
-        for (int c = part; c < 128; c += 4) {
-            const double l = L[(int64_t)(c0 + c) * b + r0 + rr];
-#pragma unroll
-            for (int q = 0; q < NQ; ++q)
-                if (q < nrhs) acc[q] = fma(l, zs[c][q], acc[q]);
-        }
-    }
-    part_reduce_sub(red, acc, nrhs, R, ldr, (int64_t)i * b + r0);
-}
-
 // Back substitution with the s x s lower triangle at L: L^T x = z for each RHS column.
 __global__ void __launch_bounds__(256) k_bwd_diag(const double *L, int ld, int b, double *R, int64_t ldr) {
     bwd_diag_body(L, ld, b, R + blockIdx.x * ldr);
-}
-
-// z_i -= L_ji^T x_j for every tile row i < j; one CTA per 64-row chunk of tile row i.
-template <int NQ>
-__global__ void __launch_bounds__(256)
-k_bwd_update(const double *W, int b, int j, double *R, int64_t ldr, int nrhs) {
-    __shared__ double xs[64][16];
-    __shared__ double S[64][65];
-    const int chunks = b / 64;
-    const int i = blockIdx.x / chunks, r0 = (blockIdx.x % chunks) * 64;
-    const double *L = W + ((int64_t)j * (j + 1) / 2 + i) * (int64_t)b * b;   // tile (j, i)
-    const int tid = threadIdx.x, rr = tid & 63, part = tid >> 6;
-    double acc[NQ];
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) acc[q] = 0.0;
-    for (int c0 = 0; c0 < b; c0 += 64) {
-        __syncthreads();
-        for (int idx = tid; idx < 4096; idx += 256) {
-            const int c = idx & 63, r = idx >> 6;
-            S[r][c] = L[(int64_t)(r0 + r) * b + c0 + c];      // (L_ji^T)[r][c] = L_ji[c][r]
-        }
-        for (int e = tid; e < 64 * nrhs; e += 256) {
-            const int c = e % 64, q = e / 64;
-            xs[c][q] = R[q * ldr + (int64_t)j * b + c0 + c];
-        }
-        __syncthreads();
-        for (int c = part; c < 64; c += 4) {
-            const double l = S[rr][c];
-#pragma unroll
-            for (int q = 0; q < NQ; ++q)
-                if (q < nrhs) acc[q] = fma(l, xs[c][q], acc[q]);
-        }
-    }
-    part_reduce_sub(reinterpret_cast<double(*)[17]>(&S[0][0]), acc, nrhs, R, ldr, (int64_t)i * b + r0);
 }
 
 // R = B - A X (absmode 0) or R = |A| X (absmode 1, B unused) for the symmetric A held as
@@ -1331,10 +1267,6 @@ void launch_fwd_diag(const double *Ljj, int b, double *R, int64_t ldr, int nrhs,
                         R + sb * S, R + (sb + 1) * S, ldr, nrhs);
     }
 }
-void launch_fwd_update(const double *W, int nt, int b, int j, double *R, int64_t ldr, int nrhs, cudaStream_t s) {
-    const int ntiles = nt - 1 - j;
-    if (ntiles > 0) NQ_DISPATCH(nrhs, k_fwd_update, ntiles * (b / 64), 256, 0, s, W, b, j, R, ldr, nrhs);
-}
 void launch_bwd_diag(const double *Ljj, int b, double *R, int64_t ldr, int nrhs, cudaStream_t s) {
     const int S = (b % DIAG_SUB) ? b : DIAG_SUB;     // tiles not a multiple of it: one block
     for (int sb = b / S - 1; sb >= 0; --sb) {
@@ -1342,10 +1274,6 @@ void launch_bwd_diag(const double *Ljj, int b, double *R, int64_t ldr, int nrhs,
         if (sb > 0)
             NQ_DISPATCH(nrhs, k_gemv_above, sb * S / 64, 256, 0, s, Ljj + sb * S, b, S, R + sb * S, R, ldr, nrhs);
     }
-}
-void launch_bwd_update(const double *W, int nt, int b, int j, double *R, int64_t ldr, int nrhs, cudaStream_t s) {
-    (void)nt;
-    if (j > 0) NQ_DISPATCH(nrhs, k_bwd_update, j * (b / 64), 256, 0, s, W, b, j, R, ldr, nrhs);
 }
 void launch_symv_resid(const double *A, int nt, int b, int64_t n, const double *X, int64_t ldx,
                        const double *B, int64_t ldb, double *R, int64_t ldr, int nrhs, int absmode,

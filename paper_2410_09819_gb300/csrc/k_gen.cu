@@ -41,29 +41,79 @@ MATERN_FN inline void temme_gammas(double mu, double &g1, double &g2) {
          m2 * -3.6968056186422057e-12)))))))));
 }
 
+// Per-call constants of the Matern correlation for smoothness nu: m = floor(nu + 1/2),
+// mu = nu - m, Temme's g1, g2 and pre = 2^(1-nu) / Gamma(nu), with
+// Gamma(nu) = Gamma(1+mu) (mu+1) ... (mu+m-1), or Gamma(1+mu)/mu when m = 0; and what the two
+// evaluations below would otherwise divide by for every element (an FP64 division is 7 FP64
+// operations): made once, on the host.
+struct MaternNu {
+    static constexpr int KS = 24, KR = 82;      // terms of the series, of the normalising sum
+    double nu, mu, g1, g2, pre;
+    double fac, ip, iq;                         // mu pi / sin(mu pi), Gamma(1+mu) / 2, Gamma(1-mu) / 2
+    double r2[KS], rm[KS], rp[KS], rf[KS];      // 1/(k^2 - mu^2), prod 1/(j - mu), prod 1/(j + mu), 1/k!
+    double a[KR], c[KR];                        // a_k = (k+1/2)^2 - mu^2, C_k = C_{k-1} a_{k-1} / k
+    int m;
+};
+
+MATERN_FN inline MaternNu matern_nu(double nu) {
+    MaternNu c;
+    c.nu = nu;
+    c.m = (int)floor(nu + 0.5);
+    c.mu = nu - c.m;
+    temme_gammas(c.mu, c.g1, c.g2);
+    c.ip = 0.5 / (c.g2 - c.mu * c.g1);          // 1/Gamma(1+mu) = g2 - mu g1
+    c.iq = 0.5 / (c.g2 + c.mu * c.g1);          // 1/Gamma(1-mu) = g2 + mu g1
+    double gam = 2.0 * c.ip;
+    if (c.m == 0) gam /= c.mu;
+    for (int j = 1; j < c.m; ++j) gam *= c.mu + j;
+    c.pre = exp2(1.0 - nu) / gam;
+    c.fac = (c.mu == 0.0) ? 1.0 : (3.141592653589793 * c.mu) / sin(3.141592653589793 * c.mu);
+    const double m2 = c.mu * c.mu;
+    c.r2[0] = 0.0;
+    c.rm[0] = c.rp[0] = c.rf[0] = 1.0;
+    for (int k = 1; k < MaternNu::KS; ++k) {
+        c.r2[k] = 1.0 / ((double)k * k - m2);
+        c.rm[k] = c.rm[k - 1] / (k - c.mu);
+        c.rp[k] = c.rp[k - 1] / (k + c.mu);
+        c.rf[k] = c.rf[k - 1] / k;
+    }
+    c.c[0] = 1.0;
+    for (int k = 0; k < MaternNu::KR; ++k) {
+        c.a[k] = (k + 0.5) * (k + 0.5) - m2;
+        if (k > 0) c.c[k] = c.c[k - 1] * (c.a[k - 1] / k);
+    }
+    return c;
+}
+
+// sinh(s) / s from e = exp(s) and 1/e, the Taylor series where the difference would cancel
+MATERN_FN inline double sinh_ratio(double s, double e, double ei) {
+    if (fabs(s) > 0.5) return 0.5 * (e - ei) / s;
+    const double t = s * s;
+    return 1.0 + t * (1.0 / 6.0) * (1.0 + t * (1.0 / 20.0) * (1.0 + t * (1.0 / 42.0) * (1.0 + t * (1.0 / 72.0) *
+               (1.0 + t * (1.0 / 110.0) * (1.0 + t * (1.0 / 156.0) * (1.0 + t * (1.0 / 210.0)))))));
+}
+
 // K_mu(x), K_{mu+1}(x) for |mu| <= 1/2, 0 < x <= 2.  With c_k = (x^2/4)^k / k!:
 //   K_mu = sum c_k f_k,  K_{mu+1} = (2/x) sum c_k (p_k - k f_k),
 //   f_k = (k f_{k-1} + p_{k-1} + q_{k-1}) / (k^2 - mu^2),  p_k = p_{k-1}/(k-mu),  q_k = q_{k-1}/(k+mu),
 //   p_0 = (x/2)^-mu Gamma(1+mu) / 2,  q_0 = (x/2)^mu Gamma(1-mu) / 2,
 //   f_0 = (mu pi / sin(mu pi)) (cosh(s) g1 + sinh(s)/s ln(2/x) g2),  s = mu ln(2/x).
 // The terms fall at least like 1/(k!)^2; at x = 2 fifteen reach the double rounding unit.
-MATERN_FN inline void bessel_k_series(double mu, double x, double g1, double g2, double &k0, double &k1) {
-    const double lg = log(2.0 / x);
-    const double s = mu * lg;
-    const double fac = (mu == 0.0) ? 1.0 : (3.141592653589793 * mu) / sin(3.141592653589793 * mu);
-    const double shs = (s == 0.0) ? 1.0 : sinh(s) / s;
-    double f = fac * (cosh(s) * g1 + shs * lg * g2);
-    const double e = exp(s);
-    double p = 0.5 * e / (g2 - mu * g1);       // 1/Gamma(1+mu) = g2 - mu g1
-    double q = 0.5 / (e * (g2 + mu * g1));     // 1/Gamma(1-mu) = g2 + mu g1
+MATERN_FN inline void bessel_k_series(const MaternNu &n, double x, double &k0, double &k1) {
+    const double lg = -log(0.5 * x);
+    const double s = n.mu * lg;
+    const double e = exp(s), ei = 1.0 / e;
+    double f = n.fac * (0.5 * (e + ei) * n.g1 + sinh_ratio(s, e, ei) * lg * n.g2);
+    const double p0 = e * n.ip, q0 = ei * n.iq;
     const double y = 0.25 * x * x;
-    double c = 1.0, s0 = f, s1 = p;
-    for (int k = 1; k <= 60; ++k) {
+    double p = p0, q = q0, yk = 1.0, s0 = f, s1 = p;
+    for (int k = 1; k < MaternNu::KS; ++k) {
         const double dk = (double)k;
-        f = (dk * f + p + q) / (dk * dk - mu * mu);
-        p /= dk - mu;
-        q /= dk + mu;
-        c *= y / dk;
+        f = (dk * f + p + q) * n.r2[k];
+        p = p0 * n.rm[k];
+        q = q0 * n.rp[k];
+        yk *= y;
+        const double c = yk * n.rf[k];
         const double t0 = c * f, t1 = c * (p - dk * f);
         s0 += t0;
         s1 += t1;
@@ -74,46 +124,25 @@ MATERN_FN inline void bessel_k_series(double mu, double x, double g1, double g2,
 }
 
 // e^x K_mu(x), e^x K_{mu+1}(x) for |mu| <= 1/2, x > 2.  U_k satisfies
-//   U_{k-1} - 2(k+x) U_k + a_k U_{k+1} = 0,  a_k = (k+1/2)^2 - mu^2,
-// so r_k = U_k / U_{k-1} = 1 / (2(k+x) - a_k r_{k+1}), started at r_{K+1} = 0.  The sum
-// S = sum C_k U_k / U_0 with C_k / C_{k-1} = a_{k-1} / k is nested alongside,
-//   T_{k-1} = 1 + (a_{k-1}/k) r_k T_k,  S = T_0,
-// and then e^x K_mu = sqrt(pi / 2x) / S,  K_{mu+1} / K_mu = (mu + 1/2 + x + (mu^2 - 1/4) r_1) / x.
+//   U_{k-1} = 2(k+x) U_k - a_k U_{k+1},  a_k = (k+1/2)^2 - mu^2,
+// taken backward from U_{K+1} = 0, U_K = 1 (at most 2^82 83! / 2, far from overflow), with the sum
+// S = sum C_k U_k alongside, C_k / C_{k-1} = a_{k-1} / k; and then
+// e^x K_mu = sqrt(pi / 2x) / (S / U_0),  K_{mu+1} / K_mu = (mu + 1/2 + x + (mu^2 - 1/4) U_1 / U_0) / x.
 // K = 6 + 150/x terms keep the truncation below the rounding unit for every x > 2.
-MATERN_FN inline void bessel_k_ratio(double mu, double x, double &k0, double &k1) {
+MATERN_FN inline void bessel_k_ratio(const MaternNu &n, double x, double &k0, double &k1) {
     const int K = 6 + (int)ceil(150.0 / x);
-    const double m2 = mu * mu;
-    double r = 0.0, T = 1.0;
+    double u1 = 0.0, u0 = 1.0, S = 0.0;                  // U_{k+1}, U_k
+    double bk = 2.0 * (K + x);
     for (int k = K; k >= 1; --k) {
-        const double dk = (double)k;
-        const double ak = (dk + 0.5) * (dk + 0.5) - m2;
-        const double am = (dk - 0.5) * (dk - 0.5) - m2;
-        r = 1.0 / (2.0 * (dk + x) - ak * r);
-        T = 1.0 + (am / dk) * r * T;
+        S += n.c[k] * u0;
+        const double u = bk * u0 - n.a[k] * u1;
+        u1 = u0;
+        u0 = u;
+        bk -= 2.0;
     }
-    k0 = sqrt(3.141592653589793 / (2.0 * x)) / T;
-    k1 = k0 * (mu + 0.5 + x + (m2 - 0.25) * r) / x;
-}
-
-// Per-call constants of the Matern correlation for smoothness nu: m = floor(nu + 1/2),
-// mu = nu - m, Temme's g1, g2 and pre = 2^(1-nu) / Gamma(nu), with
-// Gamma(nu) = Gamma(1+mu) (mu+1) ... (mu+m-1), or Gamma(1+mu)/mu when m = 0.
-struct MaternNu {
-    double nu, mu, g1, g2, pre;
-    int m;
-};
-
-MATERN_FN inline MaternNu matern_nu(double nu) {
-    MaternNu c;
-    c.nu = nu;
-    c.m = (int)floor(nu + 0.5);
-    c.mu = nu - c.m;
-    temme_gammas(c.mu, c.g1, c.g2);
-    double gam = 1.0 / (c.g2 - c.mu * c.g1);
-    if (c.m == 0) gam /= c.mu;
-    for (int j = 1; j < c.m; ++j) gam *= c.mu + j;
-    c.pre = exp2(1.0 - nu) / gam;
-    return c;
+    S += u0;                                             // C_0 = 1
+    k0 = sqrt(3.141592653589793 / (2.0 * x)) / (S / u0);
+    k1 = k0 * (n.mu + 0.5 + x + (n.mu * n.mu - 0.25) * (u1 / u0)) / x;
 }
 
 // 2^(1-nu)/Gamma(nu) x^nu K_nu(x), the Matern correlation of Eq. 2 at x = h/a >= 0 (1 at 0).
@@ -126,8 +155,8 @@ MATERN_FN inline double matern_corr(const MaternNu &c, double x) {
     const bool small = x <= 2.0;
     if (small && c.nu * log(2.0 / x) > 600.0) return 1.0;
     double k0, k1;
-    if (small) bessel_k_series(c.mu, x, c.g1, c.g2, k0, k1);
-    else bessel_k_ratio(c.mu, x, k0, k1);
+    if (small) bessel_k_series(c, x, k0, k1);
+    else bessel_k_ratio(c, x, k0, k1);
     double kn = k0;
     if (c.m > 0) {
         for (int j = 1; j < c.m; ++j) {
@@ -169,8 +198,14 @@ __device__ __forceinline__ double scaled_distance(double dx, double dy, const Ra
 template <int NU2>
 __global__ void __launch_bounds__(256)
 k_matern(double *A, int64_t n, int b, const double *__restrict__ pts, double sigma2, const __grid_constant__ Range g,
-         const __grid_constant__ MaternNu cn, double nugget) {
-    __shared__ uint64_t table[fx::EXP_TABLE];
+         const __grid_constant__ MaternNu general, double nugget) {
+    __shared__ uint64_t table[NU2 ? fx::EXP_TABLE : 1];
+    __shared__ __align__(16) unsigned char cbuf[NU2 ? 1 : sizeof(MaternNu)];    // lanes read its tables at their own k
+    const MaternNu &cn = *reinterpret_cast<const MaternNu *>(cbuf);
+    if (NU2 == 0) {
+        for (int i = threadIdx.x; i < (int)(sizeof(MaternNu) / 4); i += 256)
+            reinterpret_cast<uint32_t *>(cbuf)[i] = reinterpret_cast<const uint32_t *>(&general)[i];
+    }
     if (NU2)
         for (int i = threadIdx.x; i < fx::EXP_TABLE; i += 256) table[i] = fx::exp_entry(i);
     const int t = blockIdx.y;

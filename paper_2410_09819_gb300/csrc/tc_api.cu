@@ -1004,7 +1004,7 @@ void tc_destroy(tc_handle h) {
     if (h->s) cudaStreamSynchronize(h->s);
     for (DevBuf *d : {&h->W, &h->Acopy, &h->status, &h->scratch, &h->tables, &h->partials, &h->vec, &h->sumsq,
                       &h->pool_hi, &h->pool_lo, &h->pool16, &h->pool8, &h->mxtab, &h->logdiag, &h->dpool, &h->ztab,
-                      &h->invbuf, &h->stab})
+                      &h->invbuf, &h->stab, &h->sweep})
         release(*d);
     if (h->graph) cudaGraphExecDestroy(h->graph);
     release(h->bstage);
@@ -1224,34 +1224,33 @@ int tile_chol_logdet(tc_handle h, double *logdet_out) {
     return TC_OK;
 }
 
-// Forward (and optionally back) substitution with the factor tiles at W (nt tile rows) on
-// the padded column-major buffer R (leading dimension ldr = nt*b), nrhs <= 16 per pass.
-static int subst_w(tc_handle h, const double *W, int nt, double *R, int64_t ldr, int nrhs, bool back) {
-    const int b = h->b;
-    const int64_t bb = (int64_t)b * b;
-    for (int c0 = 0; c0 < nrhs; c0 += 16) {
-        const int nc = std::min(16, nrhs - c0);
-        double *Rc = R + (int64_t)c0 * ldr;
-        for (int j = 0; j < nt; ++j) {
-            launch_fwd_diag(W + tidx(j, j) * bb, b, Rc + (int64_t)j * b, ldr, nc, h->s);
-            CK_LAUNCH();
-            launch_fwd_update(W, nt, b, j, Rc, ldr, nc, h->s);
-            if (j + 1 < nt) CK_LAUNCH();
-        }
-        if (!back) continue;
-        for (int j = nt - 1; j >= 0; --j) {
-            launch_bwd_diag(W + tidx(j, j) * bb, b, Rc + (int64_t)j * b, ldr, nc, h->s);
-            CK_LAUNCH();
-            launch_bwd_update(W, nt, b, j, Rc, ldr, nc, h->s);
-            if (j > 0) CK_LAUNCH();
-        }
+// Forward (and optionally back) substitution on the padded column-major buffer R (leading dimension
+// ldr = nt*b): in core one sweep per direction (k_sweep.cu), out of core tile by tile.
+static int subst(tc_handle h, double *R, int64_t ldr, int nrhs, bool back) {
+    if (h->ooc) return ooc_subst(h, R, ldr, nrhs, back, nullptr);
+    int *w = static_cast<int *>(h->sweep.p);
+    for (int f = 0; f < (back ? 2 : 1); ++f) {
+        const int e = launch_sweep(static_cast<const double *>(h->W.p), h->b, (int)(ldr / 64), R, ldr, nrhs, f == 0, w + 1, w, h->s,
+                                   wait_limit_ns(h));
+        if (e != cudaSuccess) return cuda_fail(h, (cudaError_t)e, "substitution sweep", __LINE__);
+        CK_LAUNCH();
     }
     return TC_OK;
 }
 
-static int subst(tc_handle h, double *R, int64_t ldr, int nrhs, bool back) {
-    if (h->ooc) return ooc_subst(h, R, ldr, nrhs, back, nullptr);
-    return subst_w(h, static_cast<const double *>(h->W.p), h->nt, R, ldr, nrhs, back);
+// Before the sweeps of a call: room for their counters, and their error word cleared.
+static int sweep_begin(tc_handle h) {
+    const int rc = ensure(h, h->sweep, (1 + SWEEP_GROUPS) * sizeof(int));
+    if (rc) return rc;
+    CK(cudaMemsetAsync(h->sweep.p, 0, sizeof(int), h->s));
+    return TC_OK;
+}
+// After them: waits for the stream and reports a wait of a sweep that ran into its bound.
+static int sweep_end(tc_handle h) {
+    int e = 0;
+    CK(cudaMemcpyAsync(&e, h->sweep.p, sizeof e, cudaMemcpyDeviceToHost, h->s));
+    CK(cudaStreamSynchronize(h->s));
+    return e ? set_err(h, TC_ERR_TIMEOUT, "a substitution sweep timed out waiting for a block") : TC_OK;
 }
 
 int tile_chol_solve(tc_handle h, int nrhs, const double *B, int64_t ldb, double *X, int64_t ldx, int max_refine,
@@ -1276,8 +1275,7 @@ int tile_chol_solve(tc_handle h, int nrhs, const double *B, int64_t ldb, double 
     CK(cudaMemcpy2DAsync(Bd, ldr * sizeof(double), B, ldb * sizeof(double), n * sizeof(double), nrhs,
                          cudaMemcpyDefault, h->s));
     CK(cudaMemcpyAsync(Xd, Bd, colbytes, cudaMemcpyDeviceToDevice, h->s));
-    rc = subst(h, Xd, ldr, nrhs, true);
-    if (rc) return rc;
+    if ((rc = sweep_begin(h)) || (rc = subst(h, Xd, ldr, nrhs, true))) return rc;
     double *sc = static_cast<double *>(h->scratch.p);
     // ||A||_inf (once per factor): max row sum of |A| = max of |A| * ones
     if (h->ooc) max_refine = 0;      // A was overwritten by the out-of-core factor: no residuals
@@ -1337,7 +1335,7 @@ int tile_chol_solve(tc_handle h, int nrhs, const double *B, int64_t ldb, double 
     }
     CK(cudaMemcpy2DAsync(X, ldx * sizeof(double), Xd, ldr * sizeof(double), n * sizeof(double), nrhs,
                          cudaMemcpyDefault, h->s));
-    CK(cudaStreamSynchronize(h->s));
+    if ((rc = sweep_end(h))) return rc;
     if (stats) {
         memset(stats, 0, sizeof *stats);
         stats->t_ms = now_ms() - t0;
@@ -1361,13 +1359,12 @@ int tile_chol_loglik(tc_handle h, const double *y, double *loglik_out) {
         double *z = static_cast<double *>(h->vec.p);
         CK(cudaMemsetAsync(z, 0, (size_t)ldr * sizeof(double), h->s));
         CK(cudaMemcpyAsync(z, y, (size_t)h->n * sizeof(double), cudaMemcpyDefault, h->s));
-        rc = subst(h, z, ldr, 1, false);
-        if (rc) return rc;
+        if ((rc = sweep_begin(h)) || (rc = subst(h, z, ldr, 1, false))) return rc;
         double *sc = static_cast<double *>(h->scratch.p);
         launch_dot_self(z, h->n, sc, h->s);
         CK_LAUNCH();
         CK(cudaMemcpyAsync(&quad, sc, sizeof(double), cudaMemcpyDeviceToHost, h->s));
-        CK(cudaStreamSynchronize(h->s));
+        if ((rc = sweep_end(h))) return rc;
     }
     *loglik_out = -0.5 * (double)h->n * std::log(two_pi) - 0.5 * h->logdet - 0.5 * quad;
     return TC_OK;

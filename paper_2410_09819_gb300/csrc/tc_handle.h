@@ -48,6 +48,7 @@ struct tc_handle_s {
     DevBuf tables;     // schedule tables
     DevBuf partials;   // split-K partial blocks
     DevBuf vec;        // solve workspace
+    DevBuf sweep;      // substitution sweeps: error word, progress counters
     DevBuf sumsq;      // tile sums of squares
     // mixed precision: operand pools, tables and tensor maps
     DevBuf pool_hi, pool_lo, pool16, pool8;

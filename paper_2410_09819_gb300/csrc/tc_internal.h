@@ -159,11 +159,17 @@ void launch_fix_padding_tile(double *T, int b, int nv, int diag, cudaStream_t s)
 void launch_fwd_update_tile(const double *L, int b, int i, int j, double *R, int64_t ldr, int nrhs, cudaStream_t s);
 void launch_bwd_update_tile(const double *L, int b, int i, int j, double *R, int64_t ldr, int nrhs, cudaStream_t s);
 
+// ------------------------------------------------------------------ launchers (k_sweep.cu)
+// Forward (L z = r) or back (L^T x = z) substitution of nrhs right-hand sides of nblk 64-row blocks
+// (column-major, leading dimension ldr), in place; progress: SWEEP_GROUPS counters.  Returns a
+// cudaError_t of the cooperative launch; a wait that runs into its bound (0: 4 s) sets *err.
+constexpr int SWEEP_GROUPS = 64;
+int launch_sweep(const double *W, int b, int nblk, double *r, int64_t ldr, int nrhs, bool fwd, int *progress, int *err,
+                 cudaStream_t s, unsigned long long limit_ns);
+
 // solves (column-major right-hand sides, leading dimension ldr, nrhs <= 16 per launch)
 void launch_fwd_diag(const double *Ljj, int b, double *R, int64_t ldr, int nrhs, cudaStream_t s);
-void launch_fwd_update(const double *W, int nt, int b, int j, double *R, int64_t ldr, int nrhs, cudaStream_t s);
 void launch_bwd_diag(const double *Ljj, int b, double *R, int64_t ldr, int nrhs, cudaStream_t s);
-void launch_bwd_update(const double *W, int nt, int b, int j, double *R, int64_t ldr, int nrhs, cudaStream_t s);
 void launch_symv_resid(const double *A, int nt, int b, int64_t n, const double *X, int64_t ldx,
                        const double *B, int64_t ldb, double *R, int64_t ldr, int nrhs, int absmode,
                        cudaStream_t s);
