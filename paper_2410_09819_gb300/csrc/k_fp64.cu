@@ -101,17 +101,24 @@ k_dgemm_reduce(const DRed *__restrict__ reds, int ld, const double *__restrict__
 // Factor the 64 x 64 lower block at D in place (right-looking in shared memory).  A non-positive
 // pivot records the 1-based global column in *status and stops.
 //
-// What bounds it: latency, then the FP64 pipe of one SM.  A dependent FP64 operation takes 66
-// cycles, a division 440 and a square root 690, and a warp's FP64 instruction holds its SM quarter
-// for 64 cycles whatever lanes are active.  So 128 threads (one warp a quarter); the pivot's root and
-// its reciprocal come from integer arithmetic (fixed_exp.h: the same correctly rounded values in
-// about 450 cycles together); while warps 0 and 1 form column j, warps 2 and 3 already go through
-// what is left of step j - 1, element lists in column order so that a finished column costs nothing.
-// Every element sees the same operations in the same order as in the plain loop.  A block took 94 us
-// with a square root, a division and three barriers of 256 threads in every step.
-constexpr int POTRF_THREADS = 128;
+// What bounds it: latency.  A dependent FP64 operation (a comparison too) takes 66 cycles, a division
+// 440 and a square root 690, and a warp's FP64 instruction holds its SM quarter for 64 cycles whatever
+// lanes are active.  So warps 0 and 1 run the chain, a thread per row with its element of the
+// current column in a register: the pivot's root and its reciprocal in integer arithmetic
+// (fixed_exp.h: the same correctly rounded values), one multiplication, one barrier, one
+// multiply-add for the next column; warps 2 to 5 meanwhile take the previous step to the columns
+// behind, through an element list in column order in which a finished column costs nothing.  Every
+// element sees the same operations in the same order as in the plain loop.   A block took 94 us with a
+// square root, a division and three barriers of 256 threads a step, 73 us with two barriers and
+// FP64 comparisons on the chain, 52 us here.
+constexpr int POTRF_THREADS = 192;
+__device__ __forceinline__ bool positive(double d) {       // d > 0 without the FP64 pipe
+    const long long w = __double_as_longlong(d);
+    return w > 0 && w <= 0x7FF0000000000000ll;
+}
 __device__ __forceinline__ void pivot_root(double d, double &sd, double &rp) {
-    if (d > 1e-280 && d < 1e280) {
+    const int e = __double2hiint(d) >> 20;
+    if (e > 100 && e < 1946) {
         const fx::Num h = fx::sqrt_rn(d);
         sd = fx::value(h);
         rp = fx::value(fx::recip_rn(h));
@@ -122,52 +129,56 @@ __device__ __forceinline__ void pivot_root(double d, double &sd, double &rp) {
 }
 __device__ __forceinline__ void potrf64_body(double *D, int ld, int col0, int *status) {
     __shared__ double S[64][65];                 // S[c][r], r >= c: L_rc once column c is done
-    __shared__ double zs[2][64], ls[2][64];      // column j before and after its scaling
+    __shared__ double ls[2][64];                 // column j of L
+    __shared__ int fail;
     __shared__ uint16_t tab[2080];               // elements (c << 8 | r), columns from the last to the first
     const int tid = threadIdx.x, warp = tid >> 5;
     for (int idx = tid; idx < 4096; idx += POTRF_THREADS) {
         const int r = idx & 63, c = idx >> 6;
         if (r >= c) {
-            const double v = D[(int64_t)c * ld + r];
-            S[c][r] = v;
-            if (c == 0) zs[0][r] = v;
+            S[c][r] = D[(int64_t)c * ld + r];
             tab[(63 - c) * (64 - c) / 2 + r - c] = (uint16_t)(c << 8 | r);
         }
     }
+    if (tid == 0) fail = 0;
     __syncthreads();
-    int fail = 0;
-    for (int j = 0; j < 64; ++j) {
-        // zs[j & 1]: column j; ls[j - 1 & 1]: column j - 1 of L, which columns j + 1 .. 63 have not
-        // seen yet
-        const int cur = j & 1, prv = cur ^ 1;
-        const double d = zs[cur][j];
-        if (!(d > 0.0)) {                        // every thread reads the same pivot
-            fail = j + 1;
-            break;
-        }
-        const int n = j > 0 ? (63 - j) * (64 - j) / 2 : 0;   // elements of columns j + 1 ..
-        // the root costs a warp about as much as 320 elements
-        const int h = n + 640 < 2 * n ? (n + 640) / 2 : n;
-        if (warp < 2) {
-            double sd, rp;
-            pivot_root(d, sd, rp);
-            if (tid >= j) {
-                const double l = tid == j ? sd : zs[cur][tid] * rp;
-                ls[cur][tid] = l;
-                S[j][tid] = l;
+    if (warp < 2) {
+        double z = S[0][tid], d = S[0][0];       // row tid of column j, and its pivot
+        for (int j = 0; j < 64; ++j) {
+            const int cur = j & 1;
+            if (positive(d)) {
+                double sd, rp;
+                pivot_root(d, sd, rp);
+                if (tid >= j) {
+                    z = tid == j ? sd : z * rp;
+                    ls[cur][tid] = z;
+                    S[j][tid] = z;
+                }
+            } else if (tid == 0) {
+                fail = j + 1;
+            }
+            __syncthreads();                     // column j is there, step j - 1 everywhere
+            if (!positive(d)) break;
+            if (j < 63) {
+                const double l = ls[cur][j + 1];
+                d = fma(-l, l, S[j + 1][j + 1]);
+                if (tid > j) z = fma(-z, l, S[j + 1][tid]);
             }
         }
-        const int e1 = warp < 2 ? n : h;
+    } else {
+        for (int j = 0; j < 64; ++j) {
+            const int cur = j & 1;
+            __syncthreads();
+            if (fail) break;
+            const int n = (62 - j) * (63 - j) / 2;        // elements of columns j + 2 ..
 #pragma unroll 4
-        for (int e = (warp < 2 ? h : 0) + (tid & 63); e < e1; e += 64) {
-            const int c = tab[e] >> 8, r = tab[e] & 63;
-            S[c][r] = fma(-ls[prv][r], ls[prv][c], S[c][r]);
+            for (int e = tid - 64; e < n; e += POTRF_THREADS - 64) {
+                const int c = tab[e] >> 8, r = tab[e] & 63;
+                S[c][r] = fma(-ls[cur][r], ls[cur][c], S[c][r]);
+            }
         }
-        __syncthreads();
-        if (j < 63 && tid > j && tid < 64)       // column j + 1 of step j
-            zs[prv][tid] = fma(-ls[cur][tid], ls[cur][j + 1], S[j + 1][tid]);
-        __syncthreads();
     }
+    __syncthreads();
     if (fail) {
         if (tid == 0) atomicCAS(status, 0, col0 + fail);
         return;
@@ -200,8 +211,8 @@ __device__ __forceinline__ void strip_solve(double (*Ss)[65], double (*Ls)[65], 
 
 // POTRF panel: rows below the factored 64-block within the diagonal tile, X L^T = C for
 // PANEL_ROWS rows a CTA, one warp a row: lane l holds columns l and l + 32, x_j travels by shuffle,
-// and no step needs a barrier.  Bound by the FP64 pipe (160 warp operations of 64 cycles a row): 8
-// rows take 10 us, against 28 us for 16 rows with two block barriers a step.
+// and no step needs a barrier.  Bound by the FP64 pipe (160 warp operations of 64 cycles a row, 10 us
+// for 8 rows): a launch takes 17 us, where 16 rows with two block barriers a step took 28 us.
 constexpr int PANEL_ROWS = 8;
 __device__ __forceinline__ void panel_body(double *Pb, const double *L, int ld) {
     __shared__ double Ls[64][65], rinv[64];      // Ls[j][c] = l_cj, c >= j
@@ -807,62 +818,55 @@ void launch_trsm_rows_batched(const PEntry *e, int n, int max_rows, int ld, cuda
 
 
 // POTRF trailing update: C -= P P^T with the 64 columns P below the factored block at D, on the
-// 64 x 64 blocks of the lower part (diagonal ones whole), four CTAs of 32 x 32 elements each.  The FP64
-// pipe bounds it (1.7 multiply-adds a clock and SM): one CTA a 64 x 64 block keeps its SM busy for 69
-// us, and the 15 x 16 / 2 of them below the first panel of a 1024 tile are fewer than the SMs, so
-// every step took 69 us; with quarter-size blocks the steps of that tile take half of that on average.
-constexpr int SYRK_B = 32;
+// 64 x 64 blocks of the lower part (diagonal ones whole), sixteen CTAs of 16 x 16 elements each.  The
+// FP64 pipe bounds it (1.7 multiply-adds a clock and SM): one CTA a 64 x 64 block keeps its SM busy for
+// 69 us, and the 15 x 16 / 2 of them below the first panel of a 1024 tile are fewer than the SMs, so
+// every step took 69 us (35 us on average in blocks of 32 x 32, 27 us in these).  At tile 2048 the 84 us
+// of a step are the pipe's.
+constexpr int SYRK_B = 16, SYRK_THREADS = 64;
 __device__ __forceinline__ void syrk_body(double *D, int ld) {
     __shared__ double X[64][SYRK_B], Y[64][SYRK_B];
-    const int t = blockIdx.x >> 2, tid = threadIdx.x;
+    const int t = blockIdx.x >> 4, tid = threadIdx.x;
     int bi = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
     while (bi * (bi + 1) / 2 > t) --bi;
     while ((bi + 1) * (bi + 2) / 2 <= t) ++bi;
-    const int bj = 2 * (t - bi * (bi + 1) / 2) + ((blockIdx.x >> 1) & 1);
-    bi = 2 * bi + (blockIdx.x & 1);
+    const int bj = 4 * (t - bi * (bi + 1) / 2) + ((blockIdx.x >> 2) & 3);
+    bi = 4 * bi + (blockIdx.x & 3);
     const double *P = D + 64;
     double *C = D + (int64_t)(64 + bj * SYRK_B) * ld + 64 + bi * SYRK_B;
-    const int r = tid & 31, q = tid >> 5;
+    const int r = tid & 15, q = tid >> 4;
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
         X[q + 4 * k][r] = P[(int64_t)(q + 4 * k) * ld + bi * SYRK_B + r];
         Y[q + 4 * k][r] = P[(int64_t)(q + 4 * k) * ld + bj * SYRK_B + r];
     }
-    // 2 rows x 4 columns a thread
-    const int tx = tid & 15, ty = tid >> 4;
-    double acc[2][4] = {};
+    // a row and four columns a thread
+    double acc[4] = {};
     __syncthreads();
 #pragma unroll 16
     for (int k = 0; k < 64; ++k) {
-        const double a0 = X[k][tx], a1 = X[k][tx + 16];
+        const double a = X[k][r];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const double y = Y[k][ty + 8 * c];
-            acc[0][c] = fma(a0, y, acc[0][c]);
-            acc[1][c] = fma(a1, y, acc[1][c]);
-        }
+        for (int c = 0; c < 4; ++c) acc[c] = fma(a, Y[k][q + 4 * c], acc[c]);
     }
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        C[(int64_t)(ty + 8 * c) * ld + tx] -= acc[0][c];
-        C[(int64_t)(ty + 8 * c) * ld + tx + 16] -= acc[1][c];
-    }
+    for (int c = 0; c < 4; ++c) C[(int64_t)(q + 4 * c) * ld + r] -= acc[c];
 }
-__global__ void __launch_bounds__(128) k_syrk_rows_batched(const PEntry *__restrict__ e, int ld) {
+__global__ void __launch_bounds__(SYRK_THREADS) k_syrk_rows_batched(const PEntry *__restrict__ e, int ld) {
     const PEntry E = e[blockIdx.y];
     if (!failed(E.status)) syrk_body(E.D, ld);
 }
-__global__ void __launch_bounds__(128) k_syrk_rows(double *D, int ld, const int *status) {
+__global__ void __launch_bounds__(SYRK_THREADS) k_syrk_rows(double *D, int ld, const int *status) {
     if (!failed(status)) syrk_body(D, ld);
 }
 void launch_syrk_rows_batched(const PEntry *e, int n, int rows, int ld, cudaStream_t s) {
     const int m = rows / 64;
     for (int i = 0; i < n && m > 0; i += 65535)
-        k_syrk_rows_batched<<<dim3(2 * m * (m + 1), n - i < 65535 ? n - i : 65535), 128, 0, s>>>(e + i, ld);
+        k_syrk_rows_batched<<<dim3(8 * m * (m + 1), n - i < 65535 ? n - i : 65535), SYRK_THREADS, 0, s>>>(e + i, ld);
 }
 void launch_syrk_rows(double *D, int rows, int ld, const int *status, cudaStream_t s) {
     const int m = rows / 64;
-    if (m > 0) k_syrk_rows<<<2 * m * (m + 1), 128, 0, s>>>(D, ld, status);
+    if (m > 0) k_syrk_rows<<<8 * m * (m + 1), SYRK_THREADS, 0, s>>>(D, ld, status);
 }
 
 // log|A_i| = 2 sum log L_ii for every matrix of a batch (one CTA each, fixed order)
