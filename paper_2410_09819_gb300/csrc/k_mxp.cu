@@ -529,7 +529,8 @@ static EncodeTiledFn encode_fn() {
 // 2-D map over a pool: rows = nslots * b, columns = b elements of esize bytes; box of
 // (128 bytes) x box_rows with 128-byte swizzle.
 // rows of b elements; box: box_k_bytes (128 or 64, swizzled to match) x box_rows
-int make_pool_map_k(CUtensorMap *map, void *pool, int64_t nslots, int b, int esize, int box_rows, int box_k_bytes) {
+static int make_pool_map_k(CUtensorMap *map, void *pool, int64_t nslots, int b, int esize, int box_rows,
+                           int box_k_bytes) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return -1;
     if (box_k_bytes != 128 && box_k_bytes != 64) return -1;

@@ -58,6 +58,14 @@ constexpr unsigned long long ZLIMIT_NS = 4000000000ull;   // default bound of a 
 constexpr unsigned long long ZDRAIN_NS = 2000000000ull;   // bound of the teardown waits
 
 // ------------------------------------------------------------------- digit planes
+// Base-256 planes lie as the shared memory of k_zgemm wants them: columns in blocks of ZKE, in a block
+// row after row of 64 bytes, the 16-byte pieces of a row in the order of the 64-byte swizzle
+// (piece c of row r at c ^ (r / 2 mod 4)).  A stage's part of a plane is then one contiguous piece of 8
+// or 2 KB, which a plain bulk copy brings at 117 bytes a clock and SM (95 on all SMs at once); boxes
+// of 64-byte rows through a tensor map came at 60, a row a clock, however the rows lay.
+__device__ __forceinline__ int64_t plane_at(int b, int row, int col) {      // element (row, col), col % 8 == 0
+    return ((int64_t)(col / ZKE) * b + row) * ZKE + 8 * (((col % ZKE) / 8) ^ ((row >> 1) & 3));
+}
 // Base-256 planes of eight adjacent columns of a row (k_zgemm), one 16-byte store per plane.
 __device__ __forceinline__ void put_planes8(const long long (&q)[8], __half *P, int64_t o, int64_t bb) {
     uint32_t lo[8], hi[8];
@@ -125,7 +133,7 @@ __device__ __forceinline__ void planes_of_tile(const double *T, int b, bool tran
             long long q[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) q[u] = fixed56(S[c + u][r], e);
-            put_planes8(q, reinterpret_cast<__half *>(P), (int64_t)(r0 + r) * b + c0 + c, bb);
+            put_planes8(q, reinterpret_cast<__half *>(P), plane_at(b, r0 + r, c0 + c), bb);
         } else {
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -158,6 +166,7 @@ k_digits(const double *W, int b, const int *tiles, const double *amax, uint8_t *
 // In-core form: item i is items[i]; its sources are the consecutive digit slots
 // it.xoff + n and it.yoff + n.
 struct ZArgs {
+    const uint8_t *pool;
     const ZItem *items;
     int nitems;
     const int *exps;
@@ -181,6 +190,7 @@ struct ZArgs {
 // ntiles x (b/ZBM) x (b/ZBN) blocks; blocks entirely above the diagonal of a `lower` tile
 // carry no work.
 struct ZGroupArgs {
+    const uint8_t *pool;
     double *C[ZG_MAX];
     uint16_t xs[ZG_MAX][ZK_MAX];   // X_n of tile g: digit slot xs[g][n]
     uint16_t ys[ZK_MAX];           // Y_n (shared by the group): digit slot ys[n]
@@ -220,7 +230,7 @@ __device__ __forceinline__ int z_kblocks(const Args &a, const ZItem &it) {
 // Persistent update kernel: C -= sum_{n<k} X_n Y_n^T for 128 x ZBN output blocks, X_n the
 // tiles (m, n) and Y_n the tiles (k, n), through their first P digit planes and the pairs
 // s + t < P (launch_form below lists which P serves which output precision).
-//   warp 0  TMA producer: per source and 32 elements of K one stage, the P X planes of the
+//   warp 0  copies: per source and 32 elements of K one stage, the P X planes of the
 //           block's 128 rows and the P Y planes of its 32 columns;
 //   warp 1  MMA issuer: per stage and X plane s, one tcgen05.mma per 16 elements of K with
 //           N = ZBN (P - s) multiplies it by all its partners Y_0 .. Y_{P-1-s} at once; column
@@ -238,10 +248,11 @@ __device__ __forceinline__ int z_kblocks(const Args &a, const ZItem &it) {
 // prologue).
 // What bounds it: the tensor pipe.  Per 128 elements of K the 8 x 7 MMAs of P = 7 take
 // 8 (112 + 96 + 80 + 64 + 48 + 2 x 41) = 3856 cycles for 128 x 32 outputs (an MMA takes
-// max(41, N / 2) cycles); measured 4990, of which 750 wait for a stage's copies (56 bytes a clock
-// and SM).  The updates of an FP64 factorization of order 32768, tile 1024: 346 ms with base 16 in
-// E4M3 (105 pairs, 128 x 16 items), 186 ms here (1.70 PFLOP/s of FP16 pair work).  64 columns in
-// two buffers do not fit TMEM.
+// max(41, N / 2) cycles); measured 4990 with boxes of 64-byte rows, of which 750 waited for a stage's
+// copies (56 bytes a clock and SM, a row a clock).  All P = 7 products of an FP64 factorization of
+// order 32768, tile 1024: 212 ms with those, 199 ms with bulk copies of the blocked planes (its
+// updates alone took 346 ms with base 16 in E4M3: 105 pairs, 128 x 16 items).  64 columns in two
+// buffers do not fit TMEM.
 //
 // Failure handling: every pipeline wait gives up after args.limit_ns (or when another role
 // set the abort flag), and the CTA then sets *err and stops issuing.  Before the TMEM is
@@ -250,8 +261,7 @@ __device__ __forceinline__ int z_kblocks(const Args &a, const ZItem &it) {
 // depend on nothing outside the CTA, so they end) and are bounded by ZDRAIN_NS.
 template <int P, class Args>
 __global__ void __maxnreg__(168)   // 320 threads: 3 warps on some SMSP x 32 x 168 <= 16K registers
-k_zgemm(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapY,
-        const __grid_constant__ Args args) {
+k_zgemm(const __grid_constant__ Args args) {
     static_assert(P <= ZS && 2 * P * ZBN <= 512, "two accumulator buffers fit TMEM");
     extern __shared__ __align__(1024) uint8_t zsmem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(zsmem_raw) + 1023) & ~uintptr_t(1023));
@@ -296,24 +306,28 @@ k_zgemm(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtens
     const uint32_t tmem = *tmem_holder;
 
     if (warp == 0) {
-        // --------------------------------------------------------------- TMA producer
+        // --------------------------------------------------------------- producer (bulk copies)
         int st = 0, ph = 1, issued = 0;             // empty slots: phase 1 passes
+        const int64_t plane = 2 * (int64_t)b * b, slot = ZS * plane;
         bool ok = true;
         for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
             ZItem it;
             if (!args.tile(item, it)) continue;
             const int kblocks = z_kblocks(args, it);
             for (int n = 0; n < k && ok; ++n) {
-                const int xrow = args.xsrc(it, n) * ZS * b + it.bm * ZBM, yrow = args.ysrc(it, n) * ZS * b + it.bn * ZBN;
+                const uint8_t *x = args.pool + args.xsrc(it, n) * slot + it.bm * ZX_BYTES;
+                const uint8_t *y = args.pool + args.ysrc(it, n) * slot + it.bn * ZY_BYTES;
                 for (int kb = 0; kb < kblocks; ++kb) {
                     if (!z_wait_all(empty + st, ph, abort_flag, lim)) { ok = false; break; }
                     uint8_t *xs = smem + st * ZSTAGE, *ys = xs + ZS * ZX_BYTES;
                     z_expect_w(full + st, P * (ZX_BYTES + ZY_BYTES));
 #pragma unroll
                     for (int s = 0; s < P; ++s) {
-                        z_tma_w(xs + s * ZX_BYTES, &mapX, kb * ZKE, xrow + s * b, full + st);
-                        z_tma_w(ys + s * ZY_BYTES, &mapY, kb * ZKE, yrow + s * b, full + st);
+                        z_bulk_w(xs + s * ZX_BYTES, x + s * plane, ZX_BYTES, full + st);
+                        z_bulk_w(ys + s * ZY_BYTES, y + s * plane, ZY_BYTES, full + st);
                     }
+                    x += (int64_t)b * ZKB;
+                    y += (int64_t)b * ZKB;
                     ++issued;
                     if (++st == ZST) { st = 0; ph ^= 1; }
                 }
@@ -525,11 +539,6 @@ void launch_amax_ptr(const double *src, int64_t count, double *out, cudaStream_t
 void launch_set_identity(double *T, int b, cudaStream_t s) { k_set_identity<<<64, 256, 0, s>>>(T, b); }
 
 // ------------------------------------------------------------------------- host side
-// map over the base-256 digit pool: slots x 7 planes x b rows of b FP16 values; box 32 values x box_rows
-int make_digit_map(CUtensorMap *map, void *pool, int64_t nslots, int b, int box_rows) {
-    return make_pool_map_k(map, pool, nslots * ZS, b, 2, box_rows, ZKB);
-}
-
 size_t zgemm_smem_bytes() { return (size_t)ZST * ZSTAGE + 1024 + 256; }
 
 static int sm_count() {            // per device, cached
@@ -567,7 +576,7 @@ void launch_add_tiles(double *W, int b, const int *tiles, int ntiles, const doub
 // P planes of base 256 are worth 2P base-16 digits: they round an operand to 2^-(8P+1) of its
 // scale, and the pairs they leave out stay below 2^-(8P) of the product's.
 template <class Args>
-static void launch_form(int planes, const CUtensorMap &mx, const CUtensorMap &my, const Args &a, int nitems, cudaStream_t s) {
+static void launch_form(int planes, const Args &a, int nitems, cudaStream_t s) {
     static std::atomic<unsigned long long> attr{0};
     const size_t smem = zgemm_smem_bytes();
     if (attrs_pending(attr)) {
@@ -579,26 +588,27 @@ static void launch_form(int planes, const CUtensorMap &mx, const CUtensorMap &my
         mark_attrs_set(attr);
     }
     const int grid = nitems < sm_count() ? nitems : sm_count();      // persistent: one CTA per SM
-    if (planes == 10) k_zgemm<5, Args><<<grid, ZTHREADS, smem, s>>>(mx, my, a);
-    else if (planes == 7) k_zgemm<4, Args><<<grid, ZTHREADS, smem, s>>>(mx, my, a);
-    else if (planes == 6) k_zgemm<3, Args><<<grid, ZTHREADS, smem, s>>>(mx, my, a);
-    else if (planes == 4) k_zgemm<2, Args><<<grid, ZTHREADS, smem, s>>>(mx, my, a);
-    else k_zgemm<7, Args><<<grid, ZTHREADS, smem, s>>>(mx, my, a);
+    if (planes == 10) k_zgemm<5, Args><<<grid, ZTHREADS, smem, s>>>(a);
+    else if (planes == 7) k_zgemm<4, Args><<<grid, ZTHREADS, smem, s>>>(a);
+    else if (planes == 6) k_zgemm<3, Args><<<grid, ZTHREADS, smem, s>>>(a);
+    else if (planes == 4) k_zgemm<2, Args><<<grid, ZTHREADS, smem, s>>>(a);
+    else k_zgemm<7, Args><<<grid, ZTHREADS, smem, s>>>(a);
 }
 
-void launch_zgemm(const CUtensorMap &mx, const CUtensorMap &my, const ZItem *items, int nitems, const int *exps, int k,
+void launch_zgemm(const uint8_t *pool, const ZItem *items, int nitems, const int *exps, int k,
                   int b, int *err, cudaStream_t s, int planes, int assign, int tri, unsigned long long limit_ns,
                   int stall) {
     if (nitems <= 0 || k <= 0) return;
-    const ZArgs a{items, nitems, exps, k, b, err, assign, tri, limit_ns ? limit_ns : ZLIMIT_NS, stall};
-    launch_form(planes, mx, my, a, nitems, s);
+    const ZArgs a{pool, items, nitems, exps, k, b, err, assign, tri, limit_ns ? limit_ns : ZLIMIT_NS, stall};
+    launch_form(planes, a, nitems, s);
 }
 
-void launch_zgemm_group(const CUtensorMap &mx, const CUtensorMap &my, const ZGroup &g, const int *exps, int b,
-                        int *err, cudaStream_t s, int planes, int tri, unsigned long long limit_ns, int stall) {
+void launch_zgemm_group(const uint8_t *pool, const ZGroup &g, const int *exps, int b, int *err,
+                        cudaStream_t s, int planes, int tri, unsigned long long limit_ns, int stall) {
     if (g.ntiles <= 0 || g.k <= 0) return;
     ZGroupArgs a;
     memset(&a, 0, sizeof a);
+    a.pool = pool;
     for (int t = 0; t < g.ntiles; ++t) {
         a.C[t] = g.C[t];
         if (g.lower[t]) a.lower |= 1u << t;
@@ -614,7 +624,7 @@ void launch_zgemm_group(const CUtensorMap &mx, const CUtensorMap &my, const ZGro
     a.tri = tri;
     a.limit_ns = limit_ns ? limit_ns : ZLIMIT_NS;
     a.stall = stall;
-    launch_form(planes, mx, my, a, g.ntiles * (b / ZBM) * (b / ZBN), s);
+    launch_form(planes, a, g.ntiles * (b / ZBM) * (b / ZBN), s);
 }
 
 }  // namespace tc

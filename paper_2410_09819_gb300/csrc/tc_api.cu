@@ -607,9 +607,6 @@ int prepare_factor(tc_handle h, const Plan &P, const MxpPlan *M, PlanDev &D) {
             D.pairs = reinterpret_cast<unsigned long long *>(zb + opc);
         }
         h->pairs_dev = D.pairs;
-        if (P.zwidth == Z_BN && (make_digit_map(&h->map_zx, h->dpool.p, Tt, h->b, 128) ||
-                                 make_digit_map(&h->map_zy, h->dpool.p, Tt, h->b, Z_BN)))
-            return set_err(h, TC_ERR_CUDA, "cuTensorMapEncodeTiled failed for the digit planes");
         if (P.zwidth == Z64_BN && make_zgemm64_maps(&h->maps64, h->dpool.p, Tt * Z16_PLANES, h->b))
             return set_err(h, TC_ERR_CUDA, "cuTensorMapEncodeTiled failed for the digit planes (3D maps)");
     }
@@ -679,7 +676,7 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
                 launch_zgemm64(h->maps64, D.zitems + C.z0, C.nz, D.zexps, k, b, status + 1, h->s, zp64, 0, 0,
                                wait_limit_ns(h), wait_test(h));
             else
-                launch_zgemm(h->map_zx, h->map_zy, D.zitems + C.z0, C.nz, D.zexps, k, b, status + 1, h->s, 14, 0, 0,
+                launch_zgemm(static_cast<const uint8_t *>(h->dpool.p), D.zitems + C.z0, C.nz, D.zexps, k, b, status + 1, h->s, 14, 0, 0,
                              wait_limit_ns(h), wait_test(h));
             span_end(h, sp);
             CK_LAUNCH();
@@ -766,21 +763,21 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
                 CK_LAUNCH();
                 launch_digits_src(Lkk, b, 0, gl, am_l + gl, pool, D.zexps, h->s);
                 CK_LAUNCH();
-                launch_zgemm(h->map_zx, h->map_zy, D.zinvc + C.v0, C.nv, D.zexps, 1, b, status + 1, h->s, 14, 1, 1,
+                launch_zgemm(static_cast<const uint8_t *>(h->dpool.p), D.zinvc + C.v0, C.nv, D.zexps, 1, b, status + 1, h->s, 14, 1, 1,
                              wait_limit_ns(h), wait_test(h));
                 CK_LAUNCH();
                 launch_tile_amax(W, b, D.dtiles + C.dg0, C.ndg, am_x, h->s, X0);
                 CK_LAUNCH();
                 launch_digits(W, b, D.dtiles + C.dg0, C.ndg, am_x, pool, D.zexps, h->s, false, X0);
                 CK_LAUNCH();
-                launch_zgemm(h->map_zx, h->map_zy, D.zref + C.v0, C.nv, D.zexps, 1, b, status + 1, h->s, 14, 0, 1,
+                launch_zgemm(static_cast<const uint8_t *>(h->dpool.p), D.zref + C.v0, C.nv, D.zexps, 1, b, status + 1, h->s, 14, 0, 1,
                              wait_limit_ns(h), wait_test(h));
                 CK_LAUNCH();
                 launch_tile_amax(W, b, D.dtiles + C.dg0, C.ndg, am_r, h->s);
                 CK_LAUNCH();
                 launch_digits(W, b, D.dtiles + C.dg0, C.ndg, am_r, pool, D.zexps, h->s, false);
                 CK_LAUNCH();
-                launch_zgemm(h->map_zx, h->map_zy, D.zinv + C.v0, C.nv, D.zexps, 1, b, status + 1, h->s, ZREF_PLANES, 1, 1,
+                launch_zgemm(static_cast<const uint8_t *>(h->dpool.p), D.zinv + C.v0, C.nv, D.zexps, 1, b, status + 1, h->s, ZREF_PLANES, 1, 1,
                              wait_limit_ns(h), wait_test(h));
                 CK_LAUNCH();
                 launch_add_tiles(W, b, D.dtiles + C.dg0, C.ndg, X0, h->s);

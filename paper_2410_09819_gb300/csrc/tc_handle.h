@@ -54,10 +54,9 @@ struct tc_handle_s {
     DevBuf pool_hi, pool_lo, pool16, pool8;
     DevBuf mxtab;
     CUtensorMap map_hi{}, map_lo{}, map16{}, map8{};
-    // emulated FP64 updates: digit planes, their tables and tensor maps
+    // emulated FP64 updates: digit planes and their tables
     DevBuf dpool, ztab, invbuf;
     DevBuf stab;       // grouped batched-solve task tables
-    CUtensorMap map_zx{}, map_zy{};
     tc::Z64Maps maps64{};                // 3D digit-plane maps of the mixed-precision update kernel
     // matrices of the last (batched) factorization
     std::vector<MatDesc> mats;

@@ -277,11 +277,12 @@ void launch_add_tile(double *dst, const double *src, int b, cudaStream_t s);    
 // Y tiles are lower triangular; limit_ns: bound of each pipeline wait (0: 4 s), after which *err
 // is set and the call ends; stall != 0: the failure-detection test hook (the MMA issuer waits on
 // a barrier nothing arrives at).
-void launch_zgemm(const CUtensorMap &mx, const CUtensorMap &my, const ZItem *items, int nitems, const int *exps, int k,
+// pool: the digit planes, slot t (7 planes of b x b FP16 values, k_ozaki.cu) at 14 t b^2 bytes.
+void launch_zgemm(const uint8_t *pool, const ZItem *items, int nitems, const int *exps, int k,
                   int b, int *err, cudaStream_t s, int planes, int assign, int tri, unsigned long long limit_ns,
                   int stall);
-void launch_zgemm_group(const CUtensorMap &mx, const CUtensorMap &my, const ZGroup &g, const int *exps, int b,
-                        int *err, cudaStream_t s, int planes, int tri, unsigned long long limit_ns, int stall);
+void launch_zgemm_group(const uint8_t *pool, const ZGroup &g, const int *exps, int b, int *err,
+                        cudaStream_t s, int planes, int tri, unsigned long long limit_ns, int stall);
 // Plane counts of a mixed-precision update launch (k_zgemm64): per source, the X / Y planes its
 // stored formats can have non-zero (src_planes_tab; nullptr: all), and a pair budget relative to
 // the output tile's scale: su = rref - floor((e_out - e_x - e_y - 4 margin) / 4), within
@@ -297,11 +298,9 @@ void launch_digits_src(const double *src, int b, int transpose, int dst, const d
                        cudaStream_t s, bool e4m3 = false);
 void launch_amax_ptr(const double *src, int64_t count, double *out, cudaStream_t s);
 void launch_set_identity(double *T, int b, cudaStream_t s);
-int make_digit_map(CUtensorMap *map, void *pool, int64_t nslots, int b, int box_rows);
 
 // ------------------------------------------------------------------ launchers (k_mxp.cu)
 int make_pool_map(CUtensorMap *map, void *pool, int64_t nslots, int b, int esize, int box_rows);
-int make_pool_map_k(CUtensorMap *map, void *pool, int64_t nslots, int b, int esize, int box_rows, int box_k_bytes);
 // 3D map over nplanes byte planes of b x b (row-major, K innermost): box 128 bytes x box_rows x depth
 int make_plane_map3(CUtensorMap *map, void *pool, int64_t nplanes, int b, int box_rows, int depth);
 int make_zgemm64_maps(Z64Maps *m, void *pool, int64_t nplanes, int b);

@@ -59,7 +59,7 @@ struct TileCache {
     double *amax = nullptr;      // per-slot max |a| of the (stored) tile
     double *amaxL = nullptr;     // per-slot max |a| before rounding to the stored precision
     int *tile_e = nullptr;       // per-tile storage scale exponent (FP16 / FP8 tiles)
-    CUtensorMap mx, my, m16, m8;
+    CUtensorMap m16, m8;
     std::vector<char> has_amax, dig, c16, c8;
     // host side
     double *host = nullptr;      // the matrix in host memory (tile layout), in/out
@@ -291,8 +291,6 @@ int init_cache(tc_handle h, TileCache &C, double *host, int nt, int b, bool digi
         C.e16 = C.exps + nd;
         C.e8 = C.e16 + nd;
         C.tile_e = C.e8 + nd;
-        if (make_digit_map(&C.mx, C.dpool, nd, b, 128) || make_digit_map(&C.my, C.dpool, nd, b, Z_BN))
-            return set_err(h, TC_ERR_CUDA, "cuTensorMapEncodeTiled failed for the digit-plane cache");
         C.dig.assign(ns, 0);
         C.has_amax.assign(ns, 0);
     }
@@ -582,7 +580,7 @@ extern "C" int tile_chol_factor_ooc(tc_handle h, int64_t n, int b, double *A_til
                             zg.ntiles = cnt;
                             zg.k = kc;
                             for (int q = 0; q < kc; ++q) zg.ys[q] = ys[q];
-                            launch_zgemm_group(C.mx, C.my, zg, C.exps, b, status + 1, h->s, f == OP_Z14 ? 14 : 10, 0, wait_limit_ns(h), wait_test(h));
+                            launch_zgemm_group(C.dpool, zg, C.exps, b, status + 1, h->s, f == OP_Z14 ? 14 : 10, 0, wait_limit_ns(h), wait_test(h));
                         } else {
                             qg.ntiles = cnt;
                             qg.k = kc;
@@ -715,7 +713,7 @@ extern "C" int tile_chol_factor_ooc(tc_handle h, int64_t n, int b, double *A_til
                     if (refine) ref[nref++] = i;
                 }
                 for (int p = 0; p < 4; ++p)
-                    launch_zgemm_group(C.mx, C.my, z1[p], C.exps, b, status + 1, h->s, ZTRSM_PLANES[p], 1, wait_limit_ns(h), wait_test(h));
+                    launch_zgemm_group(C.dpool, z1[p], C.exps, b, status + 1, h->s, ZTRSM_PLANES[p], 1, wait_limit_ns(h), wait_test(h));
                 if (nref) {
                     ZGroup z2, z3;
                     z2.ntiles = z3.ntiles = nref;
@@ -730,9 +728,9 @@ extern "C" int tile_chol_factor_ooc(tc_handle h, int64_t n, int b, double *A_til
                         z2.C[r] = z3.C[r] = C.ptr(so[i]);
                         z2.xs[r][0] = z3.xs[r][0] = so[i];
                     }
-                    launch_zgemm_group(C.mx, C.my, z2, C.exps, b, status + 1, h->s, 14, 1, wait_limit_ns(h), wait_test(h));  // R = C - X0 L^T
+                    launch_zgemm_group(C.dpool, z2, C.exps, b, status + 1, h->s, 14, 1, wait_limit_ns(h), wait_test(h));  // R = C - X0 L^T
                     for (int r = 0; r < nref; ++r) C.planes_of(C.ptr(so[ref[r]]), so[ref[r]]);
-                    launch_zgemm_group(C.mx, C.my, z3, C.exps, b, status + 1, h->s, ZREF_PLANES, 1, wait_limit_ns(h), wait_test(h));  // R L^{-T}
+                    launch_zgemm_group(C.dpool, z3, C.exps, b, status + 1, h->s, ZREF_PLANES, 1, wait_limit_ns(h), wait_test(h));  // R L^{-T}
                     for (int r = 0; r < nref; ++r)
                         launch_add_tile(C.ptr(so[ref[r]]), inv + (int64_t)(1 + ref[r]) * C.bb, b, h->s);
                 }

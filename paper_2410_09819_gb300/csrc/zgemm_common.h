@@ -69,12 +69,12 @@ __device__ __forceinline__ void z_expect_w(uint64_t *bar, uint32_t bytes) {
         "@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}\n" ::"r"(z_smem(bar)), "r"(bytes)
         : "memory");
 }
-__device__ __forceinline__ void z_tma_w(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar) {
+// contiguous piece: both addresses and the size are multiples of 16 bytes
+__device__ __forceinline__ void z_bulk_w(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
     asm volatile(
         "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
-        "@e cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n\t}\n" ::"r"(
-            z_smem(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z_smem(bar))
+        "@e cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n\t}\n" ::"r"(z_smem(dst)),
+        "l"(src), "r"(bytes), "r"(z_smem(bar))
         : "memory");
 }
 // 3D tile load (K bytes, rows within a digit plane, plane index): consecutive planes in one copy
