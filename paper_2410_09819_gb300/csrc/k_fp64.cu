@@ -1378,60 +1378,118 @@ k_trsm_tile(const __grid_constant__ TGroup g, const double *L, int ld, int b, co
 }
 
 // Mixed maps: Y = L^{-1} for a lower-triangular b x b tile L (column-major, ld = b), by forward
-// substitution L y_c = e_c column by column.  CTA x owns columns 4x .. 4x+3 and
-// b-4-4x .. b-1-4x: a long and a short group, so every CTA carries about the same work
-// (column c costs (b - c)^2 / 2 multiply-adds).  For each group, and each 64-row block from
-// the group's first nonzero row on, the product with the already solved rows (kept in shared
-// memory) is followed by the 64 x 64 diagonal solve.
+// substitution L y_c = e_c column by column, two columns a CTA (column c costs (b - c)^2 / 2
+// multiply-adds, the longest come first).  For each 64-row block from the columns' own on, the product
+// with the solved rows, kept in shared memory, is followed by the block's triangle: a warp per
+// column, y_j and with it the next row by shuffle, the division in integer arithmetic (the same
+// rounding, fixed_exp.h).
 // The products with Y of a mixed factorization keep 10, 6 or 4 of its digit planes, so what they
 // cut off, and with it the last bit of a stored FP32, FP16 or FP8 value here and there, follows the
-// inverse's own rounding: it stays this column-by-column substitution, although the doubling of
-// k_bgemm.cu (all-FP64 maps) is several times as fast.
-constexpr int TRINV_COLS = 4;
-__device__ __forceinline__ void trinv_body(const double *__restrict__ L, int b, double *__restrict__ Y) {
-    extern __shared__ double tsm[];
-    double *Ys = tsm;                               // b x 4: the group's columns, row-major by row
-    double(*Ld)[65] = reinterpret_cast<double(*)[65]>(tsm + (size_t)b * TRINV_COLS);
-    double(*Acc)[TRINV_COLS] = reinterpret_cast<double(*)[TRINV_COLS]>(tsm + (size_t)b * TRINV_COLS + 64 * 65);
-    const int tid = threadIdx.x;
-    const int r = tid & 63, cg = tid >> 6;          // row in block, column of the group
-    for (int grp = 0; grp < 2; ++grp) {
-        const int c0 = grp == 0 ? (int)blockIdx.x * TRINV_COLS : b - TRINV_COLS - (int)blockIdx.x * TRINV_COLS;
-        const int ib0 = c0 / 64;
-        __syncthreads();                            // the previous group's output is written
-        for (int i = tid; i < ib0 * 64 * TRINV_COLS; i += 256) Ys[i] = 0.0;
-        for (int ib = ib0; ib < b / 64; ++ib) {
-            const int row = ib * 64 + r;
-            double a = (row == c0 + cg) ? 1.0 : 0.0;
-            for (int l = ib0 * 64; l < ib * 64; ++l) a = fma(-L[(int64_t)l * b + row], Ys[l * TRINV_COLS + cg], a);
-            Acc[r][cg] = a;
-            for (int i = tid; i < 4096; i += 256) {
-                const int rr = i & 63, cc = i >> 6;
-                Ld[rr][cc] = (rr >= cc) ? L[(int64_t)(ib * 64 + cc) * b + ib * 64 + rr] : 0.0;
-            }
-            __syncthreads();
-            for (int j = 0; j < 64; ++j) {
-                if (tid < TRINV_COLS) Acc[j][tid] = Acc[j][tid] / Ld[j][j];
-                __syncthreads();
-                {
-                    const int rr = tid / TRINV_COLS, cc = tid % TRINV_COLS;    // 64 x 4 = 256 threads
-                    if (rr > j) Acc[rr][cc] = fma(-Ld[rr][j], Acc[j][cc], Acc[rr][cc]);
-                }
-                __syncthreads();
-            }
-            Ys[(ib * 64 + tid / TRINV_COLS) * TRINV_COLS + tid % TRINV_COLS] = Acc[tid / TRINV_COLS][tid % TRINV_COLS];
-            __syncthreads();
-        }
-        for (int i = tid; i < b * TRINV_COLS; i += 256) {
-            const int rr = i % b, cc = i / b;
-            Y[(int64_t)(c0 + cc) * b + rr] = Ys[rr * TRINV_COLS + cc];
-        }
-    }
+// inverse's own rounding: it stays this column-by-column substitution, every element's multiply-adds in
+// ascending order, although the doubling of k_bgemm.cu (all-FP64 maps) is several times as fast.
+// What bounds it: the FP64 pipe (b^3 / 6 multiply-adds, 2.7 ms for a tile of 2048).  So L's blocks
+// arrive one ahead of their use, and the SM's other CTAs run while one is on its chain.  A tile of
+// 2048: 4.24 ms with four columns and 256 threads, barriers in the triangle and L read where it is
+// used, 3.23 ms here.
+constexpr int TRINV_COLS = 2, TRINV_THREADS = 128;
+struct TrinvDiv {
+    unsigned long long m, v;
+    int e, ok;
+};
+static size_t trinv_smem(int b) {
+    return (2 * 4096 + (size_t)b * TRINV_COLS + 64 * TRINV_COLS) * sizeof(double) + 64 * sizeof(TrinvDiv);
+}
+// RN(z / l), l the divisor D was made from
+__device__ __forceinline__ double trinv_div(double z, double l, const TrinvDiv &D) {
+    const unsigned long long w = (unsigned long long)__double_as_longlong(z);
+    const int e = (int)(w >> 52) & 2047;
+    if (w == 0 && D.ok) return z;
+    if (!D.ok || e <= 400 || e >= 1646) return z / l;      // quotients stay normal in between
+    fx::Num h;
+    h.m = (w & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+    h.e = e - 1075;
+    fx::Divisor a;
+    a.m = D.m;
+    a.v = D.v;
+    a.e = D.e;
+    return __longlong_as_double(__double_as_longlong(fx::value(fx::div_rn(h, a))) | (long long)(w & (1ull << 63)));
+}
+// block (ib, jb) of L into S[column][row]
+__device__ __forceinline__ void trinv_load(double *S, const double *__restrict__ L, int b, int ib, int jb) {
+#pragma unroll 8
+    for (int i = threadIdx.x; i < 4096; i += TRINV_THREADS)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(S + i)),
+                     "l"(L + (int64_t)(jb * 64 + (i >> 6)) * b + ib * 64 + (i & 63))
+                     : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
 }
 // several tiles at once (grid.y = entry): the diagonal tiles of a batch's column
-__global__ void __launch_bounds__(256) k_trinv_batched(const TEntry *__restrict__ e, int b) {
-    const TEntry E = e[blockIdx.y];
-    trinv_body(E.L, b, E.Y);
+__global__ void __launch_bounds__(TRINV_THREADS) k_trinv_batched(const TEntry *__restrict__ e, int b) {
+    extern __shared__ double tsm[];
+    double *S = tsm;                                          // two 64 x 64 blocks of L
+    double *Ys = tsm + 2 * 4096;                              // the solved rows, column by column
+    double *Acc = Ys + (size_t)b * TRINV_COLS;                // one block's rows
+    TrinvDiv *Dv = reinterpret_cast<TrinvDiv *>(Acc + 64 * TRINV_COLS);
+    const double *__restrict__ L = e[blockIdx.y].L;
+    const int tid = threadIdx.x, r = tid & 63, cg = tid >> 6, warp = tid >> 5, lane = tid & 31;
+    const int c = blockIdx.x * TRINV_COLS + cg, ib0 = (int)blockIdx.x * TRINV_COLS / 64;
+    double *Y = e[blockIdx.y].Y + (int64_t)c * b, *Yc = Ys + (size_t)cg * b;
+    for (int i = r; i < ib0 * 64; i += 64) Y[i] = 0.0;
+    trinv_load(S, L, b, ib0, ib0);
+    int cur = 0;
+    for (int ib = ib0; ib < b / 64; ++ib) {
+        double a = (ib * 64 + r == c) ? 1.0 : 0.0;
+        for (int jb = ib0; jb <= ib; ++jb, cur ^= 1) {
+            const int ni = jb < ib ? ib : ib + 1, nj = jb < ib ? jb + 1 : ib0;
+            // the other buffer's readers passed the barrier that ended their step
+            if (ni < b / 64) {
+                trinv_load(S + (cur ^ 1) * 4096, L, b, ni, nj);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+            }
+            __syncthreads();
+            const double *B = S + cur * 4096;
+            if (jb < ib) {
+#pragma unroll 16
+                for (int l = 0; l < 64; ++l) a = fma(-B[l * 64 + r], Yc[jb * 64 + l], a);
+            } else {
+                Acc[cg * 64 + r] = a;
+                if (cg == 0) {
+                    const double d = B[r * 65];
+                    const int x = (int)((unsigned long long)__double_as_longlong(d) >> 52);     // sign included
+                    TrinvDiv D;
+                    D.ok = x > 400 && x < 1646;
+                    const fx::Divisor q = fx::make_divisor(D.ok ? d : 1.0);
+                    D.m = q.m;
+                    D.v = q.v;
+                    D.e = q.e;
+                    Dv[r] = D;
+                }
+                __syncthreads();
+                if (warp < TRINV_COLS) {
+                    double z0 = Acc[warp * 64 + lane], z1 = Acc[warp * 64 + lane + 32];
+                    for (int j = 0; j < 32; ++j) {
+                        const double y = trinv_div(__shfl_sync(0xffffffffu, z0, j), B[j * 65], Dv[j]);
+                        if (lane == j) z0 = y;
+                        if (lane > j) z0 = fma(-B[j * 64 + lane], y, z0);
+                        z1 = fma(-B[j * 64 + lane + 32], y, z1);
+                    }
+                    for (int j = 32; j < 64; ++j) {
+                        const double y = trinv_div(__shfl_sync(0xffffffffu, z1, j - 32), B[j * 65], Dv[j]);
+                        if (lane == j - 32) z1 = y;
+                        if (lane > j - 32) z1 = fma(-B[j * 64 + lane + 32], y, z1);
+                    }
+                    double *out = Ys + (size_t)warp * b + ib * 64;
+                    out[lane] = z0;
+                    out[lane + 32] = z1;
+                }
+                __syncthreads();
+                Y[ib * 64 + r] = Yc[ib * 64 + r];
+            }
+            __syncthreads();
+        }
+    }
 }
 
 // sum of log of the nv leading diagonal entries of one tile, fixed order, into *out
@@ -1547,14 +1605,12 @@ void launch_trsm_group(double *const *C, int ntiles, const double *L, int ld, in
 }
 void launch_trinv_columns(const TEntry *e, int n, int b, cudaStream_t s) {
     if (n <= 0) return;
-    const size_t smem = ((size_t)b * TRINV_COLS + 64 * 65 + 64 * TRINV_COLS) * sizeof(double);
     static std::atomic<unsigned long long> attr{0};
     if (attrs_pending(attr)) {     // sized for the largest tile it serves (b <= 2048)
-        cudaFuncSetAttribute(k_trinv_batched, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(((size_t)2048 * TRINV_COLS + 64 * 65 + 64 * TRINV_COLS) * sizeof(double)));
+        cudaFuncSetAttribute(k_trinv_batched, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)trinv_smem(2048));
         mark_attrs_set(attr);
     }
-    k_trinv_batched<<<dim3(b / (2 * TRINV_COLS), n), 256, smem, s>>>(e, b);
+    k_trinv_batched<<<dim3(b / TRINV_COLS, n), TRINV_THREADS, trinv_smem(b), s>>>(e, b);
 }
 void launch_logdiag_tile(const double *D, int b, int nv, double *out, cudaStream_t s) {
     k_logdiag_tile<<<1, 256, 0, s>>>(D, b, nv, out);
