@@ -46,6 +46,32 @@ __device__ __forceinline__ uint4 digit8(const uint32_t (&lo)[8], const uint32_t 
     }
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
+// RN((2^24 hi + lo) 2^e) in integer arithmetic: two 64-bit conversions, a product and a multiply-add
+// a value kept the FP64 pipe busy for 9000 cycles an item of k_zgemm.
+__device__ __forceinline__ double fixed_sum(long long hi, long long lo, int e) {
+    unsigned long long l = ((unsigned long long)hi << 24) + (unsigned long long)lo;
+    long long h = (hi >> 40) + (lo >> 63) + (l < (unsigned long long)lo ? 1 : 0);
+    const unsigned long long sign = (unsigned long long)h & (1ull << 63);
+    if (sign) {
+        l = 0 - l;
+        h = ~h + (l == 0 ? 1 : 0);
+    }
+    if ((h | (long long)l) == 0) return 0.0;
+    int x = 1022 + 127 + e;                             // biased exponent less one of a leading bit 127
+    if (h == 0) {
+        h = (long long)l;
+        l = 0;
+        x -= 64;
+    }
+    const int n = __clzll(h);
+    x -= n;
+    unsigned long long m = (unsigned long long)h << n;
+    if (n) m |= l >> (64 - n);
+    m |= (l << n) != 0 ? 1 : 0;                         // what lies below, for ties
+    const unsigned long long q = (m >> 11) + (((m & 2047) + 1023 + ((m >> 11) & 1)) >> 11);
+    if (x < 0 || x > 2044) return ldexp(sign ? -(double)q : (double)q, x - 1074);
+    return __longlong_as_double((long long)(sign | (((unsigned long long)x << 52) + q)));
+}
 __device__ __forceinline__ void biased8(const long long (&q)[8], uint32_t (&lo)[8], uint32_t (&hi)[8]) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) {

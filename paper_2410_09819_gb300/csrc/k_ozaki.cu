@@ -454,7 +454,6 @@ k_zgemm(const __grid_constant__ Args args) {
                 }
             }
             if (!ok) break;
-            const double s_hi = ldexp(1.0, E0 - 40), s_lo = ldexp(1.0, E0 - 64);
             const int row = it.bm * ZBM + quarter * 32 + lane;
             // all of C's values are requested before the first store, so the loads' latencies overlap
             // (one after another they cost 20000 cycles an item, which the MMAs then waited for)
@@ -464,7 +463,7 @@ k_zgemm(const __grid_constant__ Args args) {
             for (int j = 0; j < COLS; ++j) v[j] = args.assign ? 0.0 : c[(int64_t)j * b];
 #pragma unroll
             for (int j = 0; j < COLS; ++j) {
-                const double sum = fma((double)lo[j], s_lo, (double)hi[j] * s_hi);
+                const double sum = fixed_sum(hi[j], lo[j], E0 - 64);
                 c[(int64_t)j * b] = args.assign ? sum : v[j] - sum;
             }
         }
