@@ -11,9 +11,9 @@
 //
 // What bounds it: one right-hand side, the chain from block to block (counter and solution through
 // L2, one 64 x 64 product, the 64-step triangle); many, the FP64 pipe (n^2 / 2 multiply-adds a
-// sweep and column).  n = 32768, one column: 4.7 ms forward and 6.2 ms back, 9 and 12 us a block,
+// sweep and column).  n = 32768, one column: 4.4 ms forward and 4.7 ms back, 9 us a block,
 // where launches per tile with triangles of 256 rows in one CTA took 12.9 and 13.9 ms; n = 8192, 64
-// columns: 4.0 and 4.8 ms, where they took 24.3 and 26.4 ms.
+// columns: 4.0 and 4.2 ms, where they took 24.3 and 26.4 ms.
 #include "tc_internal.h"
 #include "zgemm_common.h"
 
@@ -110,6 +110,12 @@ k_sweep(const double *__restrict__ W, int b, int nblk, double *r, int64_t ldr, i
         double acc[NA];
 #pragma unroll
         for (int q = 0; q < NA; ++q) acc[q] = 0.0;
+        double u0 = 0.0, u1 = 0.0;                     // a warp per right-hand side: its rows of r
+        double *x = rg + (warp < nq ? warp : 0) * ldr + (int64_t)i * 64;
+        if (warp < nq) {
+            u0 = __ldcg(x + lane);
+            u1 = __ldcg(x + lane + 32);
+        }
         int have = 0;
         for (int t = 0; t < s; ++t) {
             const int j = FWD ? t : nblk - 1 - t;
@@ -180,19 +186,27 @@ k_sweep(const double *__restrict__ W, int b, int nblk, double *r, int64_t ldr, i
                 for (int c = 0; c < NQ; ++c) red[c * 4 + part][rr] = acc[c];
             }
         } else {
+            // sums over the lanes: in every step a lane hands on the half of its sums that the other
+            // lane keeps (9 additions a lane instead of 40 for one column, 31 instead of 160 for four,
+            // and an addition holds its SM quarter for 64 cycles)
 #pragma unroll
-            for (int q = 0; q < 8 * NQ; ++q) {
-                double v = acc[q];
+            for (int o = 16, n = 4 * NQ; o > 0; o >>= 1, n >>= 1) {
+                const bool up = lane & o;
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                if (lane == 0) red[(q % NQ) * 4][8 * warp + q / NQ] = v;
+                for (int q = 0; q < 4 * NQ; ++q)
+                    if (q < n) {
+                        const double send = up ? acc[q] : acc[q + n], keep = up ? acc[q + n] : acc[q];
+                        acc[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                    }
+                if (n == 0) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
             }
+            constexpr int LANES = 32 / (8 * NQ);
+            const int q = lane / LANES;
+            if (lane % LANES == 0) red[(q % NQ) * 4][8 * warp + q / NQ] = acc[0];
         }
         __syncthreads();
-        if (warp < nq) {                               // a warp per right-hand side
-            double *x = rg + warp * ldr + (int64_t)i * 64;
+        if (warp < nq) {
             const double(*rd)[64] = red + 4 * warp;
-            double u0 = __ldcg(x + lane), u1 = __ldcg(x + lane + 32);
             if (FWD) {
                 u0 -= (rd[0][lane] + rd[1][lane]) + (rd[2][lane] + rd[3][lane]);
                 u1 -= (rd[0][lane + 32] + rd[1][lane + 32]) + (rd[2][lane + 32] + rd[3][lane + 32]);
@@ -203,8 +217,8 @@ k_sweep(const double *__restrict__ W, int b, int nblk, double *r, int64_t ldr, i
             sweep_tri<FWD>(M, u0, u1);
             __stcg(x + lane, u0 * rinv[lane]);
             __stcg(x + lane + 32, u1 * rinv[lane + 32]);
-            __threadfence();
         }
+        // (the release below covers the stores that the barrier orders before it)
         if constexpr (NQ == 1) __syncwarp();
         else __syncthreads();
         if (tid == 0) asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(progress), "r"(s + 1) : "memory");
