@@ -172,7 +172,9 @@ struct ZArgs {
     const int *exps;
     int k, b;
     int *err;
-    int assign;         // 0: C -= sum X Y^T;  1: C = sum X Y^T
+    int assign;         // 0: C -= sum X Y^T;  1: C = sum X Y^T;  2: C = its counterpart in `add` + sum X Y^T
+    const ZItem *add;   // assign 2: items whose C holds the summand
+    double *amax;       // not null: largest |C| of the results of item it goes to amax[it.ct] (ct >= 0)
     int tri;            // 1: the Y tiles are lower triangular (row j is zero beyond column j)
     unsigned long long limit_ns;    // bound of each pipeline wait
     int stall;                      // test hook: wait first on a barrier nothing arrives at
@@ -183,6 +185,8 @@ struct ZArgs {
     }
     __device__ int xsrc(const ZItem &it, int n) const { return it.xoff + n; }
     __device__ int ysrc(const ZItem &it, int n) const { return it.yoff + n; }
+    __device__ const double *base(const ZItem &it, int i) const { return assign == 2 ? add[i].C : it.C; }
+    __device__ double *amax_of(const ZItem &it) const { return amax && it.ct >= 0 ? amax + it.ct : nullptr; }
 };
 
 // Out-of-core form: up to ZG_MAX output tiles of one tile column, whose sources sit in
@@ -215,6 +219,8 @@ struct ZGroupArgs {
     }
     __device__ int xsrc(const ZItem &it, int n) const { return xs[it.xoff][n]; }
     __device__ int ysrc(const ZItem &, int n) const { return ys[n]; }
+    __device__ const double *base(const ZItem &it, int) const { return it.C; }
+    __device__ double *amax_of(const ZItem &) const { return nullptr; }
 };
 
 // Stages of ZKE elements of K that item `it` multiplies per source: all of them, or with a lower
@@ -457,14 +463,24 @@ k_zgemm(const __grid_constant__ Args args) {
             const int row = it.bm * ZBM + quarter * 32 + lane;
             // all of C's values are requested before the first store, so the loads' latencies overlap
             // (one after another they cost 20000 cycles an item, which the MMAs then waited for)
-            double *c = it.C + (int64_t)(it.bn * ZBN + half * COLS) * b + row;
+            const int64_t o = (int64_t)(it.bn * ZBN + half * COLS) * b + row;
+            const double *src = args.base(it, item) + o;
+            double *c = it.C + o;
             double v[COLS];
 #pragma unroll
-            for (int j = 0; j < COLS; ++j) v[j] = args.assign ? 0.0 : c[(int64_t)j * b];
+            for (int j = 0; j < COLS; ++j) v[j] = args.assign == 1 ? 0.0 : src[(int64_t)j * b];
+            unsigned long long m = 0;                  // sign-cleared bit patterns order like |x|
 #pragma unroll
             for (int j = 0; j < COLS; ++j) {
                 const double sum = fixed_sum(hi[j], lo[j], E0 - 64);
-                c[(int64_t)j * b] = args.assign ? sum : v[j] - sum;
+                const double out = args.assign == 1 ? sum : args.assign == 2 ? v[j] + sum : v[j] - sum;
+                c[(int64_t)j * b] = out;
+                m = max(m, (unsigned long long)__double_as_longlong(out) & 0x7FFFFFFFFFFFFFFFull);
+            }
+            if (double *am = args.amax_of(it)) {
+#pragma unroll
+                for (int w = 16; w > 0; w >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, w));
+                if (lane == 0) atomicMax(reinterpret_cast<unsigned long long *>(am), m);
             }
         }
         if (!ok) {
@@ -503,15 +519,6 @@ __global__ void k_lower_only(double *T, int b) {
     const int64_t bb = (int64_t)b * b;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < bb; e += (int64_t)gridDim.x * blockDim.x)
         if (e % b < e / b) T[e] = 0.0;
-}
-
-// tile tiles[y] of W += the y-th tile of src
-__global__ void k_add_tiles(double *W, int b, const int *tiles, const double *src) {
-    const int64_t bb = (int64_t)b * b;
-    double *T = W + (int64_t)tiles[blockIdx.y] * bb;
-    const double *S = src + (int64_t)blockIdx.y * bb;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < bb; e += (int64_t)gridDim.x * blockDim.x)
-        T[e] += S[e];
 }
 
 __global__ void k_set_identity(double *T, int b) {
@@ -568,10 +575,6 @@ __global__ void k_add_tile(double *dst, const double *src, int64_t count) {
 void launch_add_tile(double *dst, const double *src, int b, cudaStream_t s) {
     k_add_tile<<<608, 256, 0, s>>>(dst, src, (int64_t)b * b);
 }
-void launch_add_tiles(double *W, int b, const int *tiles, int ntiles, const double *src, cudaStream_t s) {
-    if (ntiles > 0) k_add_tiles<<<dim3(64, ntiles), 256, 0, s>>>(W, b, tiles, src);
-}
-
 // P planes of base 256 are worth 2P base-16 digits: they round an operand to 2^-(8P+1) of its
 // scale, and the pairs they leave out stay below 2^-(8P) of the product's.
 template <class Args>
@@ -596,9 +599,9 @@ static void launch_form(int planes, const Args &a, int nitems, cudaStream_t s) {
 
 void launch_zgemm(const uint8_t *pool, const ZItem *items, int nitems, const int *exps, int k,
                   int b, int *err, cudaStream_t s, int planes, int assign, int tri, unsigned long long limit_ns,
-                  int stall) {
+                  int stall, double *amax, const ZItem *add) {
     if (nitems <= 0 || k <= 0) return;
-    const ZArgs a{pool, items, nitems, exps, k, b, err, assign, tri, limit_ns ? limit_ns : ZLIMIT_NS, stall};
+    const ZArgs a{pool, items, nitems, exps, k, b, err, assign, add, amax, tri, limit_ns ? limit_ns : ZLIMIT_NS, stall};
     launch_form(planes, a, nitems, s);
 }
 

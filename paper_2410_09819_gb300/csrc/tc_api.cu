@@ -194,7 +194,8 @@ Plan build_plan(tc_handle h, double *W, int *status) {
                         double *Cp = T(M, m, k);
                         const int xo = (int)(M.tile0 + tidx(m, 0)), yo = (int)(M.tile0 + tidx(k, 0));
                         int items = 0;
-                        const int ct = (int)(M.tile0 + tidx(m, k));
+                        // (all-FP64: the diagonal tile's amax slot belongs to its inverse)
+                        const int ct = m == k && !M.mixed ? -1 : (int)(M.tile0 + tidx(m, k));
                         for_tile_items(b, m == k, [&](int bm, int bn) {
                             P.zitems.push_back({Cp, xo, yo, (uint16_t)bm, (uint16_t)bn, ct});
                             ++items;
@@ -259,10 +260,10 @@ Plan build_plan(tc_handle h, double *W, int *status) {
                 const int sx = (int)(M.tile0 + tidx(m, k));
                 // mixed maps: the products run on the 128 x 64 kernel (fixed plane counts)
                 for_tile_items(b, false, [&](int bm, int bn) {
-                    P.zinv.push_back({Cp, sx, sinv, (uint16_t)bm, (uint16_t)bn});
+                    P.zinv.push_back({Cp, sx, sinv, (uint16_t)bm, (uint16_t)bn, sx});
                     if (P.inv_refine) {
-                        P.zinvc.push_back({Cs, sx, sinv, (uint16_t)bm, (uint16_t)bn});
-                        P.zref.push_back({Cp, sx, sl, (uint16_t)bm, (uint16_t)bn});
+                        P.zinvc.push_back({Cs, sx, sinv, (uint16_t)bm, (uint16_t)bn, sx});
+                        P.zref.push_back({Cp, sx, sl, (uint16_t)bm, (uint16_t)bn, sx});
                     }
                 }, P.inv_refine ? Z_BN : zw);
                 C.nvp[p] += (int)(P.zinv.size() - before);
@@ -677,7 +678,7 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
                                wait_limit_ns(h), wait_test(h));
             else
                 launch_zgemm(static_cast<const uint8_t *>(h->dpool.p), D.zitems + C.z0, C.nz, D.zexps, k, b, status + 1, h->s, 14, 0, 0,
-                             wait_limit_ns(h), wait_test(h));
+                             wait_limit_ns(h), wait_test(h), P.inv_refine ? D.zamax2 : nullptr);
             span_end(h, sp);
             CK_LAUNCH();
             ++h->upd_launches[TC_FP64];
@@ -736,8 +737,10 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
                 launch_digits_src(inv, b, 1, gkk, D.zamax2 + gkk, pool, D.zexps, h->s, e4m3);
                 CK_LAUNCH();
             }
-            launch_tile_amax(W, b, D.dtiles + C.dg0, C.ndg, D.zamax2, h->s);
-            CK_LAUNCH();
+            if (!P.inv_refine || !C.nz) {          // else the column's update has left its tiles' amax
+                launch_tile_amax(W, b, D.dtiles + C.dg0, C.ndg, D.zamax2, h->s);
+                CK_LAUNCH();
+            }
             launch_digits(W, b, D.dtiles + C.dg0, C.ndg, D.zamax2, pool, D.zexps, h->s, e4m3);
             CK_LAUNCH();
             if (!P.inv_refine) {
@@ -764,23 +767,17 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
                 launch_digits_src(Lkk, b, 0, gl, am_l + gl, pool, D.zexps, h->s);
                 CK_LAUNCH();
                 launch_zgemm(static_cast<const uint8_t *>(h->dpool.p), D.zinvc + C.v0, C.nv, D.zexps, 1, b, status + 1, h->s, 14, 1, 1,
-                             wait_limit_ns(h), wait_test(h));
-                CK_LAUNCH();
-                launch_tile_amax(W, b, D.dtiles + C.dg0, C.ndg, am_x, h->s, X0);
+                             wait_limit_ns(h), wait_test(h), am_x);
                 CK_LAUNCH();
                 launch_digits(W, b, D.dtiles + C.dg0, C.ndg, am_x, pool, D.zexps, h->s, false, X0);
                 CK_LAUNCH();
                 launch_zgemm(static_cast<const uint8_t *>(h->dpool.p), D.zref + C.v0, C.nv, D.zexps, 1, b, status + 1, h->s, 14, 0, 1,
-                             wait_limit_ns(h), wait_test(h));
-                CK_LAUNCH();
-                launch_tile_amax(W, b, D.dtiles + C.dg0, C.ndg, am_r, h->s);
+                             wait_limit_ns(h), wait_test(h), am_r);
                 CK_LAUNCH();
                 launch_digits(W, b, D.dtiles + C.dg0, C.ndg, am_r, pool, D.zexps, h->s, false);
                 CK_LAUNCH();
-                launch_zgemm(static_cast<const uint8_t *>(h->dpool.p), D.zinv + C.v0, C.nv, D.zexps, 1, b, status + 1, h->s, ZREF_PLANES, 1, 1,
-                             wait_limit_ns(h), wait_test(h));
-                CK_LAUNCH();
-                launch_add_tiles(W, b, D.dtiles + C.dg0, C.ndg, X0, h->s);
+                launch_zgemm(static_cast<const uint8_t *>(h->dpool.p), D.zinv + C.v0, C.nv, D.zexps, 1, b, status + 1, h->s, ZREF_PLANES, 2, 1,
+                             wait_limit_ns(h), wait_test(h), D.zamax, D.zinvc + C.v0);
                 CK_LAUNCH();
             }
             span_end(h, sp);
@@ -797,8 +794,10 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
         }
         if (C.ndg) {
             const int sp = spans ? span_begin(h, CAT_CONVERT) : -1;
-            launch_tile_amax(W, b, D.dtiles + C.dg0, C.ndg, D.zamax, h->s);
-            CK_LAUNCH();
+            if (!P.inv_refine) {                   // else the last product has left the amax
+                launch_tile_amax(W, b, D.dtiles + C.dg0, C.ndg, D.zamax, h->s);
+                CK_LAUNCH();
+            }
             launch_digits(W, b, D.dtiles + C.dg0, C.ndg, D.zamax, static_cast<uint8_t *>(h->dpool.p), D.zexps, h->s, e4m3);
             span_end(h, sp);
             CK_LAUNCH();

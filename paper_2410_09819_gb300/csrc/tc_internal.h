@@ -270,17 +270,17 @@ size_t zgemm_smem_bytes();
 void launch_digits(const double *W, int b, const int *tiles, int ntiles, const double *amax, uint8_t *pool, int *exps,
                    cudaStream_t s, bool e4m3, const double *alt = nullptr);
 void launch_lower_only(double *T, int b, cudaStream_t s);
-void launch_add_tiles(double *W, int b, const int *tiles, int ntiles, const double *src, cudaStream_t s);
 void launch_add_tile(double *dst, const double *src, int b, cudaStream_t s);     // dst += src, one b x b tile
 // Products on base-256 planes.  planes: base-16 digits that the result is to be worth (14 FP64,
-// 10 FP32 outputs, fewer for TRSM products); assign: C = sum X Y^T instead of C -= it; tri: the
+// 10 FP32 outputs, fewer for TRSM products); assign: C -= sum X Y^T (0), C = it (1), C = the item's
+// counterpart in `add` + it (2); amax: the largest |C| of each item's tile (slot ct); tri: the
 // Y tiles are lower triangular; limit_ns: bound of each pipeline wait (0: 4 s), after which *err
 // is set and the call ends; stall != 0: the failure-detection test hook (the MMA issuer waits on
 // a barrier nothing arrives at).
 // pool: the digit planes, slot t (7 planes of b x b FP16 values, k_ozaki.cu) at 14 t b^2 bytes.
 void launch_zgemm(const uint8_t *pool, const ZItem *items, int nitems, const int *exps, int k,
                   int b, int *err, cudaStream_t s, int planes, int assign, int tri, unsigned long long limit_ns,
-                  int stall);
+                  int stall, double *amax = nullptr, const ZItem *add = nullptr);
 void launch_zgemm_group(const uint8_t *pool, const ZGroup &g, const int *exps, int b, int *err,
                         cudaStream_t s, int planes, int tri, unsigned long long limit_ns, int stall);
 // Plane counts of a mixed-precision update launch (k_zgemm64): per source, the X / Y planes its
