@@ -24,7 +24,6 @@ FIXED_FN uint64_t mulhi(uint64_t a, uint64_t b) { return __umul64hi(a, b); }
 FIXED_FN int64_t mulhi_s(int64_t a, int64_t b) { return __mul64hi(a, b); }
 FIXED_FN uint32_t mulhi32(uint32_t a, uint32_t b) { return __umulhi(a, b); }
 FIXED_FN float rsqrt_f(float x) { return rsqrtf(x); }
-FIXED_FN float rcp_f(float x) { return __frcp_rn(x); }
 FIXED_FN uint32_t to_u32(float x) { return __float2uint_rz(x); }          // saturates
 FIXED_FN uint64_t bits(double x) { return (uint64_t)__double_as_longlong(x); }
 FIXED_FN double from_bits(uint64_t w) { return __longlong_as_double((long long)w); }
@@ -33,7 +32,6 @@ FIXED_FN uint64_t mulhi(uint64_t a, uint64_t b) { return (uint64_t)(((unsigned _
 FIXED_FN int64_t mulhi_s(int64_t a, int64_t b) { return (int64_t)(((__int128)a * b) >> 64); }
 FIXED_FN uint32_t mulhi32(uint32_t a, uint32_t b) { return (uint32_t)(((uint64_t)a * b) >> 32); }
 FIXED_FN float rsqrt_f(float x) { return 1.0f / sqrtf(x); }
-FIXED_FN float rcp_f(float x) { return 1.0f / x; }
 FIXED_FN uint32_t to_u32(float x) { return x >= 4294967296.0f ? 0xFFFFFFFFu : (uint32_t)x; }
 FIXED_FN uint64_t bits(double x) { uint64_t w; memcpy(&w, &x, 8); return w; }
 FIXED_FN double from_bits(uint64_t w) { double x; memcpy(&x, &w, 8); return x; }
@@ -79,29 +77,56 @@ FIXED_FN Num sqrt_rn(double s) {
     return {h, e};
 }
 
-// RN(1 / h): two Newton steps on an FP32 reciprocal to v = 2^116 / m, 64 bits to a few units, and
-// where the bits below the result leave the rounding open the product of the boundary decides.
-FIXED_FN Num recip_rn(const Num &h) {
-    if (h.m == 1ull << 52) return {1ull << 52, -104 - h.e};
-    const uint64_t X = h.m << 11;                       // v = 2^127 / X
-    const uint32_t V0 = to_u32(rcp_f((float)(uint32_t)(X >> 32)) * 9223372036854775808.0f);
-    const uint64_t P = (X >> 32) * V0 + (((X & 0xFFFFFFFFull) * V0) >> 32);
-    const int64_t E = (int64_t)((1ull << 63) - P);      // 2^63 (1 - X V0 2^-95)
-    const uint64_t V1 = ((uint64_t)V0 << 32) + (uint64_t)(((int64_t)(E >> 12) * (int64_t)V0) >> 19);
-    const int64_t E1 = (int64_t)((1ull << 63) - mulhi(X, V1));
-    const uint64_t V = V1 + (uint64_t)(((int64_t)(V1 >> 32) * E1) >> 31);
-    uint64_t q = (V >> 11) + ((V >> 10) & 1);
-    const int low = (int)(V & 2047);
-    if (low >= 1008 && low < 1040) {
-        const uint64_t t = 2 * (V >> 11) + 1;           // t m against 2^106, modulo 2^64
-        q = (V >> 11) + ((int64_t)(0 - t * h.m) > 0 ? 1 : 0);
+// RN(sqrt(s)) and RN(1 / RN(sqrt(s))) of a positive normal number together: the correction that turns
+// W into a square root turns Y into its reciprocal as well, R = 2^89 / sqrt(m); what rounding adds to
+// the root then moves the reciprocal by R^2 2^-125 times as much.
+FIXED_FN void sqrt_recip_rn(double s, Num &root, Num &recip) {
+    const uint64_t w = bits(s);
+    int e = (int)(w >> 52) - 1075;
+    uint64_t m = (w & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+    if (e & 1) {
+        m <<= 1;
+        --e;
     }
-    int e = -105 - h.e;
-    if (q >> 53) {
-        q >>= 1;
+    const uint32_t Y = to_u32(rsqrt_f((float)(uint32_t)(m >> 22)) * 140737488355328.0f);    // 2^47
+    const uint64_t A = m << 10;
+    const uint64_t P = (A >> 32) * Y + (((A & 0xFFFFFFFFull) * Y) >> 32);
+    const uint64_t Q = (P >> 32) * Y + (((P & 0xFFFFFFFFull) * Y) >> 32);
+    const int64_t E = (int64_t)((1ull << 62) - Q);
+    const int32_t E21 = (int32_t)(E >> 21);
+    const int64_t E2 = (E >> 1) + (((((int64_t)E21 * E21) >> 20) * 3) >> 3);
+    const uint64_t W = P + (uint64_t)(mulhi_s((int64_t)(P >> 1), E2 << 20) >> 17);
+    const uint64_t R = ((uint64_t)Y << 31) + (uint64_t)mulhi_s((int64_t)((uint64_t)Y << 31), E2 << 2);
+    const uint32_t S = (uint32_t)(((R >> 32) * (R >> 32)) >> 31);
+    uint64_t h = (W + 512) >> 10;
+    const int low = (int)(W & 1023);
+    if (low >= 496 && low < 528) {
+        const uint64_t t = 2 * (W >> 10) + 1;           // the boundary, and its distance modulo 2^64
+        h = (W >> 10) + ((int64_t)((m << 54) - t * t) > 0 ? 1 : 0);
+    }
+    const uint64_t V = R - (uint64_t)(((int64_t)S * (int32_t)((h << 10) - W)) >> 30);
+    e = e / 2 - 26;                                     // sqrt(s) = W 2^-36 2^(e/2), h = W 2^-10
+    if (h >> 53) {
+        h >>= 1;
         ++e;
     }
-    return {q, e};
+    root = {h, e};
+    uint64_t q = (V >> 10) + ((V >> 9) & 1);
+    const int lowv = (int)(V & 1023);
+    if (lowv >= 496 && lowv < 528) {
+        const uint64_t t = 2 * (V >> 10) + 1;           // t h against 2^106, modulo 2^64
+        q = (V >> 10) + ((int64_t)(0 - t * h) > 0 ? 1 : 0);
+    }
+    int er = -105 - e;
+    if (q >> 53) {
+        q >>= 1;
+        ++er;
+    }
+    if (h == 1ull << 52) {
+        q = 1ull << 52;
+        er = -104 - e;
+    }
+    recip = {q, er};
 }
 
 // Division by a fixed a = m 2^e: v = floor(2^116 / m), at most 2^64 - 1.

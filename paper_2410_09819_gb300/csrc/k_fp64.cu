@@ -106,12 +106,14 @@ k_dgemm_reduce(const DRed *__restrict__ reds, int ld, const double *__restrict__
 // lanes are active.  So warps 0 and 1 run the chain, a thread per row with its element of the
 // current column in a register: the pivot's root and its reciprocal in integer arithmetic
 // (fixed_exp.h: the same correctly rounded values), one multiplication, one barrier, one
-// multiply-add for the next column; warps 2 to 5 meanwhile take the previous step to the columns
+// multiply-add for the next column; warps 2 to 9 meanwhile take the previous step to the columns
 // behind, through an element list in column order in which a finished column costs nothing.  Every
-// element sees the same operations in the same order as in the plain loop.   A block took 94 us with a
+// element sees the same operations in the same order as in the plain loop.  A block took 94 us with a
 // square root, a division and three barriers of 256 threads a step, 73 us with two barriers and
-// FP64 comparisons on the chain, 52 us here.
-constexpr int POTRF_THREADS = 192;
+// FP64 comparisons on the chain, 52 us with the reciprocal's own Newton steps after the root and four
+// warps on the rest, 38 us here (of a step's 1100 cycles the root and reciprocal take 490; a warp
+// of its own for them, with named barriers, gains 5 %).
+constexpr int POTRF_THREADS = 320;
 __device__ __forceinline__ bool positive(double d) {       // d > 0 without the FP64 pipe
     const long long w = __double_as_longlong(d);
     return w > 0 && w <= 0x7FF0000000000000ll;
@@ -119,9 +121,10 @@ __device__ __forceinline__ bool positive(double d) {       // d > 0 without the 
 __device__ __forceinline__ void pivot_root(double d, double &sd, double &rp) {
     const int e = __double2hiint(d) >> 20;
     if (e > 100 && e < 1946) {
-        const fx::Num h = fx::sqrt_rn(d);
+        fx::Num h, q;
+        fx::sqrt_recip_rn(d, h, q);
         sd = fx::value(h);
-        rp = fx::value(fx::recip_rn(h));
+        rp = fx::value(q);
     } else {
         sd = sqrt(d);
         rp = 1.0 / sd;
