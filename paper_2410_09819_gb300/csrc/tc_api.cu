@@ -1302,12 +1302,8 @@ int tile_chol_solve(tc_handle h, int nrhs, const double *B, int64_t ldb, double 
     for (;; ++it) {
         if (max_refine == 0) break;
         // R = B - A X and the normwise backward error per column
-        for (int c0 = 0; c0 < nrhs; c0 += 16) {
-            const int nc = std::min(16, nrhs - c0);
-            launch_symv_resid(h->A_dev, nt, b, n, Xd + (int64_t)c0 * ldr, ldr, Bd + (int64_t)c0 * ldr, ldr,
-                              Rd + (int64_t)c0 * ldr, ldr, nc, 0, h->s);
-            CK_LAUNCH();
-        }
+        launch_symv_resid(h->A_dev, nt, b, n, Xd, ldr, Bd, ldr, Rd, ldr, nrhs, 0, h->s);
+        CK_LAUNCH();
         CK(cudaMemsetAsync(sc, 0, 3 * nrhs * sizeof(double), h->s));
         launch_colmax_abs(Rd, ldr, n, nrhs, sc, h->s);
         CK_LAUNCH();
