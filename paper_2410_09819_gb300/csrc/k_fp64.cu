@@ -549,62 +549,6 @@ __device__ __forceinline__ void bwd_diag_body(const double *L, int ld, int b, T 
     }
 }
 
-// Inside a diagonal tile, after a sub-block solve: R[r] -= sum_c L[c ld + r] Z[c] for the
-// `rows` rows below the sub-block (one CTA per 64 rows, four partial sums per row).
-template <int NQ>
-__global__ void __launch_bounds__(256)
-k_gemv_below(const double *L, int ld, int cols, const double *Z, double *R, int64_t ldr, int nrhs) {
-    __shared__ double red[64][17];
-    const int tid = threadIdx.x, rr = tid & 63, part = tid >> 6, r0 = blockIdx.x * 64;
-    double acc[NQ];
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) acc[q] = 0.0;
-    for (int c = part; c < cols; c += 4) {
-        const double l = L[(int64_t)c * ld + r0 + rr];
-#pragma unroll
-        for (int q = 0; q < NQ; ++q)
-            if (q < nrhs) acc[q] = fma(l, Z[q * ldr + c], acc[q]);
-    }
-    part_reduce_sub(red, acc, nrhs, R, ldr, r0);
-}
-
-// The back-substitution counterpart: R[i] -= sum_c L[i ld + c] X[c] for the rows above the
-// sub-block (L points at the sub-block's first row, column 0; a warp per output row, lanes
-// along c, so each row of L^T is read contiguously).
-template <int NQ>
-__global__ void __launch_bounds__(256)
-k_gemv_above(const double *L, int ld, int cols, const double *X, double *R, int64_t ldr, int nrhs) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int i = blockIdx.x * 64 + warp; i < blockIdx.x * 64 + 64; i += 8) {
-        double acc[NQ];
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) acc[q] = 0.0;
-        for (int c = lane; c < cols; c += 32) {
-            const double l = L[(int64_t)i * ld + c];
-#pragma unroll
-            for (int q = 0; q < NQ; ++q)
-                if (q < nrhs) acc[q] = fma(l, X[q * ldr + c], acc[q]);
-        }
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            double v = acc[q];
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0 && q < nrhs) R[q * ldr + i] -= v;
-        }
-    }
-}
-
-// Forward substitution with the s x s lower triangle at L (leading dimension ld): L z = r for
-// each RHS column (one CTA each).
-__global__ void __launch_bounds__(256) k_fwd_diag(const double *L, int ld, int b, double *R, int64_t ldr) {
-    fwd_diag_body(L, ld, b, R + blockIdx.x * ldr);
-}
-
-// Back substitution with the s x s lower triangle at L: L^T x = z for each RHS column.
-__global__ void __launch_bounds__(256) k_bwd_diag(const double *L, int ld, int b, double *R, int64_t ldr) {
-    bwd_diag_body(L, ld, b, R + blockIdx.x * ldr);
-}
-
 // R = B - A X (absmode 0) or R = |A| X (absmode 1, B unused) for the symmetric A held as
 // lower tiles; rows and columns >= n (padding) contribute nothing and R's padding is 0.  A CTA takes
 // 64 rows and one of the groups of NQ columns; the groups of the same rows are neighbours and
@@ -1271,28 +1215,6 @@ void launch_fix_padding(double *W, int nt, int b, int64_t n, cudaStream_t s) {
 void launch_zero_upper_diag(double *W, int nt, int b, int64_t n, cudaStream_t s) {
     k_zero_upper_diag<<<dim3(64, (n % b) ? 2 * nt - 1 : nt), 256, 0, s>>>(W, nt, b, n);
 }
-// A diagonal tile's substitution in sub-blocks of DIAG_SUB rows: a one-CTA triangular solve
-// per sub-block, then a many-CTA product with the rest of its columns (the one-CTA part,
-// bound by a single SM's FP64 rate, shrinks from b^2/2 to b DIAG_SUB/2 multiply-adds).
-constexpr int DIAG_SUB = 256;
-void launch_fwd_diag(const double *Ljj, int b, double *R, int64_t ldr, int nrhs, cudaStream_t s) {
-    const int S = (b % DIAG_SUB) ? b : DIAG_SUB;     // tiles not a multiple of it: one block
-    for (int sb = 0; sb < b / S; ++sb) {
-        k_fwd_diag<<<nrhs, 256, 0, s>>>(Ljj + (int64_t)sb * S * b + sb * S, b, S, R + sb * S, ldr);
-        const int rows = b - (sb + 1) * S;
-        if (rows > 0)
-            NQ_DISPATCH(nrhs, k_gemv_below, rows / 64, 256, 0, s, Ljj + (int64_t)sb * S * b + (sb + 1) * S, b, S,
-                        R + sb * S, R + (sb + 1) * S, ldr, nrhs);
-    }
-}
-void launch_bwd_diag(const double *Ljj, int b, double *R, int64_t ldr, int nrhs, cudaStream_t s) {
-    const int S = (b % DIAG_SUB) ? b : DIAG_SUB;     // tiles not a multiple of it: one block
-    for (int sb = b / S - 1; sb >= 0; --sb) {
-        k_bwd_diag<<<nrhs, 256, 0, s>>>(Ljj + (int64_t)sb * S * b + sb * S, b, S, R + sb * S, ldr);
-        if (sb > 0)
-            NQ_DISPATCH(nrhs, k_gemv_above, sb * S / 64, 256, 0, s, Ljj + sb * S, b, S, R + sb * S, R, ldr, nrhs);
-    }
-}
 void launch_symv_resid(const double *A, int nt, int b, int64_t n, const double *X, int64_t ldx,
                        const double *B, int64_t ldb, double *R, int64_t ldr, int nrhs, int absmode,
                        cudaStream_t s) {
@@ -1544,64 +1466,76 @@ __global__ void k_fix_padding_tile(double *T, int b, int nv, int diag) {
     }
 }
 
-// r_i -= L_ij z_j for one tile L_ij (ptr), rows of tile row i; grid = b/64 chunks
+// r_i -= L_ij z_j for one tile L_ij (ptr).  What bounds these two: reading the tile, if enough CTAs
+// share it.  16 rows a CTA (a column's 128 bytes at a time), 16 threads a row, each with its next
+// eight elements in flight while z is staged; backwards a warp per row of L^T.  A tile
+// of 1024, one column: forward 39 us with 64 rows a CTA, 12.5 us here; backward 62 us with 64 rows
+// staged in shared memory.
+constexpr int TU_ROWS = 16, TU_COLS = 128;
 template <int NQ>
 __global__ void __launch_bounds__(256)
 k_fwd_update_tile(const double *L, int b, int i, int j, double *R, int64_t ldr, int nrhs) {
-    __shared__ double zs[128][16];
-    __shared__ double red[64][17];
-    const int r0 = blockIdx.x * 64;
-    const int tid = threadIdx.x, rr = tid & 63, part = tid >> 6;
+    __shared__ double buf[16 * NQ * (TU_ROWS + 1)];
+    double(*zs)[NQ] = reinterpret_cast<double(*)[NQ]>(buf);                                    // TU_COLS rows of z, then
+    double(*red)[NQ][TU_ROWS + 1] = reinterpret_cast<double(*)[NQ][TU_ROWS + 1]>(buf);         // the 16 parts' sums
+    static_assert(TU_COLS <= 16 * (TU_ROWS + 1), "z fits their place");
+    const int r0 = blockIdx.x * TU_ROWS;
+    const int tid = threadIdx.x, rr = tid & 15, part = tid >> 4;
     double acc[NQ];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) acc[q] = 0.0;
-    for (int c0 = 0; c0 < b; c0 += 128) {
-        __syncthreads();
-        for (int e = tid; e < 128 * nrhs; e += 256) {
-            const int c = e % 128, q = e / 128;
-            zs[c][q] = R[q * ldr + (int64_t)j * b + c0 + c];
-        }
-        __syncthreads();
-        for (int c = part; c < 128; c += 4) {
-            const double l = L[(int64_t)(c0 + c) * b + r0 + rr];
+    for (int c0 = 0; c0 < b; c0 += TU_COLS) {
+        const int nc = min(TU_COLS, b - c0);
+        double l[TU_COLS / 16];
 #pragma unroll
-            for (int q = 0; q < NQ; ++q)
-                if (q < nrhs) acc[q] = fma(l, zs[c][q], acc[q]);
+        for (int u = 0; u < TU_COLS / 16; ++u)
+            l[u] = part + 16 * u < nc ? L[(int64_t)(c0 + part + 16 * u) * b + r0 + rr] : 0.0;
+        __syncthreads();
+        for (int e = tid; e < TU_COLS * NQ; e += 256) {
+            const int c = e % TU_COLS, q = e / TU_COLS;
+            zs[c][q] = c < nc && q < nrhs ? R[q * ldr + (int64_t)j * b + c0 + c] : 0.0;
         }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < TU_COLS / 16; ++u)
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) acc[q] = fma(l[u], zs[part + 16 * u][q], acc[q]);
     }
-    part_reduce_sub(red, acc, nrhs, R, ldr, (int64_t)i * b + r0);
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) red[part][q][rr] = acc[q];
+    __syncthreads();
+    for (int e = tid; e < TU_ROWS * nrhs; e += 256) {
+        const int r = e % TU_ROWS, q = e / TU_ROWS;
+        double sum = 0.0;
+#pragma unroll
+        for (int p = 0; p < 16; ++p) sum += red[p][q][r];
+        R[q * ldr + (int64_t)i * b + r0 + r] -= sum;
+    }
 }
 
-// z_i -= L_ji^T x_j for one tile L_ji (ptr); grid = b/64 chunks of tile row i
+// z_i -= L_ji^T x_j for one tile L_ji (ptr)
 template <int NQ>
 __global__ void __launch_bounds__(256)
 k_bwd_update_tile(const double *L, int b, int i, int j, double *R, int64_t ldr, int nrhs) {
-    __shared__ double xs[64][16];
-    __shared__ double S[64][65];
-    const int r0 = blockIdx.x * 64;
-    const int tid = threadIdx.x, rr = tid & 63, part = tid >> 6;
+    const int lane = threadIdx.x & 31, r = blockIdx.x * 8 + (threadIdx.x >> 5);
+    const double *l = L + (int64_t)r * b, *x = R + (int64_t)j * b;
     double acc[NQ];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) acc[q] = 0.0;
-    for (int c0 = 0; c0 < b; c0 += 64) {
-        __syncthreads();
-        for (int idx = tid; idx < 4096; idx += 256) {
-            const int c = idx & 63, r = idx >> 6;
-            S[r][c] = L[(int64_t)(r0 + r) * b + c0 + c];
-        }
-        for (int e = tid; e < 64 * nrhs; e += 256) {
-            const int c = e % 64, q = e / 64;
-            xs[c][q] = R[q * ldr + (int64_t)j * b + c0 + c];
-        }
-        __syncthreads();
-        for (int c = part; c < 64; c += 4) {
-            const double l = S[rr][c];
+#pragma unroll 8
+    for (int c = lane; c < b; c += 32) {
+        const double v = l[c];
 #pragma unroll
-            for (int q = 0; q < NQ; ++q)
-                if (q < nrhs) acc[q] = fma(l, xs[c][q], acc[q]);
-        }
+        for (int q = 0; q < NQ; ++q)
+            if (q < nrhs) acc[q] = fma(v, __ldcg(x + q * ldr + c), acc[q]);
     }
-    part_reduce_sub(reinterpret_cast<double(*)[17]>(&S[0][0]), acc, nrhs, R, ldr, (int64_t)i * b + r0);
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+        if (lane == 0 && q < nrhs) R[q * ldr + (int64_t)i * b + r] -= acc[q];
+    }
 }
 
 void launch_dgemm_tile(const DJob &job, int ld, cudaStream_t s) {
@@ -1643,10 +1577,10 @@ void launch_fix_padding_tile(double *T, int b, int nv, int diag, cudaStream_t s)
     k_fix_padding_tile<<<64, 256, 0, s>>>(T, b, nv, diag);
 }
 void launch_fwd_update_tile(const double *L, int b, int i, int j, double *R, int64_t ldr, int nrhs, cudaStream_t s) {
-    NQ_DISPATCH(nrhs, k_fwd_update_tile, b / 64, 256, 0, s, L, b, i, j, R, ldr, nrhs);
+    NQ_DISPATCH(nrhs, k_fwd_update_tile, b / TU_ROWS, 256, 0, s, L, b, i, j, R, ldr, nrhs);
 }
 void launch_bwd_update_tile(const double *L, int b, int i, int j, double *R, int64_t ldr, int nrhs, cudaStream_t s) {
-    NQ_DISPATCH(nrhs, k_bwd_update_tile, b / 64, 256, 0, s, L, b, i, j, R, ldr, nrhs);
+    NQ_DISPATCH(nrhs, k_bwd_update_tile, b / 8, 256, 0, s, L, b, i, j, R, ldr, nrhs);
 }
 
 }  // namespace tc

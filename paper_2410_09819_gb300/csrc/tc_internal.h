@@ -168,8 +168,6 @@ int launch_sweep(const double *W, int b, int nblk, double *r, int64_t ldr, int n
                  cudaStream_t s, unsigned long long limit_ns);
 
 // solves (column-major right-hand sides, leading dimension ldr, nrhs <= 16 per launch)
-void launch_fwd_diag(const double *Ljj, int b, double *R, int64_t ldr, int nrhs, cudaStream_t s);
-void launch_bwd_diag(const double *Ljj, int b, double *R, int64_t ldr, int nrhs, cudaStream_t s);
 void launch_symv_resid(const double *A, int nt, int b, int64_t n, const double *X, int64_t ldx,
                        const double *B, int64_t ldb, double *R, int64_t ldr, int nrhs, int absmode,
                        cudaStream_t s);

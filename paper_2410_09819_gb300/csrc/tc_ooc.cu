@@ -817,12 +817,14 @@ int ooc_subst(tc_handle h, double *R, int64_t ldr, int nrhs, bool back, int64_t 
     TileCache C;
     int rc = init_cache(h, C, h->host_factor, nt, b, false);
     if (rc) return rc;
+    int *err = static_cast<int *>(h->sweep.p), *progress = err + 1;      // (the caller clears and reads err)
     for (int c0 = 0; c0 < nrhs; c0 += 16) {
         const int nc = std::min(16, nrhs - c0);
         double *Rc = R + (int64_t)c0 * ldr;
         for (int j = 0; j < nt; ++j) {
             ACQ(sd, (int)tidx(j, j), true);
-            launch_fwd_diag(C.ptr(sd), b, Rc + (int64_t)j * b, ldr, nc, h->s);
+            CK((cudaError_t)launch_sweep(C.ptr(sd), b, b / 64, Rc + (int64_t)j * b, ldr, nc, true, progress, err, h->s,
+                                         wait_limit_ns(h)));
             CK_LAUNCH();
             C.touched(sd);
             for (int i = j + 1; i < nt; ++i) {
@@ -835,7 +837,8 @@ int ooc_subst(tc_handle h, double *R, int64_t ldr, int nrhs, bool back, int64_t 
         if (!back) continue;
         for (int j = nt - 1; j >= 0; --j) {
             ACQ(sd, (int)tidx(j, j), true);
-            launch_bwd_diag(C.ptr(sd), b, Rc + (int64_t)j * b, ldr, nc, h->s);
+            CK((cudaError_t)launch_sweep(C.ptr(sd), b, b / 64, Rc + (int64_t)j * b, ldr, nc, false, progress, err, h->s,
+                                         wait_limit_ns(h)));
             CK_LAUNCH();
             C.touched(sd);
             for (int i = 0; i < j; ++i) {
