@@ -4,6 +4,7 @@
 // (~1.05 TFLOP/s for the chip), so these kernels are DFMA-bound by a wide margin: the
 // 64 x 64 register-blocked tile below keeps the pipe saturated from one CTA per SM.
 #include "tc_internal.h"
+#include "zgemm_common.h"
 
 #define FIXED_FN __device__ __forceinline__
 #include "fixed_exp.h"
@@ -130,7 +131,7 @@ __device__ __forceinline__ void pivot_root(double d, double &sd, double &rp) {
         rp = 1.0 / sd;
     }
 }
-__device__ __forceinline__ void potrf64_body(double *D, int ld, int col0, int *status) {
+__device__ __forceinline__ bool potrf64_body(double *D, int ld, int col0, int *status) {   // false: not positive
     __shared__ double S[64][65];                 // S[c][r], r >= c: L_rc once column c is done
     __shared__ double ls[2][64];                 // column j of L
     __shared__ int fail;
@@ -139,7 +140,7 @@ __device__ __forceinline__ void potrf64_body(double *D, int ld, int col0, int *s
     for (int idx = tid; idx < 4096; idx += POTRF_THREADS) {
         const int r = idx & 63, c = idx >> 6;
         if (r >= c) {
-            S[c][r] = D[(int64_t)c * ld + r];
+            S[c][r] = __ldcg(D + (int64_t)c * ld + r);
             tab[(63 - c) * (64 - c) / 2 + r - c] = (uint16_t)(c << 8 | r);
         }
     }
@@ -184,12 +185,13 @@ __device__ __forceinline__ void potrf64_body(double *D, int ld, int col0, int *s
     __syncthreads();
     if (fail) {
         if (tid == 0) atomicCAS(status, 0, col0 + fail);
-        return;
+        return false;
     }
     for (int idx = tid; idx < 4096; idx += POTRF_THREADS) {
         const int r = idx & 63, c = idx >> 6;
         if (r >= c) D[(int64_t)c * ld + r] = S[c][r];
     }
+    return true;
 }
 __global__ void __launch_bounds__(POTRF_THREADS) k_potrf_block(double *D, int ld, int col0, int *status) {
     if (failed(status)) return;
@@ -217,17 +219,8 @@ __device__ __forceinline__ void strip_solve(double (*Ss)[65], double (*Ls)[65], 
 // and no step needs a barrier.  Bound by the FP64 pipe (160 warp operations of 64 cycles a row, 10 us
 // for 8 rows): a launch takes 17 us, where 16 rows with two block barriers a step took 28 us.
 constexpr int PANEL_ROWS = 8;
-__device__ __forceinline__ void panel_body(double *Pb, const double *L, int ld) {
-    __shared__ double Ls[64][65], rinv[64];      // Ls[j][c] = l_cj, c >= j
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    for (int idx = tid; idx < 4096; idx += 256) {
-        const int c = idx & 63, j = idx >> 6;
-        if (c >= j) Ls[j][c] = L[(int64_t)j * ld + c];
-    }
-    double z0 = Pb[(int64_t)lane * ld + warp], z1 = Pb[(int64_t)(lane + 32) * ld + warp];
-    __syncthreads();
-    if (tid < 64) rinv[tid] = 1.0 / Ls[tid][tid];
-    __syncthreads();
+__device__ __forceinline__ void panel_row(const double (*Ls)[65], const double *rinv, double &z0, double &z1) {
+    const int lane = threadIdx.x & 31;
 #pragma unroll 8
     for (int j = 0; j < 32; ++j) {
         const double x = __shfl_sync(0xffffffffu, z0, j) * rinv[j];
@@ -239,8 +232,23 @@ __device__ __forceinline__ void panel_body(double *Pb, const double *L, int ld) 
         const double x = __shfl_sync(0xffffffffu, z1, j) * rinv[j + 32];
         if (lane > j) z1 = fma(-x, Ls[j + 32][lane + 32], z1);
     }
-    Pb[(int64_t)lane * ld + warp] = z0 * rinv[lane];
-    Pb[(int64_t)(lane + 32) * ld + warp] = z1 * rinv[lane + 32];
+    z0 *= rinv[lane];
+    z1 *= rinv[lane + 32];
+}
+__device__ __forceinline__ void panel_body(double *Pb, const double *L, int ld) {
+    __shared__ double Ls[64][65], rinv[64];      // Ls[j][c] = l_cj, c >= j
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    for (int idx = tid; idx < 4096; idx += 256) {
+        const int c = idx & 63, j = idx >> 6;
+        if (c >= j) Ls[j][c] = L[(int64_t)j * ld + c];
+    }
+    double z0 = Pb[(int64_t)lane * ld + warp], z1 = Pb[(int64_t)(lane + 32) * ld + warp];
+    __syncthreads();
+    if (tid < 64) rinv[tid] = 1.0 / Ls[tid][tid];
+    __syncthreads();
+    panel_row(Ls, rinv, z0, z1);
+    Pb[(int64_t)lane * ld + warp] = z0;
+    Pb[(int64_t)(lane + 32) * ld + warp] = z1;
 }
 __global__ void __launch_bounds__(256) k_trsm_rows(double *P, const double *L, int ld, const int *status) {
     if (failed(status)) return;
@@ -825,6 +833,185 @@ void launch_syrk_rows_batched(const PEntry *e, int n, int rows, int ld, cudaStre
 void launch_syrk_rows(double *D, int rows, int ld, const int *status, cudaStream_t s) {
     const int m = rows / 64;
     if (m > 0) k_syrk_rows<<<8 * m * (m + 1), SYRK_THREADS, 0, s>>>(D, ld, status);
+}
+
+// The whole POTRF of one tile as a cooperative kernel: CTA 0 factors the 64-blocks of the diagonal, the
+// others solve the panels and update the trailing blocks, all with the operations and the order of
+// the kernels above (the same bits).  What this is for: the chain.  A step's three launches took
+// 38 + 17 + 27 us and the gaps between them at tile 1024 although only 16 of the update's blocks stand
+// before the next pivot block.  Here those 16 come first, alone on their SMs, and the next 64-block is
+// factored while the rest of the update runs: 67 us a step (86 before), 62 at tile 512 (77), 117
+// at tile 2048 (143; the pipe's own 84).
+//   * flags[0 ..]: block j is factored (-1: not positive, everyone leaves); [64 ..]: CTAs done with panel
+//     j; [128 ..] and [192 ..]: updates of diagonal block j and of block column j through step j - 1.
+//   * A 16 x 16 block belongs to one group of 64 threads for good, so its updates are in order without
+//     flags; index e counts from the last block column, so what trails step j are the first
+//     8 m (m + 1) indexes and a group takes its own from the top: diagonal block, its column, the rest.
+//   * Data of other CTAs is read through L2 (ld.cg), and every wait is bounded: a wait that runs out
+//     sets *err, and all CTAs leave.
+constexpr int PT_GROUPS = POTRF_THREADS / 64, PT_FLAGS = 64;
+constexpr size_t PT_SMEM = (size_t)PT_GROUPS * 2 * 64 * SYRK_B * sizeof(double);
+constexpr unsigned long long PT_LIMIT_NS = 4000000000ull;
+static_assert(PT_SMEM >= (64 * 65 + 64) * sizeof(double), "a panel's triangle fits the update's place");
+
+// (one thread) waits until *p is at least want; negative when it turned negative or the wait ran out
+__device__ __forceinline__ int pt_wait(const int *p, int want, int *err, unsigned long long limit_ns) {
+    int v;
+    const uint64_t t0 = z_timer();
+    for (;;) {
+        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+        if (v >= want || v < 0) return v;
+        if (*(volatile int *)err) return -1;
+        if (z_timer() - t0 > limit_ns) {
+            atomicExch(err, 1);
+            return -1;
+        }
+    }
+}
+__device__ __forceinline__ void pt_add(int *p) {          // (one thread, after a barrier) releases the CTA's or group's stores
+    __threadfence();
+    atomicAdd(p, 1);
+}
+__device__ __forceinline__ void pt_group_sync(int grp) { asm volatile("bar.sync %0, 64;" ::"r"(grp + 1) : "memory"); }
+
+__global__ void __launch_bounds__(POTRF_THREADS)
+k_potrf_tile(double *D, int ld, int nb, int col0, int *status, int *flags, int *err, unsigned long long limit_ns) {
+    extern __shared__ double pts[];
+    __shared__ int go, filled;                             // a flag per wait of a step: the next write comes after a barrier
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    int *factored = flags, *panels = flags + PT_FLAGS, *diag = flags + 2 * PT_FLAGS, *column = flags + 3 * PT_FLAGS;
+    // a tile after a failure: nothing runs (a failure in this call comes after every CTA's first panel)
+    if (tid == 0) go = !failed(status);
+    __syncthreads();
+    if (blockIdx.x == 0) {
+        if (!go) {
+            if (tid == 0) atomicExch(factored, -1);
+            return;
+        }
+        for (int j = 0; j < nb; ++j) {
+            if (j > 0) {
+                if (tid == 0) go = pt_wait(diag + j, 16, err, limit_ns) > 0;
+                __syncthreads();
+                if (!go) return;
+            }
+            const bool ok = potrf64_body(D + (int64_t)j * 64 * ld + j * 64, ld, col0 + j * 64, status);
+            __syncthreads();
+            if (tid == 0) {
+                __threadfence();
+                atomicExch(factored + j, ok ? 1 : -1);
+            }
+            if (!ok) return;
+        }
+        return;
+    }
+    const int w = (int)blockIdx.x - 1, nw = (int)gridDim.x - 1, grp = tid >> 6, gt = tid & 63;
+    for (int j = 0; j + 1 < nb; ++j) {
+        const int m = nb - 1 - j;                          // block rows below
+        if (tid == 0) {
+            go = pt_wait(factored + j, 1, err, limit_ns) > 0;
+            if (go && j > 0) go = pt_wait(column + j, 16 * (m + 1), err, limit_ns) > 0;
+        }
+        __syncthreads();
+        if (!go) return;
+        // the panel: four adjacent rows to four warps, eight warps a CTA
+        if (w < 16 * m) {
+            double(*Ls)[65] = reinterpret_cast<double(*)[65]>(pts), *rinv = pts + 64 * 65;
+            const double *L = D + (int64_t)j * 64 * ld + j * 64;
+#pragma unroll 4
+            for (int idx = tid; idx < 4096; idx += POTRF_THREADS) {
+                const int c = idx & 63, k = idx >> 6;
+                if (c >= k) Ls[k][c] = __ldcg(L + (int64_t)k * ld + c);
+            }
+            __syncthreads();
+            if (tid < 64) rinv[tid] = 1.0 / Ls[tid][tid];
+            __syncthreads();
+            if (warp < 8)
+                for (int g = w + nw * (warp >> 2); g < 16 * m; g += 2 * nw) {
+                    double *Pb = D + (int64_t)j * 64 * ld + (j + 1) * 64 + 4 * g + (warp & 3);
+                    double z0 = __ldcg(Pb + (int64_t)lane * ld), z1 = __ldcg(Pb + (int64_t)(lane + 32) * ld);
+                    panel_row(Ls, rinv, z0, z1);
+                    __stcg(Pb + (int64_t)lane * ld, z0);
+                    __stcg(Pb + (int64_t)(lane + 32) * ld, z1);
+                }
+        }
+        __syncthreads();
+        if (tid == 0) {
+            pt_add(panels + j);
+            filled = pt_wait(panels + j, nw, err, limit_ns) > 0;
+        }
+        __syncthreads();
+        if (!filled) return;
+        const int total = 8 * m * (m + 1), slots = PT_GROUPS * nw, slot = grp * nw + w;
+        int e = slot < total ? slot + (total - 1 - slot) / slots * slots : -1;
+        bool first = false;                                // does this CTA hold part of the diagonal block?
+        for (int t = total - 16; t < total; ++t) first |= t % slots % nw == w;
+        double(*X)[SYRK_B] = reinterpret_cast<double(*)[SYRK_B]>(pts + (size_t)grp * 2 * 64 * SYRK_B), (*Y)[SYRK_B] = X + 64;
+        const int r = gt & 15, q = gt >> 4;
+        const auto update = [&](int id) {
+            const int t = id >> 4;
+            int c = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
+            while (c * (c + 1) / 2 > t) --c;
+            while ((c + 1) * (c + 2) / 2 <= t) ++c;
+            const int bi = 4 * (nb - 1 - (t - c * (c + 1) / 2)) + (id & 3), bj = 4 * (nb - 1 - c) + ((id >> 2) & 3);
+            const double *P = D + (int64_t)j * 64 * ld;
+            double *C = D + (int64_t)bj * SYRK_B * ld + bi * SYRK_B;
+            pt_group_sync(grp);                            // the previous block's operands are used
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                X[q + 4 * k][r] = __ldcg(P + (int64_t)(q + 4 * k) * ld + bi * SYRK_B + r);
+                Y[q + 4 * k][r] = __ldcg(P + (int64_t)(q + 4 * k) * ld + bj * SYRK_B + r);
+            }
+            double acc[4] = {}, old[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) old[u] = __ldcg(C + (int64_t)(q + 4 * u) * ld + r);
+            pt_group_sync(grp);
+#pragma unroll 16
+            for (int k = 0; k < 64; ++k) {
+                const double a = X[k][r];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) acc[u] = fma(a, Y[k][q + 4 * u], acc[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) __stcg(C + (int64_t)(q + 4 * u) * ld + r, old[u] - acc[u]);
+            if (c == m - 1) {                              // block column j + 1
+                pt_group_sync(grp);
+                if (gt == 0) {
+                    if (id >= total - 16) pt_add(diag + j + 1);
+                    pt_add(column + j + 1);
+                }
+            }
+        };
+        if (first) {
+            if (e >= total - 16) {
+                update(e);
+                e -= slots;
+            }
+            __syncthreads();
+        }
+        for (; e >= 0; e -= slots) update(e);
+    }
+}
+size_t potrf_tile_flags() { return 4 * PT_FLAGS * sizeof(int); }
+// A tile whose steps fit the flags, from two 64-blocks on; the grid is what the first update keeps busy.
+bool potrf_tile_ok(int b) { return b >= 128 && b <= 64 * PT_FLAGS; }
+int launch_potrf_tile(double *D, int b, int col0, int *status, int *flags, int *err, cudaStream_t s,
+                      unsigned long long limit_ns) {
+    static std::atomic<unsigned long long> attr{0};
+    if (attrs_pending(attr)) {
+        cudaFuncSetAttribute(k_potrf_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PT_SMEM);
+        mark_attrs_set(attr);
+    }
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaMemsetAsync(flags, 0, potrf_tile_flags(), s);
+    if (e != cudaSuccess) return (int)e;
+    int nb = b / 64, grid = 1 + 8 * nb * (nb - 1);
+    if (grid > sms) grid = sms;
+    if (!limit_ns) limit_ns = PT_LIMIT_NS;
+    void *args[] = {(void *)&D, (void *)&b, (void *)&nb, (void *)&col0, (void *)&status, (void *)&flags, (void *)&err,
+                    (void *)&limit_ns};
+    return (int)cudaLaunchCooperativeKernel((const void *)k_potrf_tile, dim3(grid), dim3(POTRF_THREADS), args, PT_SMEM, s);
 }
 
 // log|A_i| = 2 sum log L_ii for every matrix of a batch (one CTA each, fixed order)

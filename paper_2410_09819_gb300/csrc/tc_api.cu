@@ -696,7 +696,16 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
             if (rc) return rc;
         }
         const int sp_potrf = spans ? span_begin(h, CAT_POTRF) : -1;
+        // one matrix: its tile in one kernel (a captured batch keeps the launches per step, which take
+        // the tiles of all matrices at once)
+        const bool one = spans && nmat == 1 && k < h->mats[0].nt && potrf_tile_ok(b);
+        if (one) {
+            CK((cudaError_t)launch_potrf_tile(W + (h->mats[0].tile0 + tidx(k, k)) * bb, b, k * b, status + 2,
+                                              static_cast<int *>(h->potrf.p), status + 1, h->s, wait_limit_ns(h)));
+            CK_LAUNCH();
+        }
         for (const PotrfStep &ps : C.potrf) {
+            if (one) break;
             launch_potrf_blocks(D.pentries + ps.pe0, ps.npe, b, h->s);
             CK_LAUNCH();
             if (ps.rows > 0) {
@@ -878,6 +887,7 @@ int factor_matrices(tc_handle h, tc_stats *stats, bool use_graph, const std::vec
     int *status = static_cast<int *>(h->status.p);
     double *W = static_cast<double *>(h->W.p);
     int rc = ensure(h, h->status, (2 + h->mats.size()) * sizeof(int));
+    if (!rc) rc = ensure(h, h->potrf, potrf_tile_flags());
     if (rc) return rc;
     status = static_cast<int *>(h->status.p);
     if ((rc = ensure(h, h->scratch, std::max<size_t>(4096, h->mats.size()) * sizeof(double)))) return rc;
@@ -998,7 +1008,7 @@ void tc_destroy(tc_handle h) {
     if (!h) return;
     cudaSetDevice(h->device);
     if (h->s) cudaStreamSynchronize(h->s);
-    for (DevBuf *d : {&h->W, &h->Acopy, &h->status, &h->scratch, &h->tables, &h->partials, &h->vec, &h->sumsq,
+    for (DevBuf *d : {&h->W, &h->Acopy, &h->status, &h->scratch, &h->tables, &h->partials, &h->vec, &h->sumsq, &h->potrf,
                       &h->pool_hi, &h->pool_lo, &h->pool16, &h->pool8, &h->mxtab, &h->logdiag, &h->dpool, &h->ztab,
                       &h->invbuf, &h->stab, &h->sweep})
         release(*d);

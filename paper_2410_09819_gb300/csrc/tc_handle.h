@@ -50,6 +50,7 @@ struct tc_handle_s {
     DevBuf vec;        // solve workspace
     DevBuf sweep;      // substitution sweeps: error word, progress counters
     DevBuf sumsq;      // tile sums of squares
+    DevBuf potrf;      // flags of a tile's POTRF
     // mixed precision: operand pools, tables and tensor maps
     DevBuf pool_hi, pool_lo, pool16, pool8;
     DevBuf mxtab;

@@ -112,6 +112,12 @@ void launch_dgemm_reduce(const DRed *reds, int nreds, int ld, const double *part
                          const int *status, cudaStream_t s);
 void launch_potrf_block(double *D, int ld, int col0, int *status, cudaStream_t s);
 void launch_trsm_rows(double *P, const double *L, int ld, int rows, const int *status, cudaStream_t s);
+// POTRF of one b x b tile in one cooperative kernel, where potrf_tile_ok(b): flags a buffer of
+// potrf_tile_flags() bytes (cleared here), *err set when a wait ran into its bound.  Returns a cudaError_t.
+size_t potrf_tile_flags();
+bool potrf_tile_ok(int b);
+int launch_potrf_tile(double *D, int b, int col0, int *status, int *flags, int *err, cudaStream_t s,
+                      unsigned long long limit_ns);
 void launch_potrf_blocks(const PEntry *e, int n, int ld, cudaStream_t s);
 void launch_trsm_rows_batched(const PEntry *e, int n, int max_rows, int ld, cudaStream_t s);
 // the POTRF step's trailing update: the lower part of the rows below the panel, C -= P P^T

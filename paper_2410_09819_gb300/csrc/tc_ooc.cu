@@ -483,6 +483,7 @@ extern "C" int tile_chol_factor_ooc(tc_handle h, int64_t n, int b, double *A_til
     if ((rc = init_cache(h, C, A_tiles, nt, b, zmode, mixed ? pm.data() : nullptr))) return rc;
     if ((rc = ensure(h, h->logdiag, (size_t)nt * sizeof(double)))) return rc;
     double *logdiag = static_cast<double *>(h->logdiag.p);
+    if ((rc = ensure(h, h->potrf, potrf_tile_flags()))) return rc;
     int *status = static_cast<int *>(h->status.p);
     CK(cudaMemsetAsync(status, 0, 2 * sizeof(int), h->s));
     const int nv_last = (int)(n - (int64_t)(nt - 1) * b);
@@ -658,7 +659,12 @@ extern "C" int tile_chol_factor_ooc(tc_handle h, int64_t n, int b, double *A_til
             if (g0 == k) {
                 double *D = C.ptr(sc[0]);
                 const int spp = span_begin(h, CAT_POTRF);
-                for (int jb = 0; jb < b / 64; ++jb) {
+                if (potrf_tile_ok(b)) {
+                    CK((cudaError_t)launch_potrf_tile(D, b, k * b, status, static_cast<int *>(h->potrf.p), status + 1, h->s,
+                                                      wait_limit_ns(h)));
+                    CK_LAUNCH();
+                }
+                for (int jb = 0; jb < b / 64 && !potrf_tile_ok(b); ++jb) {
                     launch_potrf_block(D + (int64_t)jb * 64 * b + jb * 64, b, k * b + jb * 64, status, h->s);
                     CK_LAUNCH();
                     if (jb + 1 < b / 64) {
