@@ -840,8 +840,10 @@ void launch_syrk_rows(double *D, int rows, int ld, const int *status, cudaStream
 // the kernels above (the same bits).  What this is for: the chain.  A step's three launches took
 // 38 + 17 + 27 us and the gaps between them at tile 1024 although only 16 of the update's blocks stand
 // before the next pivot block.  Here those 16 come first, alone on their SMs, and the next 64-block is
-// factored while the rest of the update runs: 67 us a step (86 before), 62 at tile 512 (77), 117
-// at tile 2048 (143; the pipe's own 84).
+// factored while the rest of the update runs; they take the whole CTA, an element a thread (a group of two
+// warps needs 8 us for a block's multiply-adds, eight warps 2), and the panel's rows are loaded
+// while their block is factored.  A step takes 61 us at tile 1024 (86 as launches), 58 at tile 512 (77),
+// 112 at tile 2048 (143; the pipe's own 84).
 //   * flags[0 ..]: block j is factored (-1: not positive, everyone leaves); [64 ..]: CTAs done with panel
 //     j; [128 ..] and [192 ..]: updates of diagonal block j and of block column j through step j - 1.
 //   * A 16 x 16 block belongs to one group of 64 threads for good, so its updates are in order without
@@ -877,7 +879,7 @@ __device__ __forceinline__ void pt_group_sync(int grp) { asm volatile("bar.sync 
 __global__ void __launch_bounds__(POTRF_THREADS)
 k_potrf_tile(double *D, int ld, int nb, int col0, int *status, int *flags, int *err, unsigned long long limit_ns) {
     extern __shared__ double pts[];
-    __shared__ int go, filled;                             // a flag per wait of a step: the next write comes after a barrier
+    __shared__ int ready, go, filled;    // a flag per wait of a step, so that its next write comes after a barrier
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     int *factored = flags, *panels = flags + PT_FLAGS, *diag = flags + 2 * PT_FLAGS, *column = flags + 3 * PT_FLAGS;
     // a tile after a failure: nothing runs (a failure in this call comes after every CTA's first panel)
@@ -907,13 +909,21 @@ k_potrf_tile(double *D, int ld, int nb, int col0, int *status, int *flags, int *
     const int w = (int)blockIdx.x - 1, nw = (int)gridDim.x - 1, grp = tid >> 6, gt = tid & 63;
     for (int j = 0; j + 1 < nb; ++j) {
         const int m = nb - 1 - j;                          // block rows below
-        if (tid == 0) {
-            go = pt_wait(factored + j, 1, err, limit_ns) > 0;
-            if (go && j > 0) go = pt_wait(column + j, 16 * (m + 1), err, limit_ns) > 0;
+        const int g0 = w + nw * (warp >> 2);               // the panel: four adjacent rows to four warps, eight warps a CTA
+        const bool mine = warp < 8 && g0 < 16 * m;
+        double *const Pr = D + (int64_t)(j * 64 + lane) * ld + (j + 1) * 64 + (warp & 3);
+        const int64_t half = (int64_t)32 * ld;
+        double z0 = 0.0, z1 = 0.0;
+        if (tid == 0) ready = j == 0 || pt_wait(column + j, 16 * (m + 1), err, limit_ns) > 0;
+        __syncthreads();
+        if (!ready) return;
+        if (mine) {                                        // the first rows, while block j is factored
+            z0 = __ldcg(Pr + 4 * g0);
+            z1 = __ldcg(Pr + 4 * g0 + half);
         }
+        if (tid == 0) go = pt_wait(factored + j, 1, err, limit_ns) > 0;
         __syncthreads();
         if (!go) return;
-        // the panel: four adjacent rows to four warps, eight warps a CTA
         if (w < 16 * m) {
             double(*Ls)[65] = reinterpret_cast<double(*)[65]>(pts), *rinv = pts + 64 * 65;
             const double *L = D + (int64_t)j * 64 * ld + j * 64;
@@ -925,13 +935,15 @@ k_potrf_tile(double *D, int ld, int nb, int col0, int *status, int *flags, int *
             __syncthreads();
             if (tid < 64) rinv[tid] = 1.0 / Ls[tid][tid];
             __syncthreads();
-            if (warp < 8)
-                for (int g = w + nw * (warp >> 2); g < 16 * m; g += 2 * nw) {
-                    double *Pb = D + (int64_t)j * 64 * ld + (j + 1) * 64 + 4 * g + (warp & 3);
-                    double z0 = __ldcg(Pb + (int64_t)lane * ld), z1 = __ldcg(Pb + (int64_t)(lane + 32) * ld);
+            if (mine)
+                for (int g = g0; g < 16 * m; g += 2 * nw) {
+                    if (g != g0) {
+                        z0 = __ldcg(Pr + 4 * g);
+                        z1 = __ldcg(Pr + 4 * g + half);
+                    }
                     panel_row(Ls, rinv, z0, z1);
-                    __stcg(Pb + (int64_t)lane * ld, z0);
-                    __stcg(Pb + (int64_t)(lane + 32) * ld, z1);
+                    __stcg(Pr + 4 * g, z0);
+                    __stcg(Pr + 4 * g + half, z1);
                 }
         }
         __syncthreads();
@@ -943,17 +955,43 @@ k_potrf_tile(double *D, int ld, int nb, int col0, int *status, int *flags, int *
         if (!filled) return;
         const int total = 8 * m * (m + 1), slots = PT_GROUPS * nw, slot = grp * nw + w;
         int e = slot < total ? slot + (total - 1 - slot) / slots * slots : -1;
-        bool first = false;                                // does this CTA hold part of the diagonal block?
-        for (int t = total - 16; t < total; ++t) first |= t % slots % nw == w;
         double(*X)[SYRK_B] = reinterpret_cast<double(*)[SYRK_B]>(pts + (size_t)grp * 2 * 64 * SYRK_B), (*Y)[SYRK_B] = X + 64;
         const int r = gt & 15, q = gt >> 4;
+        const double *P = D + (int64_t)j * 64 * ld;
+        // the blocks of the next diagonal block on the whole CTA, an element a thread
+        for (int t = total - 16; t < total; ++t) {
+            if (t % slots % nw != w) continue;
+            const int bi = 4 * (j + 1) + (t & 3), bj = 4 * (j + 1) + ((t >> 2) & 3), col = tid >> 4;
+            double(*XA)[SYRK_B] = reinterpret_cast<double(*)[SYRK_B]>(pts), (*YA)[SYRK_B] = XA + 64;
+            const int64_t o = (int64_t)(bj * SYRK_B + col) * ld + bi * SYRK_B + r;
+            double acc = 0.0, old = 0.0;
+            if (tid < 256) {
+                old = __ldcg(D + o);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    XA[col + 16 * k][r] = __ldcg(P + (int64_t)(col + 16 * k) * ld + bi * SYRK_B + r);
+                    YA[col + 16 * k][r] = __ldcg(P + (int64_t)(col + 16 * k) * ld + bj * SYRK_B + r);
+                }
+            }
+            __syncthreads();
+            if (tid < 256) {
+#pragma unroll 16
+                for (int k = 0; k < 64; ++k) acc = fma(XA[k][r], YA[k][col], acc);
+                __stcg(D + o, old - acc);
+            }
+            __syncthreads();
+            if (tid == 0) {
+                pt_add(diag + j + 1);
+                pt_add(column + j + 1);
+            }
+        }
+        if (e >= total - 16) e -= slots;
         const auto update = [&](int id) {
             const int t = id >> 4;
             int c = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
             while (c * (c + 1) / 2 > t) --c;
             while ((c + 1) * (c + 2) / 2 <= t) ++c;
             const int bi = 4 * (nb - 1 - (t - c * (c + 1) / 2)) + (id & 3), bj = 4 * (nb - 1 - c) + ((id >> 2) & 3);
-            const double *P = D + (int64_t)j * 64 * ld;
             double *C = D + (int64_t)bj * SYRK_B * ld + bi * SYRK_B;
             pt_group_sync(grp);                            // the previous block's operands are used
 #pragma unroll
@@ -975,19 +1013,9 @@ k_potrf_tile(double *D, int ld, int nb, int col0, int *status, int *flags, int *
             for (int u = 0; u < 4; ++u) __stcg(C + (int64_t)(q + 4 * u) * ld + r, old[u] - acc[u]);
             if (c == m - 1) {                              // block column j + 1
                 pt_group_sync(grp);
-                if (gt == 0) {
-                    if (id >= total - 16) pt_add(diag + j + 1);
-                    pt_add(column + j + 1);
-                }
+                if (gt == 0) pt_add(column + j + 1);
             }
         };
-        if (first) {
-            if (e >= total - 16) {
-                update(e);
-                e -= slots;
-            }
-            __syncthreads();
-        }
         for (; e >= 0; e -= slots) update(e);
     }
 }
