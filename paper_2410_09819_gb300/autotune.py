@@ -2,8 +2,8 @@
 
 * In core, batched: the tile size and the FP64 update engine.  The tile size sets the number
   of tasks, the parallelism per column step and the padding of ragged matrices; the engine sets
-  the kernel and block shape of the FP64 output tiles (64 x 64 FP64-pipe blocks, or 128 x 16
-  digit-plane items on the E4M3 tensor cores).  ``pick_batched_config`` times
+  the kernel and block shape of the FP64 output tiles (64 x 64 FP64-pipe blocks, or digit-plane
+  items on the tensor cores: 128 x 32 in FP16, 128 x 64 in E4M3 for mixed maps).  ``pick_batched_config`` times
   ``tile_chol_factor_batched`` (graph replay, after one capture) for each candidate on the
   caller's batch and returns the fastest.
 * Out of core: the tile size, the scheduling policy and the eviction rule under a device-cache
@@ -47,8 +47,8 @@ def pick_batched_config(make_handle, ns, make_inputs, tiles=(128, 256), engines=
 
     The engine fixes the kernel, and with it the block shape, of the FP64 output tiles (the
     diagonal and every tile the map keeps in FP64): fp64_mode 0 runs them on the FP64 pipe in
-    64 x 64 register blocks, fp64_mode 2 on the E4M3 tensor cores in 128 x 16 digit-plane
-    items; FP16 / FP8 tiles always take the 128 x 128 tensor-core blocks.  make_handle(mode)
+    64 x 64 register blocks, fp64_mode 2 on the tensor cores in digit-plane items (128 x 32 in
+    FP16, 128 x 64 in E4M3 for mixed maps); FP16 / FP8 tiles always take the 128 x 128 tensor-core blocks.  make_handle(mode)
     returns a new handle (a context manager) for an engine; make_inputs(b) -> (A_list, maps).
     Returns ((b, mode), {(b, mode): seconds}); tile sizes the engine cannot run (the
     digit-plane engine needs multiples of 128) are left out."""
