@@ -1,9 +1,10 @@
 // Input preparation on the device: the Matern covariance of Eq. 2 (Section III-D) written
 // straight into the lower tile layout, and the per-tile sums of squares behind the
-// precision criterion of Section IV-C.  Both are HBM-bound (8 bytes written or read per
-// element).
+// precision criterion of Section IV-C: integer work bounds the first, the FP64 pipe and HBM the
+// second (at the kernels below).
 #include "tc_internal.h"
 
+#include <algorithm>
 #include <cooperative_groups.h>
 
 #define FIXED_FN __host__ __device__ __forceinline__
@@ -327,9 +328,13 @@ k_tile_sumsq(const double *A, int b, int64_t n, double *out, int t0) {
 void launch_matern(double *A, int64_t n, int b, int nt, const double *pts, double sigma2, double a,
                    int nu2, double nu, double nugget, cudaStream_t s) {
     const int T = nt * (nt + 1) / 2;
-    // at least 16 elements a thread (a CTA fills a table of 1024 entries first), 64 CTAs a tile at most
+    // 16 elements a thread (a CTA fills a table of 1024 entries first), 64 CTAs a tile at most; few tiles
+    // take as many CTAs as fill the SMs with eight each, down to a column a CTA (nu = 0.8, 15 tiles of 128:
+    // 835 us with four CTAs a tile, 281 us; nu = 3/2, 6 tiles of 256: 50 and 40 us)
     int gx = (int)((int64_t)b * b / 4096);
     gx = gx < 1 ? 1 : gx > 64 ? 64 : gx;
+    const int fill = (8 * 152 + T - 1) / T, columns = b < 256 ? b / (256 / b) : b;
+    gx = std::max(gx, std::min(fill, columns));
     Range g{};
     g.a = a;
     g.fast = a > 1e-100 && a < 1e100;
