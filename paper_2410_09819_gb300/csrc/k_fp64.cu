@@ -1103,13 +1103,14 @@ __global__ void __launch_bounds__(256) k_fwd_update_g(const SUpd *__restrict__ u
 #pragma unroll
     for (int q = 0; q < NQ; ++q) acc[q] = 0.0;
     for (int c0 = 0; c0 < b; c0 += 128) {
+        const int nc = min(128, b - c0);          // a tile need not be a multiple of 128
         __syncthreads();
         for (int e = tid; e < 128 * nrhs; e += 256) {
             const int c = e % 128, q = e / 128;
-            zs[c][q] = R[U.src + q * U.ldr + c0 + c];
+            if (c < nc) zs[c][q] = R[U.src + q * U.ldr + c0 + c];
         }
         __syncthreads();
-        for (int c = part; c < 128; c += 4) {
+        for (int c = part; c < nc; c += 4) {
             const double l = U.L[(int64_t)(c0 + c) * b + U.r0 + rr];
 #pragma unroll
             for (int q = 0; q < NQ; ++q)
@@ -1194,13 +1195,14 @@ __global__ void __launch_bounds__(256) k_fwd_update_gf(const SUpd *__restrict__ 
 #pragma unroll
     for (int q = 0; q < NQ; ++q) acc[q] = 0.f;
     for (int c0 = 0; c0 < b; c0 += 128) {
+        const int nc = min(128, b - c0);          // a tile need not be a multiple of 128
         __syncthreads();
         for (int e = tid; e < 128 * nrhs; e += 256) {
             const int c = e % 128, q = e / 128;
-            zs[c][q] = R[U.src + q * U.ldr + c0 + c];
+            if (c < nc) zs[c][q] = R[U.src + q * U.ldr + c0 + c];
         }
         __syncthreads();
-        for (int c = part; c < 128; c += 4) {
+        for (int c = part; c < nc; c += 4) {
             const float l = (float)U.L[(int64_t)(c0 + c) * b + U.r0 + rr];
 #pragma unroll
             for (int q = 0; q < NQ; ++q)
