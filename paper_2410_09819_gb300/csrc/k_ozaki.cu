@@ -254,11 +254,11 @@ __device__ __forceinline__ int z_kblocks(const Args &a, const ZItem &it) {
 // prologue).
 // What bounds it: the tensor pipe.  Per 128 elements of K the 8 x 7 MMAs of P = 7 take
 // 8 (112 + 96 + 80 + 64 + 48 + 2 x 41) = 3856 cycles for 128 x 32 outputs (an MMA takes
-// max(41, N / 2) cycles); measured 4990 with boxes of 64-byte rows, of which 750 waited for a stage's
-// copies (56 bytes a clock and SM, a row a clock).  All P = 7 products of an FP64 factorization of
-// order 32768, tile 1024: 212 ms with those, 199 ms with bulk copies of the blocked planes (its
-// updates alone took 346 ms with base 16 in E4M3: 105 pairs, 128 x 16 items).  64 columns in two
-// buffers do not fit TMEM.
+// max(41, N / 2) cycles).  Measured 4990 with boxes of 64-byte rows, of which 750 waited for a stage's
+// copies (56 bytes a clock and SM, a row a clock); 4700 with bulk copies of the blocked planes, 450 of
+// them waiting for stages and 270 for accumulators at the ends of items.  All P = 7 products of an FP64
+// factorization of order 32768, tile 1024: 212 -> 197 ms (its updates alone took 346 ms with base 16
+// in E4M3: 105 pairs, 128 x 16 items).  64 columns in two buffers do not fit TMEM.
 //
 // Failure handling: every pipeline wait gives up after args.limit_ns (or when another role
 // set the abort flag), and the CTA then sets *err and stops issuing.  Before the TMEM is
