@@ -9,6 +9,7 @@
 #define FIXED_FN __device__ __forceinline__
 #include "fixed_exp.h"
 
+#include <algorithm>
 #include <cmath>
 
 namespace tc {
@@ -1036,7 +1037,7 @@ int launch_potrf_tile(double *D, int b, int col0, int *status, int *flags, int *
     if (e != cudaSuccess) return (int)e;
     int nb = b / 64, grid = 1 + 8 * nb * (nb - 1);
     if (grid > sms) grid = sms;
-    if (!limit_ns) limit_ns = PT_LIMIT_NS;
+    limit_ns = limit_ns ? std::max(limit_ns, GRID_WAIT_MIN_NS) : PT_LIMIT_NS;
     void *args[] = {(void *)&D, (void *)&b, (void *)&nb, (void *)&col0, (void *)&status, (void *)&flags, (void *)&err,
                     (void *)&limit_ns};
     return (int)cudaLaunchCooperativeKernel((const void *)k_potrf_tile, dim3(grid), dim3(POTRF_THREADS), args, PT_SMEM, s);

@@ -17,6 +17,8 @@
 #include "tc_internal.h"
 #include "zgemm_common.h"
 
+#include <algorithm>
+
 namespace tc {
 
 constexpr unsigned long long SWEEP_LIMIT_NS = 4000000000ull;   // default bound of the wait for a block
@@ -258,7 +260,7 @@ static cudaError_t sweep_launch(const double *W, int b, int nblk, double *r, int
 // (their chains run side by side, and four-column groups would multiply padding).
 int launch_sweep(const double *W, int b, int nblk, double *r, int64_t ldr, int nrhs, bool fwd, int *progress, int *err,
                  cudaStream_t s, unsigned long long limit_ns) {
-    if (!limit_ns) limit_ns = SWEEP_LIMIT_NS;
+    limit_ns = limit_ns ? std::max(limit_ns, GRID_WAIT_MIN_NS) : SWEEP_LIMIT_NS;
     if (nrhs < 4)
         return (int)(fwd ? sweep_launch<true, 1>(W, b, nblk, r, ldr, nrhs, progress, err, s, limit_ns)
                          : sweep_launch<false, 1>(W, b, nblk, r, ldr, nrhs, progress, err, s, limit_ns));

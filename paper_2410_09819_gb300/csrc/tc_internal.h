@@ -112,6 +112,10 @@ void launch_dgemm_reduce(const DRed *reds, int nreds, int ld, const double *part
                          const int *status, cudaStream_t s);
 void launch_potrf_block(double *D, int ld, int col0, int *status, cudaStream_t s);
 void launch_trsm_rows(double *P, const double *L, int ld, int rows, const int *status, cudaStream_t s);
+// Least bound of a wait for other CTAs of a cooperative kernel (k_potrf_tile, k_sweep).  Such a wait lasts
+// as long as their work, up to a millisecond at tile 4096, so a limit set for the microseconds of a
+// tensor-core pipeline does not end it.
+constexpr unsigned long long GRID_WAIT_MIN_NS = 100000000ull;
 // POTRF of one b x b tile in one cooperative kernel, where potrf_tile_ok(b): flags a buffer of
 // potrf_tile_flags() bytes (cleared here), *err set when a wait ran into its bound.  Returns a cudaError_t.
 size_t potrf_tile_flags();
