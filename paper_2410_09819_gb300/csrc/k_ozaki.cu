@@ -147,8 +147,9 @@ __device__ __forceinline__ void planes_of_tile(const double *T, int b, bool tran
     }
 }
 
-// exps[t] = smallest e with amax[t] <= 2^e; planes of tile t at pool + 14 t b^2.  The values come
-// from tile t of W, or (alt != nullptr) from the blockIdx.y-th tile of the contiguous buffer alt.
+// exps[t] = smallest e with amax[t] <= 2^e (Z_ZERO_EXP for a zero tile, whose digits are zero with any
+// exponent); planes of tile t at pool + 14 t b^2.  The values come from tile t of W, or
+// (alt != nullptr) from the blockIdx.y-th tile of the contiguous buffer alt.
 template <bool E4M3>
 __global__ void __launch_bounds__(256)
 k_digits(const double *W, int b, const int *tiles, const double *amax, uint8_t *pool, int *exps, const double *alt) {
@@ -156,7 +157,8 @@ k_digits(const double *W, int b, const int *tiles, const double *amax, uint8_t *
     const int64_t bb = (int64_t)b * b;
     const int e = z_digit_exp(amax[t]);
     if (blockIdx.x == 0 && threadIdx.x == 0) exps[t] = e;
-    planes_of_tile<E4M3>(alt ? alt + (int64_t)blockIdx.y * bb : W + (int64_t)t * bb, b, false, e, pool + (int64_t)t * Z_SLOT * bb);
+    planes_of_tile<E4M3>(alt ? alt + (int64_t)blockIdx.y * bb : W + (int64_t)t * bb, b, false, e == Z_ZERO_EXP ? 0 : e,
+                         pool + (int64_t)t * Z_SLOT * bb);
 }
 
 // --------------------------------------------------------------------- update kernel
@@ -411,7 +413,8 @@ k_zgemm(const __grid_constant__ Args args) {
             ZItem it;
             if (!args.tile(item, it)) continue;
             const int kblocks = z_kblocks(args, it);
-            // the largest scale of the item's sources: the unit of the sums
+            // the largest scale of the item's sources: the unit of the sums (zero tiles cannot be it,
+            // unless every source has one: then the sums are zero)
             int E0 = -(1 << 30);
             for (int n = lane; n < k; n += 32) E0 = max(E0, args.exps[args.xsrc(it, n)] + args.exps[args.ysrc(it, n)]);
             E0 = __reduce_max_sync(0xffffffffu, E0);
@@ -501,7 +504,7 @@ __global__ void __launch_bounds__(256)
 k_digits_src(const double *src, int b, int transpose, int dst, const double *amax, uint8_t *pool, int *exps) {
     const int e = z_digit_exp(*amax);
     if (blockIdx.x == 0 && threadIdx.x == 0) exps[dst] = e;
-    planes_of_tile<E4M3>(src, b, transpose != 0, e, pool + (int64_t)dst * Z_SLOT * b * b);
+    planes_of_tile<E4M3>(src, b, transpose != 0, e == Z_ZERO_EXP ? 0 : e, pool + (int64_t)dst * Z_SLOT * b * b);
 }
 
 // max |src[e]| as the largest sign-cleared bit pattern (non-negative doubles order like their

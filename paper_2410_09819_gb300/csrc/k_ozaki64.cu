@@ -71,8 +71,9 @@ struct Args {
 
 // Plane counts of one source: su, the budget of plane pairs s + t < su (from the scales: a pair
 // whose scale 2^(e_x + e_y) lies d binary orders below the output tile's input scale 2^e_out
-// keeps floor((d - 4 margin) / 4) planes fewer than rref, within [1, 14]), and the X / Y planes
-// its stored formats can have non-zero (the skipped products are exact zeros).
+// keeps floor((d - 4 margin) / 4) planes fewer than rref, within [1, 14]; Z_ZERO_EXP leaves an output
+// tile that is zero so far all 14 and a zero source one), and the X / Y planes its stored formats can
+// have non-zero (the skipped products are exact zeros).
 struct Shape {
     int sx, sy, su;
 };

@@ -153,9 +153,15 @@ __device__ __forceinline__ void z_ld16(uint32_t taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// Smallest e with amax <= 2^e (0 for amax <= 0): a tile's digit exponent.
+// Smallest e with amax <= 2^e: a tile's digit exponent.  A tile that is all zeros has no scale: its exponent
+// lies so far below every other (at least -1074, so -2148 for two operands) that no product with it
+// reaches that of two tiles with values, whatever the other operand (at most 2^1024).  Nothing else
+// would do: with exponent 0, one zero tile set the unit of k_zgemm's sums, and in a matrix of scale 1e-20
+// they lost all their bits; a zero output tile took the planes of k_zgemm64's sources.
+constexpr int Z_ZERO_EXP = -4096;
 __device__ __forceinline__ int z_digit_exp(double amax) {
-    if (!(amax > 0.0)) return 0;
+    if (amax == 0.0) return Z_ZERO_EXP;
+    if (!(amax > 0.0)) return 0;                     // NaN
     int ex;
     const double f = frexp(amax, &ex);
     return (f == 0.5) ? ex - 1 : ex;
