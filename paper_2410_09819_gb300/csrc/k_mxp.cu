@@ -93,6 +93,22 @@ __global__ void k_tile_amax(const double *W, int b, const int *tiles, double *am
     if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned long long *>(amax + t), m);
 }
 
+// The same for the last diagonal tile of every matrix that ends inside it, padding left out: its ones say
+// nothing about the tile's scale.
+__global__ void k_last_tile_amax(const LEntry *e, const double *W, int b, double *amax) {
+    const LEntry E = e[blockIdx.y];
+    const int64_t bb = (int64_t)b * b, last = tidx(E.nt - 1, E.nt - 1);
+    const int nv = (int)(E.n - (int64_t)(E.nt - 1) * b);
+    if (nv == b) return;
+    const double *T = E.W + last * bb;
+    unsigned long long m = 0;
+    for (int c = blockIdx.x; c < nv; c += gridDim.x)
+        for (int r = threadIdx.x; r < nv; r += blockDim.x)
+            m = max(m, (unsigned long long)__double_as_longlong(T[(int64_t)c * b + r]) & 0x7FFFFFFFFFFFFFFFull);
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned long long *>(amax + (E.W - W) / bb + last), m);
+}
+
 // W tile <- its value stored in precision prec[t] (Section IV-C), and amax of the result
 __global__ void k_store_round(double *W, int b, const int *tiles, const uint8_t *prec, const double *amaxL,
                               double *amaxS) {
@@ -615,6 +631,10 @@ void launch_tile_amax(const double *W, int b, const int *tiles, int ntiles, doub
         const int nt = ntiles - t0 < 65535 ? ntiles - t0 : 65535;
         k_tile_amax<<<dim3(tile_ctas(nt), nt), 256, 0, s>>>(W, b, tiles + t0, amax, alt ? alt + (int64_t)t0 * b * b : nullptr);
     }
+}
+void launch_last_tile_amax(const LEntry *e, int count, const double *W, int b, double *amax, cudaStream_t s) {
+    for (int i = 0; i < count; i += 65535)
+        k_last_tile_amax<<<dim3(32, count - i < 65535 ? count - i : 65535), 256, 0, s>>>(e + i, W, b, amax);
 }
 void launch_store_round(double *W, int b, const int *tiles, int ntiles, const uint8_t *prec, const double *amaxL,
                         double *amaxS, cudaStream_t s) {

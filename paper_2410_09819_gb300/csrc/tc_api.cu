@@ -509,7 +509,8 @@ struct PlanDev {
     const int *dtiles = nullptr;
     const uint8_t *zplanes = nullptr;   // leading non-zero digit planes per tile (mixed maps), else null
     double *oamax = nullptr;            // mixed: input amax of every tile (plane budgets of the updates)
-    const int *alltiles = nullptr;      // mixed: 0 .. Ttot-1 (the tile list of that amax)
+    const int *alltiles = nullptr;      // mixed: the tiles of that amax (all but last diagonal ones that hold padding)
+    int nalltiles = 0;
     unsigned long long *pairs = nullptr;   // mixed: plane pairs multiplied, FP64 / FP32 outputs
     int *zexps = nullptr;
     double *zamax = nullptr;
@@ -577,7 +578,10 @@ int prepare_factor(tc_handle h, const Plan &P, const MxpPlan *M, PlanDev &D) {
         for (const MatDesc &Md : h->mats) any_mixed |= Md.mixed;
         if (any_mixed) {
             int *all = reinterpret_cast<int *>(zh.data() + oall);
-            for (int64_t t = 0; t < Tt; ++t) all[t] = (int)t;
+            for (const MatDesc &Md : h->mats) {
+                const int64_t tiles = tidx(Md.nt, 0) - (Md.n % h->b ? 1 : 0);
+                for (int64_t t = 0; t < tiles; ++t) all[D.nalltiles++] = (int)(Md.tile0 + t);
+            }
             uint8_t *pl = reinterpret_cast<uint8_t *>(zh.data() + opl);
             memset(pl, 14, Tt);
             for (const MatDesc &Md : h->mats) {
@@ -638,8 +642,14 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
         // scale of every output tile before its updates: the reference of its plane budgets
         CK(cudaMemsetAsync(D.oamax, 0, P.Ttot * sizeof(double), h->s));
         CK(cudaMemsetAsync(D.pairs, 0, 2 * sizeof(unsigned long long), h->s));
-        launch_tile_amax(W, b, D.alltiles, (int)P.Ttot, D.oamax, h->s);
+        launch_tile_amax(W, b, D.alltiles, D.nalltiles, D.oamax, h->s);
         CK_LAUNCH();
+        bool ragged = false;
+        for (const MatDesc &Md : h->mats) ragged |= Md.n % b != 0;
+        if (ragged) {
+            launch_last_tile_amax(D.lentries, nmat, W, b, D.oamax, h->s);
+            CK_LAUNCH();
+        }
     }
     // mixed-precision digit-plane updates: per-source plane budgets relative to the output
     // tile's input scale (FP64 outputs: 14 reference planes; FP32 outputs: 10), margin 2 planes

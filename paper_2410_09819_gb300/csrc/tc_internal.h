@@ -322,6 +322,8 @@ void launch_qgemm(int kind, const CUtensorMap &a0, const CUtensorMap &a1, const 
                   int k, int b, int *err, cudaStream_t s, unsigned long long limit_ns = 0, int stall = 0);
 void launch_tile_amax(const double *W, int b, const int *tiles, int ntiles, double *amax, cudaStream_t s,
                       const double *alt = nullptr);
+// largest |a| of the valid part of the last diagonal tile of every matrix whose order is no multiple of b
+void launch_last_tile_amax(const LEntry *e, int count, const double *W, int b, double *amax, cudaStream_t s);
 void launch_store_round(double *W, int b, const int *tiles, int ntiles, const uint8_t *prec, const double *amaxL,
                         double *amaxS, cudaStream_t s);
 void launch_make_copies(const double *W, int b, const CopyJob *jobs, int njobs, const double *amaxS, float *hi,

@@ -96,3 +96,29 @@ def test_mixed_factor_at_small_and_large_scales(kind, path):
         bound = 2.0 ** -23 * np.linalg.norm(np.abs(L) @ np.abs(L.T)) * 1.01
         r[s] = np.linalg.norm(s * A - L @ L.T) / bound
     assert all(v <= 1.0 for v in r.values()), r
+
+
+@pytest.mark.parametrize("path", ["core", "batch", "ooc"])
+@pytest.mark.parametrize("n", [NT * B - 1, 2 * B + 1])
+def test_mixed_factor_of_a_ragged_order_at_small_scales(n, path):
+    # the ones on the padded diagonal are not the scale of the last diagonal tile
+    i = np.arange(n)
+    A = np.exp(-0.05 * np.abs(i[:, None] - i)) + 0.01 * np.eye(n)
+    nt = -(-n // B)
+    pm = np.zeros((nt, nt), dtype=np.uint8)
+    pm[1:, 0] = oracle.FP32
+    pm = pm.reshape(-1)
+    r = {}
+    for s in (1.0, 1e-10, 1e-20):
+        if path == "batch":
+            with tc.Handle(0, fp64_mode=2) as H:
+                dev = [to_dev(pack_padded(s * m, B)) for m in (A[:B, :B], A)]
+                one = np.zeros(1, dtype=np.uint8)
+                assert tc.tile_chol_factor_batched(H.h, [B, n], B, dev, [one, pm])[0] == 0
+                Lt = torch.empty_like(dev[1])
+                tc.tile_chol_get_factor_batched(H.h, 1, Lt)
+                L = unpack_lower(Lt, n, B)
+        else:
+            L = (in_core if path == "core" else out_of_core)(s * A, 2, pm)
+        r[s] = np.linalg.norm(s * A - L @ L.T) / (2.0 ** -23 * np.linalg.norm(np.abs(L) @ np.abs(L.T)) * 1.01)
+    assert all(v <= 1.0 for v in r.values()), r
