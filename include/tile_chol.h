@@ -110,19 +110,24 @@ typedef struct {
                                    1: 3 x TF32 tensor-core products with FP32 accumulation
                                    (as with fp64_mode 0: FP32-level arithmetic, the
                                    paper's FP32 tiles).  Other values: TC_ERR_ARG. */
-    int wait_limit_us;          /* bound, in microseconds, of every wait inside the
-                                   tensor-core update kernels (a pipeline stage that does not
-                                   arrive in time); 0 (default): 4 s.  When a wait runs out the
+    int wait_limit_us;          /* bound, in microseconds, of every wait inside a kernel; 0
+                                   (default): 4 s.  In the tensor-core update kernels (a
+                                   pipeline stage that does not arrive in time) it applies as
+                                   given; in the cooperative kernels, whose CTAs wait for one
+                                   another's work (POTRF of a tile and the substitution sweeps
+                                   of a solve or log-likelihood, in every fp64_mode), it is
+                                   raised to at least 100 ms (100000).  When a wait runs out the
                                    kernel stops issuing, lets its own copies and MMAs finish,
                                    releases its tensor memory and returns; the call then
-                                   returns TC_ERR_TIMEOUT and the handle stays usable.
-                                   Negative: TC_ERR_ARG. */
+                                   returns TC_ERR_TIMEOUT, tc_last_error names the kernel and
+                                   the handle stays usable.  Negative: TC_ERR_ARG. */
     int wait_test;              /* failure-detection test hook, 0 for normal use.  Non-zero: the
                                    MMA issuer of every tensor-core update kernel first waits
                                    on a barrier that no thread arrives at, so each launch runs
                                    into its wait bound (pair it with a short wait_limit_us) and
-                                   the call returns TC_ERR_TIMEOUT.  Nothing faults or hangs:
-                                   the kernels take their normal teardown. */
+                                   the call returns TC_ERR_TIMEOUT.  2: the cooperative kernels
+                                   too first wait for work that no CTA does.  Nothing faults or
+                                   hangs: the kernels take their normal teardown. */
     int reserved[3];
 } tc_config;
 
@@ -167,9 +172,9 @@ void tc_destroy(tc_handle h);
 /* Message of the last failing call of this handle ("" if none).  Owned by the handle. */
 const char *tc_last_error(tc_handle h);
 
-/* Change the handle's cfg.wait_limit_us (bound of each wait in the tensor-core update
- * kernels, microseconds; 0: the 4 s default) and cfg.wait_test (the failure-detection test
- * hook, 0 for normal use) for its later calls, so that a caller can shorten the waits for a
+/* Change the handle's cfg.wait_limit_us (bound of each wait inside a kernel, microseconds; 0:
+ * the 4 s default; see there) and cfg.wait_test (the failure-detection test hook, 0 for normal
+ * use) for its later calls, so that a caller can shorten the waits for a
  * watchdog, or test the timeout path, and then restore them on the same handle.  The paper
  * has no counterpart (it does not discuss failure detection).  TC_ERR_ARG for a NULL handle
  * or a negative limit. */

@@ -866,7 +866,7 @@ __device__ __forceinline__ int pt_wait(const int *p, int want, int *err, unsigne
         if (v >= want || v < 0) return v;
         if (*(volatile int *)err) return -1;
         if (z_timer() - t0 > limit_ns) {
-            atomicExch(err, 1);
+            atomicExch(err, ERR_POTRF_WAIT);
             return -1;
         }
     }
@@ -878,7 +878,8 @@ __device__ __forceinline__ void pt_add(int *p) {          // (one thread, after 
 __device__ __forceinline__ void pt_group_sync(int grp) { asm volatile("bar.sync %0, 64;" ::"r"(grp + 1) : "memory"); }
 
 __global__ void __launch_bounds__(POTRF_THREADS)
-k_potrf_tile(double *D, int ld, int nb, int col0, int *status, int *flags, int *err, unsigned long long limit_ns) {
+k_potrf_tile(double *D, int ld, int nb, int col0, int *status, int *flags, int *err, unsigned long long limit_ns,
+             int stall) {
     extern __shared__ double pts[];
     __shared__ int ready, go, filled;    // a flag per wait of a step, so that its next write comes after a barrier
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -892,7 +893,7 @@ k_potrf_tile(double *D, int ld, int nb, int col0, int *status, int *flags, int *
             return;
         }
         for (int j = 0; j < nb; ++j) {
-            if (j > 0) {
+            if (j > 0 || stall) {                          // (block 0 has no updates: the test hook's wait runs out)
                 if (tid == 0) go = pt_wait(diag + j, 16, err, limit_ns) > 0;
                 __syncthreads();
                 if (!go) return;
@@ -1024,7 +1025,7 @@ size_t potrf_tile_flags() { return 4 * PT_FLAGS * sizeof(int); }
 // A tile whose steps fit the flags, from two 64-blocks on; the grid is what the first update keeps busy.
 bool potrf_tile_ok(int b) { return b >= 128 && b <= 64 * PT_FLAGS; }
 int launch_potrf_tile(double *D, int b, int col0, int *status, int *flags, int *err, cudaStream_t s,
-                      unsigned long long limit_ns) {
+                      unsigned long long limit_ns, int stall) {
     static std::atomic<unsigned long long> attr{0};
     if (attrs_pending(attr)) {
         cudaFuncSetAttribute(k_potrf_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PT_SMEM);
@@ -1039,7 +1040,7 @@ int launch_potrf_tile(double *D, int b, int col0, int *status, int *flags, int *
     if (grid > sms) grid = sms;
     limit_ns = limit_ns ? std::max(limit_ns, GRID_WAIT_MIN_NS) : PT_LIMIT_NS;
     void *args[] = {(void *)&D, (void *)&b, (void *)&nb, (void *)&col0, (void *)&status, (void *)&flags, (void *)&err,
-                    (void *)&limit_ns};
+                    (void *)&limit_ns, (void *)&stall};
     return (int)cudaLaunchCooperativeKernel((const void *)k_potrf_tile, dim3(grid), dim3(POTRF_THREADS), args, PT_SMEM, s);
 }
 

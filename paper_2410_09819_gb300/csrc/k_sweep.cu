@@ -29,6 +29,16 @@ __device__ __forceinline__ int sweep_progress(const int *p) {
     return v;
 }
 
+// (one thread) the counter once it is above t; negative when another CTA gave up or the wait ran out
+__device__ __forceinline__ int sweep_wait(const int *progress, int t, const int *err, unsigned long long limit_ns) {
+    int v = sweep_progress(progress);
+    if (v > t) return v;
+    const uint64_t t0 = z_timer();
+    while ((v = sweep_progress(progress)) <= t)
+        if (*(const volatile int *)err || z_timer() - t0 > limit_ns) return -1;
+    return v;
+}
+
 // element (0, 0) of the 64 x 64 block (i, j) of the factor, i >= j (leading dimension b)
 __device__ __forceinline__ const double *sweep_block(const double *W, int b, int i, int j) {
     const int per = b >> 6, ti = i / per, tj = j / per;
@@ -73,7 +83,7 @@ __device__ __forceinline__ void sweep_tri(const double (*M)[65], double &u0, dou
 template <bool FWD, int NQ>
 __global__ void __launch_bounds__(256, 2)
 k_sweep(const double *__restrict__ W, int b, int nblk, double *r, int64_t ldr, int nrhs, int groups, int *progress,
-        int *err, unsigned long long limit_ns) {
+        int *err, unsigned long long limit_ns, int stall) {
     // forward M[j][c] = l_cj / l_jj (c > j): u_j = z_j l_jj travels, z = u / l_jj at the end;
     // backward M[j][c] = l_jc / l_jj (c < j), likewise
     __shared__ double M[64][65], rinv[64];
@@ -119,6 +129,7 @@ k_sweep(const double *__restrict__ W, int b, int nblk, double *r, int64_t ldr, i
             u1 = __ldcg(x + lane + 32);
         }
         int have = 0;
+        if (stall && s == 0 && tid == 0 && sweep_wait(progress, 0, err, limit_ns) < 0) stop = 1;     // test hook
         for (int t = 0; t < s; ++t) {
             const int j = FWD ? t : nblk - 1 - t;
             double l[16];
@@ -138,17 +149,8 @@ k_sweep(const double *__restrict__ W, int b, int nblk, double *r, int64_t ldr, i
             __syncthreads();                           // xs of the previous block is read
             if (t >= have) {
                 if (tid == 0) {
-                    int v = sweep_progress(progress);
-                    if (v <= t) {
-                        const uint64_t t0 = z_timer();
-                        while ((v = sweep_progress(progress)) <= t) {
-                            if (*(volatile int *)err || z_timer() - t0 > limit_ns) {
-                                stop = 1;
-                                break;
-                            }
-                        }
-                    }
-                    known = v;
+                    known = sweep_wait(progress, t, err, limit_ns);
+                    if (known < 0) stop = 1;
                 }
                 __syncthreads();
                 have = known;
@@ -230,7 +232,7 @@ k_sweep(const double *__restrict__ W, int b, int nblk, double *r, int64_t ldr, i
 // Sweeps of nrhs columns; progress: SWEEP_GROUPS counters, cleared here.  Returns a cudaError_t.
 template <bool FWD, int NQ>
 static cudaError_t sweep_launch(const double *W, int b, int nblk, double *r, int64_t ldr, int nrhs, int *progress, int *err,
-                                cudaStream_t s, unsigned long long limit_ns) {
+                                cudaStream_t s, unsigned long long limit_ns, int stall) {
     int dev = 0, sms = 0, occ = 0;
     cudaGetDevice(&dev);
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -249,7 +251,7 @@ static cudaError_t sweep_launch(const double *W, int b, int nblk, double *r, int
         double *rc = r + (int64_t)c0 * ldr;
         if ((e = cudaMemsetAsync(progress, 0, groups * sizeof(int), s)) != cudaSuccess) return e;
         void *args[] = {(void *)&W, (void *)&b, (void *)&nblk, (void *)&rc, (void *)&ldr, (void *)&cols, (void *)&groups,
-                        (void *)&progress, (void *)&err, (void *)&limit_ns};
+                        (void *)&progress, (void *)&err, (void *)&limit_ns, (void *)&stall};
         e = cudaLaunchCooperativeKernel((const void *)k_sweep<FWD, NQ>, dim3(groups * per), dim3(256), args, 0, s);
         if (e != cudaSuccess) return e;
         c0 += groups * NQ;
@@ -259,13 +261,13 @@ static cudaError_t sweep_launch(const double *W, int b, int nblk, double *r, int
 // Groups of four columns share a block of L in registers; up to three columns go as groups of one
 // (their chains run side by side, and four-column groups would multiply padding).
 int launch_sweep(const double *W, int b, int nblk, double *r, int64_t ldr, int nrhs, bool fwd, int *progress, int *err,
-                 cudaStream_t s, unsigned long long limit_ns) {
+                 cudaStream_t s, unsigned long long limit_ns, int stall) {
     limit_ns = limit_ns ? std::max(limit_ns, GRID_WAIT_MIN_NS) : SWEEP_LIMIT_NS;
     if (nrhs < 4)
-        return (int)(fwd ? sweep_launch<true, 1>(W, b, nblk, r, ldr, nrhs, progress, err, s, limit_ns)
-                         : sweep_launch<false, 1>(W, b, nblk, r, ldr, nrhs, progress, err, s, limit_ns));
-    return (int)(fwd ? sweep_launch<true, 4>(W, b, nblk, r, ldr, nrhs, progress, err, s, limit_ns)
-                     : sweep_launch<false, 4>(W, b, nblk, r, ldr, nrhs, progress, err, s, limit_ns));
+        return (int)(fwd ? sweep_launch<true, 1>(W, b, nblk, r, ldr, nrhs, progress, err, s, limit_ns, stall)
+                         : sweep_launch<false, 1>(W, b, nblk, r, ldr, nrhs, progress, err, s, limit_ns, stall));
+    return (int)(fwd ? sweep_launch<true, 4>(W, b, nblk, r, ldr, nrhs, progress, err, s, limit_ns, stall)
+                     : sweep_launch<false, 4>(W, b, nblk, r, ldr, nrhs, progress, err, s, limit_ns, stall));
 }
 
 }  // namespace tc

@@ -711,7 +711,7 @@ int execute_factor(tc_handle h, const Plan &P, const MxpPlan *M, const PlanDev &
         const bool one = spans && nmat == 1 && k < h->mats[0].nt && potrf_tile_ok(b);
         if (one) {
             CK((cudaError_t)launch_potrf_tile(W + (h->mats[0].tile0 + tidx(k, k)) * bb, b, k * b, status + 2,
-                                              static_cast<int *>(h->potrf.p), status + 1, h->s, wait_limit_ns(h)));
+                                              static_cast<int *>(h->potrf.p), status + 1, h->s, wait_limit_ns(h), wait_test_grid(h)));
             CK_LAUNCH();
         }
         for (const PotrfStep &ps : C.potrf) {
@@ -951,8 +951,7 @@ int factor_matrices(tc_handle h, tc_stats *stats, bool use_graph, const std::vec
     if ((rc = collect_results(h, &bad, &err))) return rc;
     if (err) {
         h->factored = false;
-        return set_err(h, TC_ERR_TIMEOUT, err == 2 ? "tensor-core update found no operand copy (internal)"
-                                                     : "a tensor-core update timed out waiting on its pipeline");
+        return set_err(h, TC_ERR_TIMEOUT, wait_error_text(err));
     }
     if (stats) fill_stats(h, P, Mp, stats, t0, launches0, bad);
     return TC_OK;
@@ -1247,7 +1246,7 @@ static int subst(tc_handle h, double *R, int64_t ldr, int nrhs, bool back) {
     int *w = static_cast<int *>(h->sweep.p);
     for (int f = 0; f < (back ? 2 : 1); ++f) {
         const int e = launch_sweep(static_cast<const double *>(h->W.p), h->b, (int)(ldr / 64), R, ldr, nrhs, f == 0, w + 1, w, h->s,
-                                   wait_limit_ns(h));
+                                   wait_limit_ns(h), wait_test_grid(h));
         if (e != cudaSuccess) return cuda_fail(h, (cudaError_t)e, "substitution sweep", __LINE__);
         CK_LAUNCH();
     }

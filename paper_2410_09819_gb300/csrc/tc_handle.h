@@ -209,12 +209,13 @@ inline int check_nb(tc_handle h, int64_t n, int b) {
 
 int ooc_subst(tc_handle h, double *R, int64_t ldr, int nrhs, bool back, int64_t *h2d_bytes);
 
-// Bound of the tensor-core kernels' pipeline waits for this handle (0: the kernels' default).
+// Bound of the kernels' waits for this handle (0: the kernels' default).
 inline unsigned long long wait_limit_ns(tc_handle h) {
     return h->cfg.wait_limit_us > 0 ? (unsigned long long)h->cfg.wait_limit_us * 1000ull : 0ull;
 }
 // Failure-detection test hook (tc_config.wait_test): the tensor-core kernels first wait on a
-// barrier that nothing arrives at.
+// barrier that nothing arrives at; with 2 the cooperative kernels too first wait for work that no CTA does.
 inline int wait_test(tc_handle h) { return h->cfg.wait_test != 0; }
+inline int wait_test_grid(tc_handle h) { return h->cfg.wait_test == 2; }
 
 }  // namespace tc

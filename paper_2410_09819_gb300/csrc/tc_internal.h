@@ -112,16 +112,25 @@ void launch_dgemm_reduce(const DRed *reds, int nreds, int ld, const double *part
                          const int *status, cudaStream_t s);
 void launch_potrf_block(double *D, int ld, int col0, int *status, cudaStream_t s);
 void launch_trsm_rows(double *P, const double *L, int ld, int rows, const int *status, cudaStream_t s);
+// Error word of a factorization (status[1]): what gave up.  1 to 3 come from the tensor-core kernels (a
+// pipeline wait, an operand copy that is not there, a teardown wait).
+constexpr int ERR_NO_COPY = 2, ERR_POTRF_WAIT = 4;
+inline const char *wait_error_text(int code) {
+    return code == ERR_NO_COPY      ? "tensor-core update found no operand copy (internal)"
+           : code == ERR_POTRF_WAIT ? "the POTRF of a tile timed out waiting for its other blocks"
+                                    : "a tensor-core update timed out waiting on its pipeline";
+}
 // Least bound of a wait for other CTAs of a cooperative kernel (k_potrf_tile, k_sweep).  Such a wait lasts
 // as long as their work, up to a millisecond at tile 4096, so a limit set for the microseconds of a
 // tensor-core pipeline does not end it.
 constexpr unsigned long long GRID_WAIT_MIN_NS = 100000000ull;
 // POTRF of one b x b tile in one cooperative kernel, where potrf_tile_ok(b): flags a buffer of
-// potrf_tile_flags() bytes (cleared here), *err set when a wait ran into its bound.  Returns a cudaError_t.
+// potrf_tile_flags() bytes (cleared here), *err set when a wait ran into its bound; stall != 0: the
+// failure-detection test hook (a wait for updates that nothing makes).  Returns a cudaError_t.
 size_t potrf_tile_flags();
 bool potrf_tile_ok(int b);
 int launch_potrf_tile(double *D, int b, int col0, int *status, int *flags, int *err, cudaStream_t s,
-                      unsigned long long limit_ns);
+                      unsigned long long limit_ns, int stall);
 void launch_potrf_blocks(const PEntry *e, int n, int ld, cudaStream_t s);
 void launch_trsm_rows_batched(const PEntry *e, int n, int max_rows, int ld, cudaStream_t s);
 // the POTRF step's trailing update: the lower part of the rows below the panel, C -= P P^T
@@ -172,10 +181,11 @@ void launch_bwd_update_tile(const double *L, int b, int i, int j, double *R, int
 // ------------------------------------------------------------------ launchers (k_sweep.cu)
 // Forward (L z = r) or back (L^T x = z) substitution of nrhs right-hand sides of nblk 64-row blocks
 // (column-major, leading dimension ldr), in place; progress: SWEEP_GROUPS counters.  Returns a
-// cudaError_t of the cooperative launch; a wait that runs into its bound (0: 4 s) sets *err.
+// cudaError_t of the cooperative launch; a wait that runs into its bound (0: 4 s) sets *err; stall != 0: the
+// failure-detection test hook (a wait for a block that nothing solves).
 constexpr int SWEEP_GROUPS = 64;
 int launch_sweep(const double *W, int b, int nblk, double *r, int64_t ldr, int nrhs, bool fwd, int *progress, int *err,
-                 cudaStream_t s, unsigned long long limit_ns);
+                 cudaStream_t s, unsigned long long limit_ns, int stall);
 
 // solves (column-major right-hand sides, leading dimension ldr, nrhs <= 16 per launch)
 void launch_symv_resid(const double *A, int nt, int b, int64_t n, const double *X, int64_t ldx,

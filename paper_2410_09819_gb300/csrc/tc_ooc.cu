@@ -661,7 +661,7 @@ extern "C" int tile_chol_factor_ooc(tc_handle h, int64_t n, int b, double *A_til
                 const int spp = span_begin(h, CAT_POTRF);
                 if (potrf_tile_ok(b)) {
                     CK((cudaError_t)launch_potrf_tile(D, b, k * b, status, static_cast<int *>(h->potrf.p), status + 1, h->s,
-                                                      wait_limit_ns(h)));
+                                                      wait_limit_ns(h), wait_test_grid(h)));
                     CK_LAUNCH();
                 }
                 for (int jb = 0; jb < b / 64 && !potrf_tile_ok(b); ++jb) {
@@ -776,7 +776,7 @@ extern "C" int tile_chol_factor_ooc(tc_handle h, int64_t n, int b, double *A_til
     CK(cudaStreamSynchronize(h->s_d2h));
     CK(cudaStreamSynchronize(h->s_h2d));
     C.destroy();
-    if (st2[1]) return set_err(h, TC_ERR_TIMEOUT, "a tensor-core update timed out waiting on its pipeline");
+    if (st2[1]) return set_err(h, TC_ERR_TIMEOUT, wait_error_text(st2[1]));
     const int info = st2[0];
     double logdet = 0.0;
     for (int k = 0; k < nt; ++k) logdet += ld[k];
@@ -830,7 +830,7 @@ int ooc_subst(tc_handle h, double *R, int64_t ldr, int nrhs, bool back, int64_t 
         for (int j = 0; j < nt; ++j) {
             ACQ(sd, (int)tidx(j, j), true);
             CK((cudaError_t)launch_sweep(C.ptr(sd), b, b / 64, Rc + (int64_t)j * b, ldr, nc, true, progress, err, h->s,
-                                         wait_limit_ns(h)));
+                                         wait_limit_ns(h), wait_test_grid(h)));
             CK_LAUNCH();
             C.touched(sd);
             for (int i = j + 1; i < nt; ++i) {
@@ -844,7 +844,7 @@ int ooc_subst(tc_handle h, double *R, int64_t ldr, int nrhs, bool back, int64_t 
         for (int j = nt - 1; j >= 0; --j) {
             ACQ(sd, (int)tidx(j, j), true);
             CK((cudaError_t)launch_sweep(C.ptr(sd), b, b / 64, Rc + (int64_t)j * b, ldr, nc, false, progress, err, h->s,
-                                         wait_limit_ns(h)));
+                                         wait_limit_ns(h), wait_test_grid(h)));
             CK_LAUNCH();
             C.touched(sd);
             for (int i = 0; i < j; ++i) {
