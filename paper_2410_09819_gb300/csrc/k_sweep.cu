@@ -45,23 +45,32 @@ __device__ __forceinline__ const double *sweep_block(const double *W, int b, int
     return W + tidx(ti, tj) * (int64_t)b * b + (int64_t)(j - tj * per) * 64 * b + (i - ti * per) * 64;
 }
 
-// One warp solves the 64 x 64 unit triangle M against u (forward: rows in order, M[j][c], c > j;
-// backward: from the last row, M[j][c], c < j); lane l holds elements l and l + 32.  A step is a
-// shuffle and a multiply-add.
+// a / d rounded once, from the reciprocal of d in two parts, hi = RN(1 / d) and lo = RN((1 - d hi) hi): RN(a hi + a lo)
+// with a lo = part, where nothing on the way leaves the normal range; a division elsewhere.  A division
+// takes a warp about eight FP64 instructions of 64 cycles, this two; the plain product a hi is rounded twice.
+__device__ __forceinline__ double sweep_div(double a, double d, double hi, double part) {
+    const uint64_t wa = (uint64_t)__double_as_longlong(a), wd = (uint64_t)__double_as_longlong(d);
+    if (((uint32_t)(wa >> 52) & 2047) - 543u <= 960u && ((uint32_t)(wd >> 52) & 2047) - 543u <= 960u)
+        return fma(a, hi, part);
+    return wa << 1 == 0 ? a * hi : a / d;
+}
+
+// One warp solves a 64 x 64 triangle, given as the unit triangle M (forward: rows in order, M[j][c], c > j;
+// backward: from the last row, M[j][c], c < j) and its diagonal M[j][j] with the reciprocals rhi + rlo; lane l
+// holds elements l and l + 32.  A step of the chain is a shuffle and a multiply-add on the unit
+// triangle's solution u; the elements themselves are u_j / M[j][j], of which the half solved first is
+// divided while the chain runs through the other.
 template <bool FWD>
-__device__ __forceinline__ void sweep_tri(const double (*M)[65], double &u0, double &u1) {
+__device__ __forceinline__ void sweep_tri(const double (*M)[65], const double *rhi, const double *rlo, double &u0, double &u1) {
     const int lane = threadIdx.x & 31;
+    double &f = FWD ? u0 : u1, &g = FWD ? u1 : u0;     // solved first, solved second
+    const int fi = FWD ? lane : lane + 32, gi = FWD ? lane + 32 : lane;
     if (FWD) {
 #pragma unroll 8
         for (int j = 0; j < 32; ++j) {
             const double uj = __shfl_sync(0xffffffffu, u0, j);
             if (lane > j) u0 = fma(-uj, M[j][lane], u0);
             u1 = fma(-uj, M[j][lane + 32], u1);
-        }
-#pragma unroll 8
-        for (int j = 0; j < 32; ++j) {
-            const double uj = __shfl_sync(0xffffffffu, u1, j);
-            if (lane > j) u1 = fma(-uj, M[j + 32][lane + 32], u1);
         }
     } else {
 #pragma unroll 8
@@ -70,12 +79,20 @@ __device__ __forceinline__ void sweep_tri(const double (*M)[65], double &u0, dou
             if (lane < j) u1 = fma(-uj, M[j + 32][lane + 32], u1);
             u0 = fma(-uj, M[j + 32][lane], u0);
         }
-#pragma unroll 8
-        for (int j = 31; j >= 0; --j) {
-            const double uj = __shfl_sync(0xffffffffu, u0, j);
-            if (lane < j) u0 = fma(-uj, M[j][lane], u0);
+    }
+    double part;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        if (c == 0) part = f * rlo[fi];
+        if (c == 1) f = sweep_div(f, M[fi][fi], rhi[fi], part);
+#pragma unroll
+        for (int i = 8 * c; i < 8 * c + 8; ++i) {
+            const int j = FWD ? i : 31 - i;
+            const double uj = __shfl_sync(0xffffffffu, g, j);
+            if (FWD ? lane > j : lane < j) g = fma(-uj, FWD ? M[j + 32][lane + 32] : M[j][lane], g);
         }
     }
+    g = sweep_div(g, M[gi][gi], rhi[gi], g * rlo[gi]);
 }
 
 // In place on r (columns of nblk * 64 values, leading dimension ldr); group g = blockIdx.x % groups
@@ -86,7 +103,7 @@ k_sweep(const double *__restrict__ W, int b, int nblk, double *r, int64_t ldr, i
         int *err, unsigned long long limit_ns, int stall) {
     // forward M[j][c] = l_cj / l_jj (c > j): u_j = z_j l_jj travels, z = u / l_jj at the end;
     // backward M[j][c] = l_jc / l_jj (c < j), likewise
-    __shared__ double M[64][65], rinv[64];
+    __shared__ double M[64][65], rhi[64], rlo[64];
     __shared__ __align__(16) double red[4 * NQ][64], xs[64][NQ];
     __shared__ int known, stop;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -109,12 +126,23 @@ k_sweep(const double *__restrict__ W, int b, int nblk, double *r, int64_t ldr, i
         }
         if (tid == 0) known = stop = 0;
         __syncthreads();
-        if (tid < 64) rinv[tid] = 1.0 / M[tid][tid];
-        __syncthreads();
-        for (int j = warp; j < 64; j += 8) {
-            if (FWD ? (j < 31 && lane > j) : lane < j) M[j][lane] *= rinv[j];
-            if (FWD ? lane + 32 > j : lane + 32 < j) M[j][lane + 32] *= rinv[j];
+        if (tid < 64) {
+            const double d = M[tid][tid], hi = 1.0 / d;
+            rhi[tid] = hi;
+            rlo[tid] = fma(-d, hi, 1.0) * hi;
         }
+        __syncthreads();
+        // rows p and 62 - p (backward 63 - p and p + 1) of the triangle have 64 elements together, row 31 (32) 32
+        for (int p = warp; p < 32; p += 8)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int q = lane + 32 * h, first = 63 - p;         // elements of the longer row
+                if (p == 31 && h) break;
+                const int k = q < first ? q : q - first;
+                const int row = FWD ? (q < first ? p : 62 - p) : (q < first ? 63 - p : p + 1), col = FWD ? row + 1 + k : k;
+                const double v = M[row][col];
+                M[row][col] = sweep_div(v, M[row][row], rhi[row], v * rlo[row]);
+            }
         // sum over the solved blocks t = 0 .. s - 1 (in sweep order).  Forward: thread (rr, part)
         // takes row rr and 16 columns of L; backward: warp w the columns 8w .. 8w + 7 of block column
         // i, a lane two adjacent rows of the solved block
@@ -218,9 +246,9 @@ k_sweep(const double *__restrict__ W, int b, int nblk, double *r, int64_t ldr, i
                 u0 -= rd[0][lane];
                 u1 -= rd[0][lane + 32];
             }
-            sweep_tri<FWD>(M, u0, u1);
-            __stcg(x + lane, u0 * rinv[lane]);
-            __stcg(x + lane + 32, u1 * rinv[lane + 32]);
+            sweep_tri<FWD>(M, rhi, rlo, u0, u1);
+            __stcg(x + lane, u0);
+            __stcg(x + lane + 32, u1);
         }
         // (the release below covers the stores that the barrier orders before it)
         if constexpr (NQ == 1) __syncwarp();
