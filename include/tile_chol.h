@@ -87,12 +87,16 @@ typedef struct {
                                    1: both on the tensor cores through exact digit planes
                                       of every final tile (56 bits for FP64 outputs:
                                       normwise FP64 accuracy; 40 for FP32 outputs: below
-                                      2^-40 of the tile scale; base 256 in FP16, with a
-                                      mixed map base 16 in E4M3); needs 14 b^2 extra
-                                      bytes per lower tile and a tile size multiple of 128;
+                                      2^-40 of the tile scale; base 256 in FP16, or, with
+                                      a mixed map in core, base 16 in E4M3); needs 14 b^2
+                                      extra bytes per lower tile and a tile size multiple
+                                      of 128.  The factors of one mixed map in core and out
+                                      of core agree to its accuracy level, not bit for bit;
                                    2: as 1, and the TRSMs of a one-matrix factorization
                                       (in core or out of core) run on the emulated engine as
-                                      products with L_kk^{-1} (from FP64 substitution):
+                                      products with L_kk^{-1} (in core with a mixed map
+                                      from FP64 substitution, else by doubling from its
+                                      64 x 64 diagonal blocks):
                                       low-precision tiles as L_mk = C_mk L_kk^{-T}, whose
                                       error kappa(L_kk) u is far below their accuracy
                                       level; FP64 tiles with one refinement step,
@@ -105,8 +109,8 @@ typedef struct {
                                    (the offline optimum for the copy count).  Other values:
                                    TC_ERR_ARG. */
     int fp32_updates;           /* with fp64_mode >= 1, how FP32 output tiles are updated:
-                                   0 (default): 10 digit planes on the FP8 tensor cores
-                                   (truncation below 2^-40 of the tile scale, FP64 sums);
+                                   0 (default): digit planes on the tensor cores, 10 in
+                                   base 16 or 5 in base 256 (see fp64_mode; truncation below 2^-40 of the tile scale, FP64 sums);
                                    1: 3 x TF32 tensor-core products with FP32 accumulation
                                    (as with fp64_mode 0: FP32-level arithmetic, the
                                    paper's FP32 tiles).  Other values: TC_ERR_ARG. */

@@ -7,6 +7,8 @@
 // K, and in each step row r of an operand is rounded to 2^-57 of its largest entry there.  One step
 // of one block is 3584 mma.sync.m16n8k16 on one SM.
 //
+// (Also for the inverses of a mixed map out of core; in core those take k_trinv_batched, see there.)
+//
 // Why: an SM retires 1.7 FP64 multiply-adds a clock, so a 64 x 64 x 64 step on the FP64 pipe takes
 // 69 us on its SM; mma.sync runs 1010 FP16 multiply-adds a clock (measured), so the 28 digit
 // products take 3.5 us, and the conversions about as long.

@@ -1548,10 +1548,15 @@ k_trsm_tile(const __grid_constant__ TGroup g, const double *L, int ld, int b, co
 // with the solved rows, kept in shared memory, is followed by the block's triangle: a warp per
 // column, y_j and with it the next row by shuffle, the division in integer arithmetic (the same
 // rounding, fixed_exp.h).
-// The products with Y of a mixed factorization keep 10, 6 or 4 of its digit planes, so what they
-// cut off, and with it the last bit of a stored FP32, FP16 or FP8 value here and there, follows the
-// inverse's own rounding: it stays this column-by-column substitution, every element's multiply-adds in
-// ascending order, although the doubling of k_bgemm.cu (all-FP64 maps) is several times as fast.
+// In core only, and for bits rather than accuracy: the products with Y of a mixed factorization keep 10, 6
+// or 4 of its digit planes, so what they cut off, and with it the last bit of a stored FP32, FP16 or FP8
+// value here and there, follows the inverse's own rounding, and this substitution, every element's
+// multiply-adds in ascending order, keeps the factors of a map as they have been.  The doubling of
+// k_bgemm.cu, several times as fast, serves all-FP64 maps and every map out of core, where the planes are
+// base 256 and the factor is another one within the accuracy level anyway.  Its inverse is no less exact (a
+// CPU model on Matern tiles of 256 and 512, condition of L_kk 15 to 7e6: the largest entry of Y L - I is 0.09
+// to 0.7 of this one's, that of L Y - I 0.6 to 30 times it, both far below the planes' 2^-41), and the mixed
+// factors out of core are 0.82 to 0.999 times as far from 64 bits as with this one and base 16.
 // What bounds it: the FP64 pipe (b^3 / 6 multiply-adds, 2.7 ms for a tile of 2048).  So L's blocks
 // arrive one ahead of their use, and the SM's other CTAs run while one is on its chain.  A tile of
 // 2048: 4.24 ms with four columns and 256 threads, barriers in the triangle and L read where it is

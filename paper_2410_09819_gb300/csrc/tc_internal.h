@@ -239,7 +239,7 @@ inline int tile_ctas(int ntiles) {
 }
 constexpr int Z_BN = 32;     // columns of one emulated-update work item (rows: 128)
 // Digit planes of a tile (a slot of 14 b^2 bytes): 7 base-256 planes in FP16 (k_zgemm: all-FP64
-// and out-of-core factorizations) or 14 base-16 planes in E4M3 (k_zgemm64: mixed precision)
+// and out-of-core factorizations) or 14 base-16 planes in E4M3 (k_zgemm64: mixed precision in core)
 constexpr int ZF_PLANES = 7, Z16_PLANES = 14, Z_SLOT = 14;
 constexpr int Z64_BN = 64;   // columns of a work item of the mixed-precision update kernel (k_ozaki64.cu)
 // 3D maps over the digit-plane pool (K bytes, rows of a plane, plane index) for k_zgemm64:

@@ -17,7 +17,7 @@
 // The accumulators of a tile column are taken G at a time (the same left-looking order,
 // grouped so that one TRSM launch, and with tensor-core updates one update launch per
 // precision, covers G tiles and fills the GPU).  With emulated FP64 updates every slot also
-// holds the tile's 14 digit planes, made on the device when a final tile is first used as an
+// holds the tile's digit planes, made on the device when a final tile is first used as an
 // operand after it arrived (or after it was factored).
 //
 // Mixed precision (Section IV-C with Section III-C): a final tile of precision p < FP64 is
@@ -25,7 +25,7 @@
 // compact copy at p's width (4, 2 or 1 bytes per element) into a page-locked host store;
 // every later load of it moves only the compact copy and widens it on the device -- the
 // host-link traffic of re-loads shrinks with the precision, the paper's point.  Updates run
-// in the output tile's precision: FP64 and FP32 outputs on digit planes (14 / 10 planes),
+// in the output tile's precision: FP64 and FP32 outputs on digit planes (base 256, 7 / 5 planes),
 // FP16 and FP8 outputs on scaled FP16 / E4M3 operand copies made per slot on first use.
 #include "tc_handle.h"
 
