@@ -333,7 +333,7 @@ void launch_matern(double *A, int64_t n, int b, int nt, const double *pts, doubl
     // 835 us with four CTAs a tile, 281 us; nu = 3/2, 6 tiles of 256: 50 and 40 us)
     int gx = (int)((int64_t)b * b / 4096);
     gx = gx < 1 ? 1 : gx > 64 ? 64 : gx;
-    const int fill = (8 * 152 + T - 1) / T, columns = b < 256 ? b / (256 / b) : b;
+    const int fill = (8 * NSM + T - 1) / T, columns = b < 256 ? b / (256 / b) : b;
     gx = std::max(gx, std::min(fill, columns));
     Range g{};
     g.a = a;
