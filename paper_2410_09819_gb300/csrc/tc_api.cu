@@ -194,8 +194,9 @@ Plan build_plan(tc_handle h, double *W, int *status) {
                         double *Cp = T(M, m, k);
                         const int xo = (int)(M.tile0 + tidx(m, 0)), yo = (int)(M.tile0 + tidx(k, 0));
                         int items = 0;
-                        // (all-FP64: the diagonal tile's amax slot belongs to its inverse)
-                        const int ct = m == k && !M.mixed ? -1 : (int)(M.tile0 + tidx(m, k));
+                        // (all-FP64 plans: the diagonal tile's amax slot belongs to its inverse; with any
+                        // mixed map k_zgemm64 reads the scale of every output tile there)
+                        const int ct = m == k && zw == Z_BN ? -1 : (int)(M.tile0 + tidx(m, k));
                         for_tile_items(b, m == k, [&](int bm, int bn) {
                             P.zitems.push_back({Cp, xo, yo, (uint16_t)bm, (uint16_t)bn, ct});
                             ++items;
