@@ -1,13 +1,12 @@
 // FP64 products of 64 x 64 blocks on warp-level FP16 MMAs, for products too small for the
-// tile-sized tensor-core kernel (k_ozaki.cu): the inverse of a diagonal tile of an all-FP64 map.
+// tile-sized tensor-core kernel (k_ozaki.cu): the inverse of a diagonal tile of an all-FP64 map, and
+// of any map out of core (mixed maps in core take k_trinv_batched, see there).
 //
 // The arithmetic is that of k_ozaki.cu (seven base-256 digits of an operand in FP16, 28 digit
 // products s + t <= 6 with exact FP32 sums, integer recombination), but with an exponent of its
 // own for every row of X and of Y^T instead of one for a tile: X Y^T is taken in steps of 64 along
 // K, and in each step row r of an operand is rounded to 2^-57 of its largest entry there.  One step
 // of one block is 3584 mma.sync.m16n8k16 on one SM.
-//
-// (Also for the inverses of a mixed map out of core; in core those take k_trinv_batched, see there.)
 //
 // Why: an SM retires 1.7 FP64 multiply-adds a clock, so a 64 x 64 x 64 step on the FP64 pipe takes
 // 69 us on its SM; mma.sync runs 1010 FP16 multiply-adds a clock (measured), so the 28 digit

@@ -11,7 +11,7 @@
 //
 // What bounds it: one right-hand side, the chain from block to block (counter and solution through
 // L2, one 64 x 64 product, the 64-step triangle); many, the FP64 pipe (n^2 / 2 multiply-adds a
-// sweep and column).  n = 32768, one column: 4.4 ms forward and 4.7 ms back, 9 us a block,
+// sweep and column).  n = 32768, one column: 4.4 ms forward and 4.6 ms back, 9 us a block,
 // where launches per tile with triangles of 256 rows in one CTA took 12.9 and 13.9 ms; n = 8192, 64
 // columns: 4.0 and 4.2 ms, where they took 24.3 and 26.4 ms.
 #include "tc_internal.h"
